@@ -90,6 +90,13 @@ __device__ __forceinline__ float raw_or_inf(float raw) { return raw == raw ? raw
 // 2^n for -126 <= n <= 127.
 __device__ __forceinline__ float pow2(int n) { return __int_as_float((127 + n) << 23); }
 
+// Two bytes of w_xor80 (code ^ 0x80) at the selector as 1152 + code - sub, exact.
+__device__ __forceinline__ uint32_t u8x2_minus(uint32_t w_xor80, uint32_t sel, uint32_t sub) {
+    const uint32_t h = prmt(w_xor80, 0x64646464u, sel);
+    const __half2 v = __hsub2(*reinterpret_cast<const __half2*>(&h), *reinterpret_cast<const __half2*>(&sub));
+    return *reinterpret_cast<const uint32_t*>(&v);
+}
+
 __device__ __forceinline__ uint32_t word_of(const uint4& v, int i) {
     return i == 0 ? v.x : i == 1 ? v.y : i == 2 ? v.z : v.w;
 }
@@ -112,6 +119,14 @@ __device__ __forceinline__ int tok_row(int r) { return 4 * ((r & 7) >> 1) + 2 * 
 // column g (first word) and column g + 8 (second word) at rows 4c .. 4c+3.
 __device__ __forceinline__ void ldsm_t_b8_x2(uint32_t (&d)[4], const void* row) {
     asm volatile("ldmatrix.sync.aligned.m16n16.x2.trans.shared.b8 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(d[0]), "=r"(d[1]), "=r"(d[2]), "=r"(d[3])
+                 : "r"(smem_addr(row)));
+}
+
+// ldmatrix.trans of four 8x8 blocks of 16-bit elements: lanes 8i .. 8i+7 address
+// block i's rows; lane (g, c) receives, per block, column g at rows 2c, 2c+1.
+__device__ __forceinline__ void ldsm_t_b16_x4(uint32_t (&d)[4], const void* row) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
                  : "=r"(d[0]), "=r"(d[1]), "=r"(d[2]), "=r"(d[3])
                  : "r"(smem_addr(row)));
 }

@@ -78,6 +78,59 @@ __device__ __forceinline__ void philox_n(uint32_t (&x0)[N], uint32_t (&x1)[N], u
     }
 }
 
+// Constants of a counter group g under KV head counter c1 = layer * 65536 + h: what
+// the first two rounds draw from them alone.
+struct PhiloxGroup {
+    uint32_t b, hi, lo;
+};
+__device__ __forceinline__ PhiloxGroup philox_group(uint32_t g, uint32_t c1, const PhiloxKeys& key) {
+    const uint64_t p1 = (uint64_t)kPhiloxM1 * g;
+    const uint64_t p0 = (uint64_t)kPhiloxM0 * ((uint32_t)(p1 >> 32) ^ c1 ^ key.k0[0]);
+    return {(uint32_t)p1, (uint32_t)(p0 >> 32), (uint32_t)p0};
+}
+
+// Philox4x32-10 at (slot, c1, g, tag) for four groups g and tags 0 (w[0]: a K row),
+// 1 (w[1]: the V row of the same token).  The eight calls advance round by round,
+// so their multiplies overlap, and a product that two calls share is taken once:
+// 127 wide multiplies instead of 160 (134 with the group constants redrawn).
+__device__ __forceinline__ void philox_kv(uint32_t slot, const PhiloxGroup (&gr)[4], const PhiloxKeys& key,
+                                          uint32_t (&w)[2][4][4]) {
+    const uint64_t ps = (uint64_t)kPhiloxM0 * slot;
+    const uint32_t hs = (uint32_t)(ps >> 32), ls = (uint32_t)ps;
+    uint32_t ht[2], lt[2];
+#pragma unroll
+    for (int t = 0; t < 2; ++t) {   // the second round's product on the slot's side
+        const uint64_t p = (uint64_t)kPhiloxM1 * (hs ^ (uint32_t)t ^ key.k1[0]);
+        ht[t] = (uint32_t)(p >> 32);
+        lt[t] = (uint32_t)p;
+    }
+#pragma unroll
+    for (int g = 0; g < 4; ++g) {   // third round
+        const uint64_t p1 = (uint64_t)kPhiloxM1 * (gr[g].hi ^ ls ^ key.k1[1]);
+#pragma unroll
+        for (int t = 0; t < 2; ++t) {
+            const uint64_t p0 = (uint64_t)kPhiloxM0 * (ht[t] ^ gr[g].b ^ key.k0[1]);
+            w[t][g][0] = (uint32_t)(p1 >> 32) ^ lt[t] ^ key.k0[2];
+            w[t][g][1] = (uint32_t)p1;
+            w[t][g][2] = (uint32_t)(p0 >> 32) ^ gr[g].lo ^ key.k1[2];
+            w[t][g][3] = (uint32_t)p0;
+        }
+    }
+#pragma unroll
+    for (int r = 3; r < kPhiloxRounds; ++r)
+#pragma unroll
+        for (int g = 0; g < 4; ++g)
+#pragma unroll
+            for (int t = 0; t < 2; ++t) {
+                const uint64_t p0 = (uint64_t)kPhiloxM0 * w[t][g][0];
+                const uint64_t p1 = (uint64_t)kPhiloxM1 * w[t][g][2];
+                w[t][g][0] = (uint32_t)(p1 >> 32) ^ w[t][g][1] ^ key.k0[r];
+                w[t][g][2] = (uint32_t)(p0 >> 32) ^ w[t][g][3] ^ key.k1[r];
+                w[t][g][1] = (uint32_t)p1;
+                w[t][g][3] = (uint32_t)p0;
+            }
+}
+
 // ---- byte / half packing -------------------------------------------------
 
 __device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t b, uint32_t sel) {
@@ -164,6 +217,14 @@ __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t by
 // 16-byte aligned, bytes a multiple of 16.
 __device__ __forceinline__ void bulk_prefetch_l2(const void* src, uint32_t bytes) {
     asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(src), "r"(bytes) : "memory");
+}
+
+// One lane of a converged warp.  Unlike a lane test it keeps the guarded code on
+// the uniform path, which bulk copies take their operands from.
+__device__ __forceinline__ bool elect_one() {
+    uint32_t r;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(r));
+    return r != 0;
 }
 
 __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
