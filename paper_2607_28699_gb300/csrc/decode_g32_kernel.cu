@@ -115,10 +115,17 @@ __global__ void __launch_bounds__(kGwThreads, 1) decode_g32_ws_kernel(const __gr
     if (producer) {
         int k = 0, issued = 0;   // stage ring position, continued across segments
         bool stop = false;
+        const int pt = lane >> 1, hf = lane & 1;
+        PhiloxGroup grp[4];      // a CTA's segments share their KV head
+        {
+            const int hk = kFlat ? (int)blockIdx.x % p.num_kv_heads : (int)blockIdx.y;
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                grp[j] = philox_group((uint32_t)(4 * hf + j), (uint32_t)p.layer * 65536u + (uint32_t)hk, p.keys);
+        }
         // one segment's pages (the split plan has one segment: no loop around it)
         auto produce = [&](const WsSeg& cs) {
             const int b = cs.b, h = cs.h;
-            const uint32_t c1 = (uint32_t)p.layer * 65536u + (uint32_t)h;
             const int32_t* bt_row = p.block_table + (size_t)b * p.max_pages;
             int first;
             const int n_seg = ws_seg_pages<kGwPairs>(cs, pw, first);
@@ -138,7 +145,7 @@ __global__ void __launch_bounds__(kGwThreads, 1) decode_g32_ws_kernel(const __gr
                 if (i + 1 < n_seg) phys_next = __ldg(bt_row + lp + kGwPairs);
                 const bool ok = phys >= 0 && phys < p.num_pages;
                 uint8_t* st = stages + s * kGwStageBytes;
-                if (lane == 0) {
+                if (elect_one()) {   // not a lane test: the copies' operands stay on the uniform path
                     *reinterpret_cast<int*>(st + kGwOffHdr) = ok ? phys : -1;
                     if (ok) {
                         const int z = phys * p.num_kv_heads + h;
@@ -157,26 +164,16 @@ __global__ void __launch_bounds__(kGwThreads, 1) decode_g32_ws_kernel(const __gr
                 }
                 issued = k + 1;
                 if (ok) {   // dither bytes j[token][storage position], swizzled like the code tiles
-                    // K and V of tokens g, g+8 x position chunks 2c, 2c+1 (call 2i: K, 2i+1:
-                    // V), advanced round by round
-                    const uint32_t slot0 = (uint32_t)phys * kPage;
-                    uint32_t x0[8], x1[8], x2[8], x3[8];
+                    // lane 2t + hf: token t's position chunks 4 hf .. +3, K and V together
+                    uint32_t w[2][4][4];
+                    philox_kv((uint32_t)phys * kPage + pt, grp, p.keys, w);
 #pragma unroll
-                    for (int j = 0; j < 8; ++j) {
-                        const int i = j >> 1;
-                        x0[j] = slot0 + g + 8 * (i >> 1);
-                        x1[j] = c1;
-                        x2[j] = (uint32_t)(2 * c + (i & 1));
-                        x3[j] = (uint32_t)(j & 1);
-                    }
-                    philox_n<8>(x0, x1, x2, x3, p.keys);
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        const int off = swz(g + 8 * (i >> 1), 2 * c + (i & 1));
+                    for (int j = 0; j < 4; ++j) {
+                        const int off = swz(pt, 4 * hf + j);
                         *reinterpret_cast<uint4*>(st + kGwOffKd + off) =
-                            make_uint4(x0[2 * i], x1[2 * i], x2[2 * i], x3[2 * i]);
+                            make_uint4(w[0][j][0], w[0][j][1], w[0][j][2], w[0][j][3]);
                         *reinterpret_cast<uint4*>(st + kGwOffVd + off) =
-                            make_uint4(x0[2 * i + 1], x1[2 * i + 1], x2[2 * i + 1], x3[2 * i + 1]);
+                            make_uint4(w[1][j][0], w[1][j][1], w[1][j][2], w[1][j][3]);
                     }
                 }
                 __syncwarp();
@@ -316,6 +313,7 @@ __global__ void __launch_bounds__(kGwThreads, 1) decode_g32_ws_kernel(const __gr
 #pragma unroll
         for (int i = 0; i < 8; ++i) acc[i][0] = acc[i][1] = acc[i][2] = acc[i][3] = 0.f;
         int lam_exp = INT_MIN;   // P s_g 2^lam_exp stays below 2^14 (fp16)
+        float lam = 1.f;         // 2^lam_exp
         float sv_lim = 1.17549435e-38f;   // 2^(6 - lam_exp): the scale at which lam_exp must drop
         const int tv[4] = {2 * c, 2 * c + 1, 2 * c + 8, 2 * c + 9};
 
@@ -331,7 +329,8 @@ __global__ void __launch_bounds__(kGwThreads, 1) decode_g32_ws_kernel(const __gr
             }
             const uint8_t* st = stages + s * kGwStageBytes;
             const int lp = first + kGwPairs * i;
-            if (*reinterpret_cast<const int*>(st + kGwOffHdr) >= 0) {
+            const int page = *reinterpret_cast<const int*>(st + kGwOffHdr);   // < 0: outside the pool, skipped below
+            {
                 const int nvalid = min(kPage, ctx - lp * kPage);
                 const bool ok0 = g < nvalid, ok1 = g + 8 < nvalid;
                 // group scales of tokens g, g + 8
@@ -352,14 +351,6 @@ __global__ void __launch_bounds__(kGwThreads, 1) decode_g32_ws_kernel(const __gr
                             sv[r][2 * q2] = fv.x; sv[r][2 * q2 + 1] = fv.y;
                         }
                 }
-                if (nvalid < kPage) {   // the context's last page (warp-uniform): tail slots hold any bits
-#pragma unroll
-                    for (int gi = 0; gi < 4; ++gi) {
-                        if (!ok0) { sk[0][gi] = 0.f; sv[0][gi] = 0.f; }
-                        if (!ok1) { sk[1][gi] = 0.f; sv[1][gi] = 0.f; }
-                    }
-                }
-
                 // ---------------- QK, folded per group ------------------------------------
                 // rows g, g+8 are tokens g, g+8; raw[i] = (tok g, head 2c), (g, 2c+1), (g+8, 2c), (g+8, 2c+1)
                 float raw[4] = {0.f, 0.f, 0.f, 0.f};
@@ -408,8 +399,8 @@ __global__ void __launch_bounds__(kGwThreads, 1) decode_g32_ws_kernel(const __gr
                 {
                     const uint32_t wa = *reinterpret_cast<const uint32_t*>(st + kGwOffW + (g * kBands + 2 * c) * 2);
                     const uint32_t wb = *reinterpret_cast<const uint32_t*>(st + kGwOffW + ((g + 8) * kBands + 2 * c) * 2);
-                    mma1688(cb, wa, wb, a_hi);
-                    mma1688(cb, wa, wb, a_lo);
+                    const uint32_t A[4] = {wa, wb, wa, wb};   // W . a_hi + W . a_lo: W twice along k
+                    mma16816(cb, A, a_hi, a_lo);
                 }
                 float y[4], u[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
@@ -423,47 +414,83 @@ __global__ void __launch_bounds__(kGwThreads, 1) decode_g32_ws_kernel(const __gr
                         u[i] = sqrtf(tbk * ss);
                     }
                 }
-                if (nvalid < kPage) {
-#pragma unroll
-                    for (int i = 0; i < 4; ++i)
-                        if (!((i >> 1) ? ok1 : ok0)) {
-                            y[i] = -INFINITY;
-                            cb[i] = 0.f;
-                        }
-                }
-                float mx0 = fmaxf(y[0], y[2]), mx1 = fmaxf(y[1], y[3]);
-                // the reference moves lazily (a logit above it by more than 8); the
-                // column maximum over the token rows is reduced only then
-                if (__any_sync(0xffffffffu, mx0 > m_run[0] + 8.0f || mx1 > m_run[1] + 8.0f)) {
-#pragma unroll
-                    for (int o = 4; o < 32; o <<= 1) {
-                        mx0 = fmaxf(mx0, __shfl_xor_sync(0xffffffffu, mx0, o));
-                        mx1 = fmaxf(mx1, __shfl_xor_sync(0xffffffffu, mx1, o));
-                    }
-                    const bool mv0 = mx0 > m_run[0] + 8.0f, mv1 = mx1 > m_run[1] + 8.0f;
-                    const float a0 = mv0 ? (m_run[0] == -INFINITY ? 0.f : fast_exp2(m_run[0] - mx0)) : 1.f;
-                    const float a1 = mv1 ? (m_run[1] == -INFINITY ? 0.f : fast_exp2(m_run[1] - mx1)) : 1.f;
-                    if (mv0) m_run[0] = mx0;
-                    if (mv1) m_run[1] = mx1;
-                    l_part[0] *= a0; d_part[0] *= a0; db_part[0] *= a0;
-                    l_part[1] *= a1; d_part[1] *= a1; db_part[1] *= a1;
-#pragma unroll
-                    for (int gi = 0; gi < 4; ++gi) { spv[gi][0] *= a0; spv[gi][1] *= a1; }
-#pragma unroll
-                    for (int mt = 0; mt < 8; ++mt) {
-                        acc[mt][0] *= a0; acc[mt][2] *= a0;
-                        acc[mt][1] *= a1; acc[mt][3] *= a1;
-                    }
-                }
                 float pe[4], ub[4];           // ub: the Tier-B bound in log2 units
 #pragma unroll
                 for (int i = 0; i < 4; ++i) ub[i] = kTierB ? u[i] * kLog2e : 0.f;
-                bool huge;                    // warp-uniform: a bound of kHugeLog2 or more (meter_term)
-                {
-                    float big = fmaxf(fmaxf(cb[0], cb[1]), fmaxf(cb[2], cb[3]));
-                    if constexpr (kTierB) big = fmaxf(big, fmaxf(fmaxf(ub[0], ub[1]), fmaxf(ub[2], ub[3])));
-                    huge = __any_sync(0xffffffffu, big >= kHugeLog2);
+                float big = fmaxf(fmaxf(cb[0], cb[1]), fmaxf(cb[2], cb[3]));
+                if constexpr (kTierB) big = fmaxf(big, fmaxf(fmaxf(ub[0], ub[1]), fmaxf(ub[2], ub[3])));
+                float smax = 0.f;             // P s_g 2^lam_exp < 2^14: s_g 2^lam_exp < 2^6 for every group of the page
+#pragma unroll
+                for (int gi = 0; gi < 4; ++gi) smax = fmaxf(smax, fmaxf(sv[0][gi], sv[1][gi]));
+                // One warp vote finds everything that an ordinary page does not need: a page
+                // outside the pool, the context's last page, a logit more than 8 above the
+                // reference, a V scale above the P scale's limit, a bound of kHugeLog2 or more.
+                bool skip = false, huge = false;
+                if (__any_sync(0xffffffffu, page < 0 || (lp + 1) * kPage > ctx || fmaxf(y[0], y[2]) > m_run[0] + 8.0f ||
+                                                fmaxf(y[1], y[3]) > m_run[1] + 8.0f || smax >= sv_lim ||
+                                                !(big < kHugeLog2))) {
+                    skip = page < 0;
+                    if (!skip) {
+                        if (nvalid < kPage) {   // the context's last page: slots past it hold any bits
+#pragma unroll
+                            for (int gi = 0; gi < 4; ++gi) {
+                                if (!ok0) sv[0][gi] = 0.f;
+                                if (!ok1) sv[1][gi] = 0.f;
+                            }
+#pragma unroll
+                            for (int i = 0; i < 4; ++i)
+                                if (!((i >> 1) ? ok1 : ok0)) {
+                                    y[i] = -INFINITY;
+                                    cb[i] = ub[i] = 0.f;
+                                }
+                            big = fmaxf(fmaxf(cb[0], cb[1]), fmaxf(cb[2], cb[3]));
+                            if constexpr (kTierB) big = fmaxf(big, fmaxf(fmaxf(ub[0], ub[1]), fmaxf(ub[2], ub[3])));
+                            smax = 0.f;
+#pragma unroll
+                            for (int gi = 0; gi < 4; ++gi) smax = fmaxf(smax, fmaxf(sv[0][gi], sv[1][gi]));
+                        }
+                        huge = __any_sync(0xffffffffu, big >= kHugeLog2);
+                        // the reference moves lazily (a logit above it by more than 8)
+                        float mx0 = fmaxf(y[0], y[2]), mx1 = fmaxf(y[1], y[3]);
+                        if (__any_sync(0xffffffffu, mx0 > m_run[0] + 8.0f || mx1 > m_run[1] + 8.0f)) {
+#pragma unroll
+                            for (int o = 4; o < 32; o <<= 1) {
+                                mx0 = fmaxf(mx0, __shfl_xor_sync(0xffffffffu, mx0, o));
+                                mx1 = fmaxf(mx1, __shfl_xor_sync(0xffffffffu, mx1, o));
+                            }
+                            const bool mv0 = mx0 > m_run[0] + 8.0f, mv1 = mx1 > m_run[1] + 8.0f;
+                            const float a0 = mv0 ? (m_run[0] == -INFINITY ? 0.f : fast_exp2(m_run[0] - mx0)) : 1.f;
+                            const float a1 = mv1 ? (m_run[1] == -INFINITY ? 0.f : fast_exp2(m_run[1] - mx1)) : 1.f;
+                            if (mv0) m_run[0] = mx0;
+                            if (mv1) m_run[1] = mx1;
+                            l_part[0] *= a0; d_part[0] *= a0; db_part[0] *= a0;
+                            l_part[1] *= a1; d_part[1] *= a1; db_part[1] *= a1;
+#pragma unroll
+                            for (int gi = 0; gi < 4; ++gi) { spv[gi][0] *= a0; spv[gi][1] *= a1; }
+#pragma unroll
+                            for (int mt = 0; mt < 8; ++mt) {
+                                acc[mt][0] *= a0; acc[mt][2] *= a0;
+                                acc[mt][1] *= a1; acc[mt][3] *= a1;
+                            }
+                        }
+                        if (__any_sync(0xffffffffu, smax >= sv_lim)) {   // lam_exp only decreases
+                            const float wmax = __int_as_float(__reduce_max_sync(0xffffffffu, __float_as_int(smax)));
+                            const int ex = ((__float_as_int(wmax) >> 23) & 0xFF) - 126;   // wmax < 2^ex
+                            const int want = 6 - ex;
+                            if (lam_exp != INT_MIN) {   // want < lam_exp here
+                                const float f = pow2(want - lam_exp);
+#pragma unroll
+                                for (int mt = 0; mt < 8; ++mt)
+#pragma unroll
+                                    for (int e2 = 0; e2 < 4; ++e2) acc[mt][e2] *= f;
+                            }
+                            lam_exp = want;
+                            lam = pow2(lam_exp);
+                            sv_lim = pow2(6 - lam_exp);
+                        }
+                    }
                 }
+                if (!skip) {
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
                     const int e = i & 1;
@@ -485,28 +512,6 @@ __global__ void __launch_bounds__(kGwThreads, 1) decode_g32_ws_kernel(const __gr
                         if constexpr (kTierB) db_part[e] += meter_term(t, ub[i]);
                     }
                 }
-                {   // P s_g 2^lam_exp < 2^14: s_g 2^lam_exp < 2^6 for every group of the page;
-                    // lam_exp only decreases, checked per lane against sv_lim, reduced only then
-                    float smax = 0.f;
-#pragma unroll
-                    for (int gi = 0; gi < 4; ++gi) smax = fmaxf(smax, fmaxf(sv[0][gi], sv[1][gi]));
-                    if (__any_sync(0xffffffffu, smax >= sv_lim)) {
-                        const float wmax = __int_as_float(__reduce_max_sync(0xffffffffu, __float_as_int(smax)));
-                        const int ex = ((__float_as_int(wmax) >> 23) & 0xFF) - 126;   // wmax < 2^ex
-                        const int want = 6 - ex;
-                        if (lam_exp != INT_MIN) {   // want < lam_exp here
-                            const float f = pow2(want - lam_exp);
-#pragma unroll
-                            for (int mt = 0; mt < 8; ++mt)
-#pragma unroll
-                                for (int e2 = 0; e2 < 4; ++e2) acc[mt][e2] *= f;
-                        }
-                        lam_exp = want;
-                        sv_lim = pow2(6 - lam_exp);
-                    }
-                }
-                const float lam = pow2(lam_exp == INT_MIN ? 0 : lam_exp);
-
                 // ---------------- PV: acc[dim][head], one P operand per group -----------
                 // m-tile mt covers channels 16 mt .. 16 mt + 15 (group mt / 2); row g is
                 // channel 16 mt + g, row g + 8 channel 16 mt + g + 8
@@ -539,8 +544,8 @@ __global__ void __launch_bounds__(kGwThreads, 1) decode_g32_ws_kernel(const __gr
                         for (int pr = 0; pr < 2; ++pr) {
                             const uint32_t X = prmt(word_of(vq[2 * pr], wi) ^ 0x80808080u,
                                                     word_of(vq[2 * pr + 1], wi) ^ 0x80808080u, sel_interleave(pos));
-                            A[2 * pr] = s8x2_to_h2(X, kSel01);
-                            A[2 * pr + 1] = s8x2_to_h2(X, kSel23);
+                            A[2 * pr] = u8x2_minus(X, kSel01, 0x647C647Cu);       // code + 4
+                            A[2 * pr + 1] = u8x2_minus(X, kSel23, 0x647C647Cu);
                             const uint32_t Y = prmt(word_of(dv[2 * pr], wi), word_of(dv[2 * pr + 1], wi),
                                                     sel_interleave(pos));
                             H[2 * pr] = nh8(Y, kSel01);       // -h'
@@ -551,6 +556,7 @@ __global__ void __launch_bounds__(kGwThreads, 1) decode_g32_ws_kernel(const __gr
                         mma16816(acc[mt], H, bp0, bp1);
                         mma16816(acc[mt], H, bl0, bl1);
                     }
+                }
                 }
             }
             __syncwarp();
@@ -580,7 +586,7 @@ __global__ void __launch_bounds__(kGwThreads, 1) decode_g32_ws_kernel(const __gr
                 float* row = wb + (2 * c + e) * kPartialStride;
 #pragma unroll
                 for (int mt = 0; mt < 8; ++mt) {   // channels 16 mt + g and 16 mt + g + 8
-                    const float add = kKappa * spv[mt >> 1][e];
+                    const float add = (kKappa - 4.0f) * spv[mt >> 1][e];   // the codes entered raised by 4
                     row[16 * mt + g] = fmaf(acc[mt][e], inv_lam, add);
                     row[16 * mt + g + 8] = fmaf(acc[mt][e + 2], inv_lam, add);
                 }
