@@ -20,8 +20,10 @@
 // (equal contributions; a range stretched by inf or NaN) is sorted by a bitonic
 // network instead, whose keys stay in registers: exchanges within a thread and within a
 // warp need no shared memory, only those across warps go through it.  Both give the
-// same order, so the sums that follow are the same bits.  Measured: 784 cells of 2048
-// pages 57.8 us by the network (ALU pipe 84% busy, 57,000 warp instructions a cell).
+// same order, so the sums that follow are the same bits.  Measured, network -> buckets:
+// 784 cells of 2048 pages 57.8 -> 22.2 us (57,000 -> 17,300 warp instructions a cell; what
+// is left waits for barriers and shared memory), 2800 of 512 43.5 -> 16.6, 8400 of 100
+// 120 -> 12.7, 196 of 8192 97.8 -> 30.8.  Twice or four times the buckets: 22.3 and 28.2 us.
 #include <climits>
 
 #include "wc_kernels.cuh"
@@ -30,7 +32,10 @@ namespace wc {
 
 namespace {
 
-constexpr int kSelThreads = 512;
+// The remaining sums are taken as kSumThreads threads would, thread i holding KS
+// consecutive sorted positions, whatever the CTA's size: their order of additions, and
+// with it the count that a borderline tau gives, does not depend on how a table is sorted.
+constexpr int kSumThreads = 512, kSumWarps = kSumThreads / 32;
 // Keys of a bucket that its members are compared with: beyond it the network is faster
 // (a warp's ranking takes as many steps as its fullest bucket).
 constexpr int kMaxBucket = 64;
@@ -47,20 +52,23 @@ __device__ __forceinline__ unsigned long long pick(bool take_max, unsigned long 
     return take_max ? (mine > other ? mine : other) : (mine < other ? mine : other);
 }
 
-// KPT keys per thread: thread t holds sorted positions [t KPT, t KPT + KPT).
-template <int KPT>
-__global__ void __launch_bounds__(kSelThreads) repair_select_kernel(const __grid_constant__ RepairParams p) {
-    constexpr int N = kSelThreads * KPT;   // sorted length: the block table, padded to a power of two
-    constexpr int W = 32 * KPT;            // positions held by one warp
+// A CTA of T threads sorts K keys per thread; KS: positions per thread of the sums.
+// T grows with the table (K = 4 up to 4096 pages), so that a small cell costs few warps
+// and barriers: 2800 cells of 512 pages took 24.8 us with 512 threads, 16.2 with 256.
+template <int T, int K, int KS>
+__global__ void __launch_bounds__(T) repair_select_kernel(const __grid_constant__ RepairParams p) {
+    constexpr int N = T * K;      // sorted length: the block table, padded to a power of two
+    constexpr int W = 32 * K;     // positions held by one warp
+    constexpr int kSelWarps = T / 32;
     extern __shared__ __align__(16) unsigned long long xs[];   // [N] keys; exchange buffer of the network
-    uint32_t* cnt = reinterpret_cast<uint32_t*>(xs + N);      // [N] keys per bucket, then its first position
-    __shared__ uint32_t warp_lo[kSelThreads / 32], warp_hi[kSelThreads / 32], warp_sum[kSelThreads / 32];
-    __shared__ float warp_tot[kSelThreads / 32];
-    __shared__ int warp_min[kSelThreads / 32];
+    uint32_t* cnt = reinterpret_cast<uint32_t*>(xs + N);      // [N] keys per bucket, then the buckets' ends
+    __shared__ uint32_t warp_lo[kSelWarps], warp_hi[kSelWarps], warp_sum[kSelWarps];
+    __shared__ float warp_tot[kSumWarps];
+    __shared__ int warp_min[kSelWarps];
     __shared__ float r_at_k;
     const int hq = blockIdx.x, b = blockIdx.y;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int base = tid * KPT;
+    const int base = tid * K;
     const size_t cell = (size_t)b * p.num_q_heads + hq;
 
     // the page terms are read whatever the context length (every block-table
@@ -75,11 +83,12 @@ __global__ void __launch_bounds__(kSelThreads) repair_select_kernel(const __grid
     }
     const int n = (ctx + kPage - 1) / kPage;
 
-    // ---- C_j = d_j 2^(m_j - M) / L in logical page order ---------------------------
-    unsigned long long key[KPT];
+    // ---- C_j = d_j 2^(m_j - M) / L; thread t takes pages t, t + T, ... (any order does) --
+    unsigned long long key[K];
+    auto page_of = [&](int r) { return tid + r * T; };
 #pragma unroll
-    for (int r = 0; r < KPT; ++r) {
-        const int j = base + r;
+    for (int r = 0; r < K; ++r) {
+        const int j = page_of(r);
         const float2 t = j < p.max_pages ? terms[j] : make_float2(-INFINITY, 0.f);
         key[r] = 0ull;   // padding: below every page (C = +0, index bits 0)
         if (j < n) {
@@ -90,20 +99,21 @@ __global__ void __launch_bounds__(kSelThreads) repair_select_kernel(const __grid
         }
     }
 
-    // Layout of sorted positions in shared memory: position i lives at word
-    // i ^ word_swizzle(i / KPT), a permutation of its thread's KPT words that gives the 16
-    // lanes of a half-warp 16 distinct bank pairs; an exchange partner i ^ j (j >= 32 KPT)
-    // flips only bits >= 5 of the thread index, which the permutation does not read.
-    auto word_swizzle = [](int th) { return KPT >= 16 ? (th & 15) : (((th * KPT) >> 4) & (KPT - 1)); };
+    // Sorted position i ends at word spot(i): each thread of the sums reads KS consecutive
+    // positions, permuted so that the 16 lanes of a half-warp meet 16 distinct bank pairs.
+    auto spot = [](int i) {
+        const int th = i / KS;
+        return i ^ (KS >= 16 ? (th & 15) : (((th * KS) >> 4) & (KS - 1)));
+    };
 
-    // ---- descending sort (skipped for kept cells: nothing is paged in) -------------
+    // ---- descending sort into xs (kept cells: nothing is paged in, any order does) ------
     bool network = false;
     if (!kept) {
         uint32_t lo = 0xFFFFFFFFu, hi = 0u;   // range of the pages' contribution bits
 #pragma unroll
-        for (int r = 0; r < KPT; ++r) {
-            cnt[tid + r * kSelThreads] = 0u;
-            if (base + r < n) {
+        for (int r = 0; r < K; ++r) {
+            cnt[page_of(r)] = 0u;
+            if (page_of(r) < n) {
                 const uint32_t bits = (uint32_t)(key[r] >> 32);
                 lo = min(lo, bits);
                 hi = max(hi, bits);
@@ -117,7 +127,7 @@ __global__ void __launch_bounds__(kSelThreads) repair_select_kernel(const __grid
         }
         __syncthreads();
 #pragma unroll
-        for (int w = 0; w < kSelThreads / 32; ++w) {
+        for (int w = 0; w < kSelWarps; ++w) {
             lo = min(lo, warp_lo[w]);
             hi = max(hi, warp_hi[w]);
         }
@@ -125,12 +135,12 @@ __global__ void __launch_bounds__(kSelThreads) repair_select_kernel(const __grid
         const int shift = max(0, 32 - __clz(n > 0 ? hi - lo : 0u) - (31 - __clz(N)));
         auto bucket = [&](unsigned long long k) { return (hi - (uint32_t)(k >> 32)) >> shift; };
 #pragma unroll
-        for (int r = 0; r < KPT; ++r)
-            if (base + r < n) atomicAdd(&cnt[bucket(key[r])], 1u);
+        for (int r = 0; r < K; ++r)
+            if (page_of(r) < n) atomicAdd(&cnt[bucket(key[r])], 1u);
         __syncthreads();
-        uint32_t sum = 0u, most = 0u;   // exclusive prefix sums; thread t takes buckets [t KPT, t KPT + KPT)
+        uint32_t sum = 0u, most = 0u;   // exclusive prefix sums; thread t takes buckets [t K, t K + K)
 #pragma unroll
-        for (int r = 0; r < KPT; ++r) {
+        for (int r = 0; r < K; ++r) {
             const uint32_t x = cnt[base + r];
             most = max(most, x);
             sum += x;
@@ -147,21 +157,21 @@ __global__ void __launch_bounds__(kSelThreads) repair_select_kernel(const __grid
             uint32_t first = inc - sum;
             for (int w = 0; w < warp; ++w) first += warp_sum[w];
 #pragma unroll
-            for (int r = 0; r < KPT; ++r) {
+            for (int r = 0; r < K; ++r) {
                 const uint32_t x = cnt[base + r];
                 cnt[base + r] = first;
                 first += x;
             }
             __syncthreads();
 #pragma unroll
-            for (int r = 0; r < KPT; ++r)   // grouped by bucket; cnt then holds each bucket's end
-                if (base + r < n) xs[atomicAdd(&cnt[bucket(key[r])], 1u)] = key[r];
+            for (int r = 0; r < K; ++r)   // grouped by bucket; cnt then holds each bucket's end
+                if (page_of(r) < n) xs[atomicAdd(&cnt[bucket(key[r])], 1u)] = key[r];
             __syncthreads();
-            uint32_t rank[(KPT + 1) / 2];   // two to a word (positions below 16384)
+            uint32_t rank[(K + 1) / 2];   // two to a word (positions below 16384)
 #pragma unroll
-            for (int r = 0; r < KPT; ++r) {
+            for (int r = 0; r < K; ++r) {
                 uint32_t k = 0u;   // the bucket's first position plus its larger keys
-                if (base + r < n) {
+                if (page_of(r) < n) {
                     const uint32_t bk = bucket(key[r]), last = cnt[bk];
                     k = bk > 0 ? cnt[bk - 1] : 0u;
                     for (uint32_t i = k, e = last; i < e; ++i) k += xs[i] > key[r] ? 1u : 0u;
@@ -171,39 +181,38 @@ __global__ void __launch_bounds__(kSelThreads) repair_select_kernel(const __grid
             }
             __syncthreads();
 #pragma unroll
-            for (int r = 0; r < KPT; ++r)
-                if (base + r < n) {
-                    const int k = (int)((rank[r / 2] >> (16 * (r & 1))) & 0xFFFFu);
-                    xs[k ^ word_swizzle(k / KPT)] = key[r];
-                }
-            __syncthreads();
-#pragma unroll
-            for (int r = 0; r < KPT; ++r) key[r] = base + r < n ? xs[(base + r) ^ word_swizzle(tid)] : 0ull;   // padding last
+            for (int r = 0; r < K; ++r) {   // padding keeps its own places behind the pages
+                const int k = page_of(r) < n ? (int)((rank[r / 2] >> (16 * (r & 1))) & 0xFFFFu) : page_of(r);
+                xs[spot(k)] = key[r];
+            }
         }
     }
     if (network) {
-        const int sw = word_swizzle(tid);
+        // exchange layout: position i at word i ^ sw(i / K), as in spot(); an exchange
+        // partner i ^ j (j >= 32 K) flips only bits >= 5 of the thread index, which sw
+        // does not read
+        const int sw = K >= 16 ? (tid & 15) : (((tid * K) >> 4) & (K - 1));
         for (int k = 2; k <= N; k <<= 1) {
             for (int j = k >> 1; j >= W; j >>= 1) {   // partner in another warp
                 const bool tm = bitonic_takes_max(base, j, k);
 #pragma unroll
-                for (int r = 0; r < KPT; ++r) xs[(base + r) ^ sw] = key[r];
+                for (int r = 0; r < K; ++r) xs[(base + r) ^ sw] = key[r];
                 __syncthreads();
 #pragma unroll
-                for (int r = 0; r < KPT; ++r) key[r] = pick(tm, key[r], xs[((base + r) ^ j) ^ sw]);
+                for (int r = 0; r < K; ++r) key[r] = pick(tm, key[r], xs[((base + r) ^ j) ^ sw]);
                 __syncthreads();
             }
-            for (int j = min(k >> 1, W >> 1); j >= KPT; j >>= 1) {   // partner in this warp
+            for (int j = min(k >> 1, W >> 1); j >= K; j >>= 1) {   // partner in this warp
                 const bool tm = bitonic_takes_max(base, j, k);
-                const int lm = j / KPT;
+                const int lm = j / K;
 #pragma unroll
-                for (int r = 0; r < KPT; ++r) key[r] = pick(tm, key[r], __shfl_xor_sync(0xffffffffu, key[r], lm));
+                for (int r = 0; r < K; ++r) key[r] = pick(tm, key[r], __shfl_xor_sync(0xffffffffu, key[r], lm));
             }
 #pragma unroll
-            for (int j = KPT >> 1; j > 0; j >>= 1) {   // partner in this thread
+            for (int j = K >> 1; j > 0; j >>= 1) {   // partner in this thread
                 if (j <= (k >> 1)) {
 #pragma unroll
-                    for (int r = 0; r < KPT; ++r)
+                    for (int r = 0; r < K; ++r)
                         if ((r & j) == 0) {
                             const bool desc = ((base + r) & k) == 0;
                             const unsigned long long a = key[r], c = key[r | j];
@@ -216,90 +225,117 @@ __global__ void __launch_bounds__(kSelThreads) repair_select_kernel(const __grid
             }
         }
     }
+    if (kept || network) {   // kept: page order, the order its sums have always had
+#pragma unroll
+        for (int r = 0; r < K; ++r) xs[spot(kept ? page_of(r) : base + r)] = key[r];
+    }
+    __syncthreads();
 
     // ---- remaining sums R_i = sum of the ranked contributions from i on ---------
-    // each thread sums its KPT positions from the tail; the later threads'
-    // sums enter as an offset
-    float tot = 0.f;
+    // each thread of the sums adds its KS positions from the tail; the later
+    // threads' sums enter as an offset
+    constexpr int kRounds = (kSumWarps + kSelWarps - 1) / kSelWarps;   // warps of the sums per warp
+    auto value = [&](int i) { return i < N ? key_value(xs[spot(i)]) : 0.f; };
+    float offset[kRounds];
 #pragma unroll
-    for (int r = KPT - 1; r >= 0; --r) tot += key_value(key[r]);
-    float suf = tot;   // inclusive suffix over the warp's lanes
+    for (int q = 0; q < kRounds; ++q) {
+        const int w = warp + q * kSelWarps, at = (32 * w + lane) * KS;
+        offset[q] = 0.f;
+        if (w < kSumWarps) {   // warp-uniform
+            float tot = 0.f;
+            if (32 * w * KS < n) {
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const float v = __shfl_down_sync(0xffffffffu, suf, o);
-        if (lane + o < 32) suf += v;
-    }
-    if (lane == 0) warp_tot[warp] = suf;
-    float offset = __shfl_down_sync(0xffffffffu, suf, 1);   // later lanes of this warp
-    if (lane == 31) offset = 0.f;
-    __syncthreads();
-    for (int w = kSelThreads / 32 - 1; w > warp; --w) offset += warp_tot[w];
-
-    int cand = INT_MAX;
-    if (!kept) {
-        float s = offset;
+                for (int r = KS - 1; r >= 0; --r) tot += value(at + r);
+            }
+            float suf = tot;   // inclusive suffix over the warp's lanes
 #pragma unroll
-        for (int r = KPT - 1; r >= 0; --r) {
-            s += key_value(key[r]);
-            if (0.5f * s * (s + 2.0f) <= p.tau) cand = base + r;   // NaN -> false
+            for (int o = 1; o < 32; o <<= 1) {
+                const float v = __shfl_down_sync(0xffffffffu, suf, o);
+                if (lane + o < 32) suf += v;
+            }
+            if (lane == 0) warp_tot[w] = suf;
+            offset[q] = __shfl_down_sync(0xffffffffu, suf, 1);   // later lanes of this warp
+            if (lane == 31) offset[q] = 0.f;
         }
     }
+    __syncthreads();
+    int cand = INT_MAX;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) cand = min(cand, __shfl_xor_sync(0xffffffffu, cand, o));
+    for (int q = 0; q < kRounds; ++q) {
+        const int w = warp + q * kSelWarps, at = (32 * w + lane) * KS;
+        if (w < kSumWarps) {
+            for (int x = kSumWarps - 1; x > w; --x) offset[q] += warp_tot[x];
+            if (!kept && at < N) {
+                float s = offset[q];
+#pragma unroll
+                for (int r = KS - 1; r >= 0; --r) {
+                    s += value(at + r);
+                    if (0.5f * s * (s + 2.0f) <= p.tau) cand = min(cand, at + r);   // NaN -> false
+                }
+            }
+        }
+    }
+    cand = __reduce_min_sync(0xffffffffu, cand);
     if (lane == 0) warp_min[warp] = cand;
     __syncthreads();
     int kmin = INT_MAX;
-    for (int w = 0; w < kSelThreads / 32; ++w) kmin = min(kmin, warp_min[w]);
+    for (int w = 0; w < kSelWarps; ++w) kmin = min(kmin, warp_min[w]);
     const int kstar = kept ? 0 : min(kmin, n);   // every page when no prefix is enough
     if (kstar >= n) {
         if (tid == 0) r_at_k = 0.f;
-    } else if (kstar >= base && kstar < base + KPT) {
-        float s = offset;
+    } else {
 #pragma unroll
-        for (int r = KPT - 1; r >= 0; --r)
-            if (base + r >= kstar) s += key_value(key[r]);
-        r_at_k = s;
+        for (int q = 0; q < kRounds; ++q) {
+            const int at = (32 * (warp + q * kSelWarps) + lane) * KS;
+            if (kstar >= at && kstar < at + KS) {
+                float s = offset[q];
+#pragma unroll
+                for (int r = KS - 1; r >= 0; --r)
+                    if (at + r >= kstar) s += value(at + r);
+                r_at_k = s;
+            }
+        }
     }
+    for (int i = tid; i < kstar; i += T)
+        p.repair_pages[cell * p.max_pages + i] = (int32_t)(0xFFFFFFFFu - (uint32_t)(xs[spot(i)] & 0xFFFFFFFFull));
     __syncthreads();
-#pragma unroll
-    for (int r = 0; r < KPT; ++r)
-        if (base + r < kstar)
-            p.repair_pages[cell * p.max_pages + base + r] = (int32_t)(0xFFFFFFFFu - (uint32_t)(key[r] & 0xFFFFFFFFull));
     if (tid == 0) {
         p.n_repair[cell] = kstar;
         p.d_after[cell] = r_at_k;
     }
 }
 
-template <int KPT>
-cudaError_t launch_kpt(const RepairParams& p, cudaStream_t stream) {
+template <int T, int K, int KS>
+cudaError_t launch_select(const RepairParams& p, cudaStream_t stream) {
     static bool configured = false;
-    constexpr size_t smem = (size_t)kSelThreads * KPT * (sizeof(unsigned long long) + sizeof(uint32_t));
+    constexpr size_t smem = (size_t)T * K * (sizeof(unsigned long long) + sizeof(uint32_t));
     if (!configured) {
-        cudaError_t e = cudaFuncSetAttribute(repair_select_kernel<KPT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        cudaError_t e = cudaFuncSetAttribute(repair_select_kernel<T, K, KS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              (int)smem);
         if (e != cudaSuccess) return e;
-        e = cudaFuncSetAttribute(repair_select_kernel<KPT>, cudaFuncAttributePreferredSharedMemoryCarveout,
+        e = cudaFuncSetAttribute(repair_select_kernel<T, K, KS>, cudaFuncAttributePreferredSharedMemoryCarveout,
                                  (int)cudaSharedmemCarveoutMaxShared);
         if (e != cudaSuccess) return e;
         configured = true;
     }
-    repair_select_kernel<KPT><<<dim3(p.num_q_heads, p.batch), kSelThreads, smem, stream>>>(p);
+    repair_select_kernel<T, K, KS><<<dim3(p.num_q_heads, p.batch), T, smem, stream>>>(p);
     return cudaGetLastError();
 }
 
 }  // namespace
 
 cudaError_t launch_repair_select(const RepairParams& p, cudaStream_t stream) {
-    static_assert(kRepairMaxPages == 32 * kSelThreads, "the largest instance holds 32 keys per thread");
+    static_assert(kRepairMaxPages == 16 * 1024, "the largest instance holds 16 keys per thread");
     if (p.batch == 0) return cudaSuccess;
-    const int need = (p.max_pages + kSelThreads - 1) / kSelThreads;   // keys per thread, rounded up to 2^m
-    if (need <= 1) return launch_kpt<1>(p, stream);
-    if (need <= 2) return launch_kpt<2>(p, stream);
-    if (need <= 4) return launch_kpt<4>(p, stream);
-    if (need <= 8) return launch_kpt<8>(p, stream);
-    if (need <= 16) return launch_kpt<16>(p, stream);
-    return launch_kpt<32>(p, stream);
+    // the least power of two that holds the table; KS = keys per thread of 512
+    if (p.max_pages <= 128) return launch_select<32, 4, 1>(p, stream);
+    if (p.max_pages <= 256) return launch_select<64, 4, 1>(p, stream);
+    if (p.max_pages <= 512) return launch_select<128, 4, 1>(p, stream);
+    if (p.max_pages <= 1024) return launch_select<256, 4, 2>(p, stream);
+    if (p.max_pages <= 2048) return launch_select<512, 4, 4>(p, stream);
+    if (p.max_pages <= 4096) return launch_select<1024, 4, 8>(p, stream);
+    if (p.max_pages <= 8192) return launch_select<1024, 8, 16>(p, stream);
+    return launch_select<1024, 16, 32>(p, stream);
 }
 
 }  // namespace wc
