@@ -78,6 +78,37 @@ __device__ __forceinline__ void philox_n(uint32_t (&x0)[N], uint32_t (&x1)[N], u
     }
 }
 
+// Philox4x32-10 at (c0, c1, c2, 0) and (c0, c1, c2, 1) (a K row and the V row of the same
+// token), round by round: 36 wide multiplies instead of 40.
+__device__ __forceinline__ void philox_rows(uint32_t c0, uint32_t c1, uint32_t c2, const PhiloxKeys& key, uint4& w0,
+                                            uint4& w1) {
+    const uint64_t a0 = (uint64_t)kPhiloxM0 * c0, a1 = (uint64_t)kPhiloxM1 * c2;
+    const uint64_t b0 = (uint64_t)kPhiloxM0 * ((uint32_t)(a1 >> 32) ^ c1 ^ key.k0[0]);   // round 2: shared
+    const uint64_t p1 = (uint64_t)kPhiloxM1 * ((uint32_t)(b0 >> 32) ^ (uint32_t)a0 ^ key.k1[1]);   // round 3: shared
+    uint32_t x[2][4];
+#pragma unroll
+    for (int t = 0; t < 2; ++t) {
+        const uint64_t b1 = (uint64_t)kPhiloxM1 * ((uint32_t)(a0 >> 32) ^ (uint32_t)t ^ key.k1[0]);
+        const uint64_t p0 = (uint64_t)kPhiloxM0 * ((uint32_t)(b1 >> 32) ^ (uint32_t)a1 ^ key.k0[1]);
+        x[t][0] = (uint32_t)(p1 >> 32) ^ (uint32_t)b1 ^ key.k0[2];
+        x[t][1] = (uint32_t)p1;
+        x[t][2] = (uint32_t)(p0 >> 32) ^ (uint32_t)b0 ^ key.k1[2];
+        x[t][3] = (uint32_t)p0;
+    }
+#pragma unroll
+    for (int r = 3; r < kPhiloxRounds; ++r)
+#pragma unroll
+        for (int t = 0; t < 2; ++t) {
+            const uint64_t q0 = (uint64_t)kPhiloxM0 * x[t][0], q1 = (uint64_t)kPhiloxM1 * x[t][2];
+            x[t][0] = (uint32_t)(q1 >> 32) ^ x[t][1] ^ key.k0[r];
+            x[t][2] = (uint32_t)(q0 >> 32) ^ x[t][3] ^ key.k1[r];
+            x[t][1] = (uint32_t)q1;
+            x[t][3] = (uint32_t)q0;
+        }
+    w0 = make_uint4(x[0][0], x[0][1], x[0][2], x[0][3]);
+    w1 = make_uint4(x[1][0], x[1][1], x[1][2], x[1][3]);
+}
+
 // Constants of a counter group g under KV head counter c1 = layer * 65536 + h: what
 // the first two rounds draw from them alone.
 struct PhiloxGroup {

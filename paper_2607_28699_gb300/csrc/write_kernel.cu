@@ -2,11 +2,10 @@
 // K band-norm residual witness (§6.2.1 write kernel; §4.1 Eq. witness;
 // §4.2 subtractive dither).
 //
-// A CTA of 4 warps handles eight (token, KV head) units: warps 0 and 2 the K
-// rows, warps 1 and 3 the V rows, 8 lanes per row.  Each lane owns 16
-// consecutive channels, so it loads 32 B of fp16, stores 16 B of codes, and
-// (for the dither schemes) consumes exactly one Philox4x32-10 call per 16
-// channels.
+// A warp handles four (token, KV head) units, their K rows and then their V rows
+// (grouped scheme: K or V rows), 8 lanes per row.  Each lane owns 16 consecutive
+// channels, so it loads 32 B of fp16, stores 16 B of codes, and (for the dither
+// schemes) consumes exactly one Philox4x32-10 call per row and 16 channels.
 //
 // Grouped scheme (§6.2.3 "Storage side" and §6.2.5 "Fixed-channel outlier bypass"):
 // one fp16 scale per 32-channel group (a lane pair), the group amax leaving
@@ -29,15 +28,16 @@ namespace wc {
 
 namespace {
 
-// Tasks of 4 tokens per warp whose loads are all issued before any is used:
-// more bytes in flight per SM (the kernel is otherwise bound by load latency).
-constexpr int kWriteTasks = 2;
-// The grouped scheme's row routine is much larger: one task per warp keeps the
-// kernel's code small enough for the instruction cache.
-__host__ __device__ constexpr int write_tasks(int scheme) {
-    return scheme == WC_SCHEME_DITHER_INT8_G32 ? 1 : kWriteTasks;
+// A warp's tasks (rows of 4 units), whose loads are all issued before any is used: more
+// bytes in flight per SM.  The K and the V rows of the same units: the row routine is
+// then specialised for each, and their Philox calls share the products that do not see
+// the tag.  One task per warp (K rows in warps 0 and 2, V rows in 1 and 3) for the grouped
+// scheme, whose much larger row routine must stay small enough for the instruction
+// cache, and for a write of a few tokens, where one row's latency is what counts.
+__host__ __device__ constexpr int write_tasks(int scheme, bool per_head) {
+    return scheme == WC_SCHEME_DITHER_INT8_G32 || !per_head ? 1 : 2;
 }
-__host__ __device__ constexpr int write_units_per_cta(int scheme) { return 2 * 4 * write_tasks(scheme); }
+__host__ __device__ constexpr int write_units_per_cta(int scheme, bool per_head) { return 2 * 4 * write_tasks(scheme, per_head); }
 constexpr int kPerHeadMinTokens = 16;                     // per-head grid from this many tokens on
 
 // Two ways of cutting the units (token, KV head) into 4-unit tasks:
@@ -90,63 +90,49 @@ __global__ void __launch_bounds__(128, write_min_blocks(kScheme)) write_kernel(c
         __syncthreads();
         tab = &btab;
     }
-    // Warps 0, 2 take the K rows and warps 1, 3 the V rows of the same units,
-    // so the residual and witness work stays in whole warps; lanes 8i .. 8i+7
-    // own unit i of a 4-unit task.
-    const int row = warp & 1;                                                  // 0 = K, 1 = V
+    // lanes 8i .. 8i+7 own unit i of the warp's four
     const int sub = lane & 7;                                                  // 16-channel chunk
-    constexpr int kTasks = write_tasks(kScheme);
-    const int first = (blockIdx.x * 2 + (warp >> 1)) * (4 * kTasks) + (lane >> 3);
+    constexpr int kTasks = write_tasks(kScheme, kPerHead);
+    const int idx = kTasks == 1 ? (blockIdx.x * 2 + (warp >> 1)) * 4 + (lane >> 3)
+                                : (blockIdx.x * 4 + warp) * 4 + (lane >> 3);   // a token (kPerHead) or a unit
     const int n_first = kPerHead ? p.n_tok : p.n_tok * p.num_kv_heads;
-    bool live[kTasks];
-    int slot[kTasks], hs[kTasks];
+    const bool live = idx < n_first;
+    if (!__any_sync(0xffffffffu, live)) return;   // warp-uniform: a warp past the end
+    int tok = 0, h = 0;
+    if (live) {
+        if (kPerHead) {
+            tok = idx;
+            h = blockIdx.y;
+        } else {
+            tok = idx / p.num_kv_heads;
+            h = idx - tok * p.num_kv_heads;
+        }
+    }
+    const int slot = live ? __ldg(p.slot_mapping + tok) : -1;
     uint4 raw[kTasks][2];
 #pragma unroll
     for (int t = 0; t < kTasks; ++t) {
-        const int idx = first + 4 * t;   // a token (kPerHead) or a unit
-        live[t] = idx < n_first;
-        int tok = 0, h = 0;
-        if (live[t]) {
-            if (kPerHead) {
-                tok = idx;
-                h = blockIdx.y;
-            } else {
-                tok = idx / p.num_kv_heads;
-                h = idx - tok * p.num_kv_heads;
-            }
-        }
-        hs[t] = h;
-        slot[t] = live[t] ? __ldg(p.slot_mapping + tok) : -1;
+        const int row = kTasks == 1 ? (warp & 1) : t;                          // 0 = K, 1 = V
         raw[t][0] = raw[t][1] = make_uint4(0, 0, 0, 0);
-        if (live[t]) {
+        if (live) {
             const uint4* src = reinterpret_cast<const uint4*>(
                 (row == 0 ? p.k : p.v) + ((size_t)tok * p.num_kv_heads + h) * kHeadDim + sub * 16);
             raw[t][0] = __ldg(src);
             raw[t][1] = __ldg(src + 1);
         }
     }
-    // 8-bit dither: the tasks' Philox calls (one per lane each) advanced together
-    uint4 w[kTasks];
-    constexpr bool kPre = kScheme != WC_SCHEME_FP8_E4M3 && kBits == 8;
-    if constexpr (kPre) {
-        uint32_t x0[kTasks], x1[kTasks], x2[kTasks], x3[kTasks];
-#pragma unroll
-        for (int t = 0; t < kTasks; ++t) {
-            x0[t] = (uint32_t)max(slot[t], 0);
-            x1[t] = (uint32_t)p.layer * 65536u + (uint32_t)hs[t];
-            x2[t] = (uint32_t)sub;
-            x3[t] = (uint32_t)row;
-        }
-        philox_n<kTasks>(x0, x1, x2, x3, p.keys);
-#pragma unroll
-        for (int t = 0; t < kTasks; ++t) w[t] = make_uint4(x0[t], x1[t], x2[t], x3[t]);
+    if constexpr (kTasks == 1) {
+        write_row<kScheme, kBits>(p, raw[0], slot, live, h, warp & 1, sub,
+                                  kGrouped ? xrows + (warp * 4 + (lane >> 3)) * kXRowStride : nullptr, tab);
+    } else {
+        // 8-bit dither: the two rows' Philox calls advanced together
+        uint4 w[2];
+        constexpr bool kPre = kScheme != WC_SCHEME_FP8_E4M3 && kBits == 8;
+        if constexpr (kPre)
+            philox_rows((uint32_t)max(slot, 0), (uint32_t)p.layer * 65536u + (uint32_t)h, (uint32_t)sub, p.keys, w[0], w[1]);
+        write_row<kScheme, kBits>(p, raw[0], slot, live, h, 0, sub, nullptr, nullptr, kPre ? &w[0] : nullptr);
+        write_row<kScheme, kBits>(p, raw[kTasks - 1], slot, live, h, 1, sub, nullptr, nullptr, kPre ? &w[1] : nullptr);
     }
-#pragma unroll
-    for (int t = 0; t < kTasks; ++t)
-        if (__any_sync(0xffffffffu, live[t]))   // warp-uniform: a task past the end is skipped whole
-            write_row<kScheme, kBits>(p, raw[t], slot[t], live[t], hs[t], row, sub,
-                                      kGrouped ? xrows + (warp * 4 + (lane >> 3)) * kXRowStride : xrows, tab,
-                                      kPre ? &w[t] : nullptr);
 }
 
 // Bypass-pair calibration: a cluster of 8 CTAs of 32 warps per KV head.  Warp
@@ -249,7 +235,7 @@ cudaError_t launch_write(const WriteParams& p, int scheme, int bits, cudaStream_
         configured = true;
     }
     const bool per_head = p.n_tok >= kPerHeadMinTokens;
-    const int upc = write_units_per_cta(scheme);
+    const int upc = write_units_per_cta(scheme, per_head);
     const dim3 grid = per_head ? dim3((p.n_tok + upc - 1) / upc, p.num_kv_heads)
                                : dim3((p.n_tok * p.num_kv_heads + upc - 1) / upc);
     auto go = [&](auto kernel) { return launch_pdl(kernel, grid, dim3(128), 0, stream, p); };

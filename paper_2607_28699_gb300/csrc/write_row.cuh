@@ -161,8 +161,17 @@ __device__ __forceinline__ void write_row(const WriteParams& p, uint4 (&raw)[2],
     }
     if constexpr (kDither) {
         float amax = 0.0f;
+        if constexpr (!kGrouped) {   // on the fp16 pairs (exact; NaN is passed over, as fmaxf does)
+            const __half2* hv = reinterpret_cast<const __half2*>(raw);
+            __half2 mx = __hmax2(__habs2(hv[0]), __habs2(hv[1]));
 #pragma unroll
-        for (int i = 0; i < 16; ++i) amax = fmaxf(amax, ((bmask >> i) & 1u) ? 0.0f : fabsf(x[i]));
+            for (int i = 2; i < 8; ++i) mx = __hmax2(mx, __habs2(hv[i]));
+            const float2 f = __half22float2(mx);
+            amax = fmaxf(amax, fmaxf(f.x, f.y));
+        } else {
+#pragma unroll
+            for (int i = 0; i < 16; ++i) amax = fmaxf(amax, ((bmask >> i) & 1u) ? 0.0f : fabsf(x[i]));
+        }
         // the row (8 lanes) or the 32-channel group (a lane pair)
 #pragma unroll
         for (int o = 1; o < (kGrouped ? 2 : 8); o <<= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, o));
@@ -420,10 +429,9 @@ __device__ __forceinline__ void write_row(const WriteParams& p, uint4 (&raw)[2],
         __half* wdst = p.k_witness + rowidx * kBands;
         if (p.rope_layout == WC_ROPE_HALF) {
             // dims 16*sub..+7 and +8..+15 are the first (sub < 4) or second
-            // (sub >= 4) halves of bands 2*(sub&3) and 2*(sub&3)+1.
-            if (sub < 4)
-                *reinterpret_cast<__half2*>(wdst + 2 * sub) =
-                    __halves2half2(norm_up_fp16(lo + lo_p), norm_up_fp16(hi + hi_p));
+            // (sub >= 4) halves of bands 2*(sub&3) and 2*(sub&3)+1; each lane of a
+            // pair takes one of the two bands.
+            wdst[2 * (sub & 3) + (sub >> 2)] = norm_up_fp16(sub < 4 ? lo + lo_p : hi + hi_p);
         } else {
             wdst[sub] = norm_up_fp16(lo + hi);
         }
