@@ -2,8 +2,8 @@
 // K band-norm residual witness (§6.2.1 write kernel; §4.1 Eq. witness;
 // §4.2 subtractive dither).
 //
-// A warp handles four (token, KV head) units, their K rows and then their V rows
-// (grouped scheme: K or V rows), 8 lanes per row.  Each lane owns 16 consecutive
+// A warp handles four (token, KV head) units, their K rows and then their V rows, 8
+// lanes per row.  Each lane owns 16 consecutive
 // channels, so it loads 32 B of fp16, stores 16 B of codes, and (for the dither
 // schemes) consumes exactly one Philox4x32-10 call per row and 16 channels.
 //
@@ -31,32 +31,33 @@ namespace {
 // A warp's tasks (rows of 4 units), whose loads are all issued before any is used: more
 // bytes in flight per SM.  The K and the V rows of the same units: the row routine is
 // then specialised for each, and their Philox calls share the products that do not see
-// the tag.  One task per warp (K rows in warps 0 and 2, V rows in 1 and 3) for the grouped
-// scheme, whose much larger row routine must stay small enough for the instruction
-// cache, and for a write of a few tokens, where one row's latency is what counts.
-__host__ __device__ constexpr int write_tasks(int scheme, bool per_head) {
-    return scheme == WC_SCHEME_DITHER_INT8_G32 || !per_head ? 1 : 2;
-}
-__host__ __device__ constexpr int write_units_per_cta(int scheme, bool per_head) { return 2 * 4 * write_tasks(scheme, per_head); }
+// the tag.  A write of a few tokens takes one task per warp (K rows in warps 0 and 2, V
+// rows in 1 and 3): there one row's latency is what counts.  Measured at 32768 x 4 tokens
+// and heads against K and V rows in separate warps (us): 8-bit dither 31.1 -> 26.4, 10-bit
+// 39.7 -> 36.3, fp8 18.1 -> 15.7, grouped 50.1 -> 44.9 (55.4 before its packed pass).
+constexpr int write_units_per_cta(int tasks) { return 2 * 4 * tasks; }
+// The grouped row routine is the longest: until its two-task CTAs fill the SMs (6 x 152 of
+// 16 units), one task per warp is done sooner (tokens x 8 heads, us one / two tasks: 100
+// 3.8 / 4.5, 600 5.2 / 6.7, 1200 6.8 / 8.5).
+constexpr int kGroupedTwoTaskUnits = 16384;
 constexpr int kPerHeadMinTokens = 16;                     // per-head grid from this many tokens on
 
 // Two ways of cutting the units (token, KV head) into 4-unit tasks:
 //  kPerHead: grid (token groups, Hkv), a task = 4 consecutive tokens of one
 //            head, so a warp's code, scale and witness stores are contiguous
-//            runs of consecutive slots (prefill);
+//            runs of consecutive slots (prefill), K and V;
 //  else:     one index over units u = token * Hkv + h, a task = 4 consecutive
 //            units, so a one-token write of up to 8 KV heads is a single CTA
 //            (decode steps, where every SM the next decode needs counts).
-// Resident CTAs per SM the register budget is sized for: seven (72 registers)
-// for the dithered schemes, ten for fp8.  The 8-bit dither's packed fast pass
-// then spills 4 bytes; the extra warps per SM still take 4-5% off a prefill
-// write against six CTAs at 80 registers, and eight (64 registers, 48 bytes of
-// spill) are slower again.
-__host__ __device__ constexpr int write_min_blocks(int scheme) {
-    return scheme == WC_SCHEME_FP8_E4M3 ? 10 : 7;
+// Resident CTAs per SM the register budget is sized for, the best of 5 .. 9 in each case
+// (us at 32768 x 4): 8-bit dither seven at 72 registers 26.9 (six 28.5, eight 28.2, with
+// 36 bytes of spill), 10-bit six 35.7 (seven 36.3), grouped six 44.9 (seven 44.1 with 84
+// bytes of spill, which costs the 2047 x 8 write 10%), fp8 eight 15.3 (ten 15.7).
+__host__ __device__ constexpr int write_min_blocks(int scheme, int bits) {
+    return scheme == WC_SCHEME_FP8_E4M3 ? 8 : scheme == WC_SCHEME_DITHER_INT8_G32 || bits == 10 ? 6 : 7;
 }
-template <int kScheme, int kBits, bool kPerHead>
-__global__ void __launch_bounds__(128, write_min_blocks(kScheme)) write_kernel(const __grid_constant__ WriteParams p) {
+template <int kScheme, int kBits, bool kPerHead, int kTasks>
+__global__ void __launch_bounds__(128, write_min_blocks(kScheme, kBits)) write_kernel(const __grid_constant__ WriteParams p) {
     constexpr bool kGrouped = kScheme == WC_SCHEME_DITHER_INT8_G32;
     __shared__ __align__(16) uint8_t xrows[kGrouped ? 4 * 4 * kXRowStride : 16];   // [warp][unit][row]
     __shared__ BypassTable btab;
@@ -92,7 +93,6 @@ __global__ void __launch_bounds__(128, write_min_blocks(kScheme)) write_kernel(c
     }
     // lanes 8i .. 8i+7 own unit i of the warp's four
     const int sub = lane & 7;                                                  // 16-channel chunk
-    constexpr int kTasks = write_tasks(kScheme, kPerHead);
     const int idx = kTasks == 1 ? (blockIdx.x * 2 + (warp >> 1)) * 4 + (lane >> 3)
                                 : (blockIdx.x * 4 + warp) * 4 + (lane >> 3);   // a token (kPerHead) or a unit
     const int n_first = kPerHead ? p.n_tok : p.n_tok * p.num_kv_heads;
@@ -121,17 +121,17 @@ __global__ void __launch_bounds__(128, write_min_blocks(kScheme)) write_kernel(c
             raw[t][1] = __ldg(src + 1);
         }
     }
+    uint8_t* xrow = kGrouped ? xrows + (warp * 4 + (lane >> 3)) * kXRowStride : nullptr;
     if constexpr (kTasks == 1) {
-        write_row<kScheme, kBits>(p, raw[0], slot, live, h, warp & 1, sub,
-                                  kGrouped ? xrows + (warp * 4 + (lane >> 3)) * kXRowStride : nullptr, tab);
+        write_row<kScheme, kBits>(p, raw[0], slot, live, h, warp & 1, sub, xrow, tab);
     } else {
         // 8-bit dither: the two rows' Philox calls advanced together
         uint4 w[2];
         constexpr bool kPre = kScheme != WC_SCHEME_FP8_E4M3 && kBits == 8;
         if constexpr (kPre)
             philox_rows((uint32_t)max(slot, 0), (uint32_t)p.layer * 65536u + (uint32_t)h, (uint32_t)sub, p.keys, w[0], w[1]);
-        write_row<kScheme, kBits>(p, raw[0], slot, live, h, 0, sub, nullptr, nullptr, kPre ? &w[0] : nullptr);
-        write_row<kScheme, kBits>(p, raw[kTasks - 1], slot, live, h, 1, sub, nullptr, nullptr, kPre ? &w[1] : nullptr);
+        write_row<kScheme, kBits>(p, raw[0], slot, live, h, 0, sub, xrow, tab, kPre ? &w[0] : nullptr);
+        write_row<kScheme, kBits>(p, raw[kTasks - 1], slot, live, h, 1, sub, xrow, tab, kPre ? &w[1] : nullptr);
     }
 }
 
@@ -219,14 +219,15 @@ cudaError_t launch_write(const WriteParams& p, int scheme, int bits, cudaStream_
     if (p.n_tok == 0) return cudaSuccess;
     static bool configured = false;   // same carveout as the decode kernels: no L1/shared reconfiguration
     if (!configured) {
-        const void* fns[8] = {(const void*)write_kernel<WC_SCHEME_FP8_E4M3, 8, false>,
-                              (const void*)write_kernel<WC_SCHEME_DITHER_INT8, 8, false>,
-                              (const void*)write_kernel<WC_SCHEME_DITHER_INT8, 10, false>,
-                              (const void*)write_kernel<WC_SCHEME_DITHER_INT8_G32, 8, false>,
-                              (const void*)write_kernel<WC_SCHEME_FP8_E4M3, 8, true>,
-                              (const void*)write_kernel<WC_SCHEME_DITHER_INT8, 8, true>,
-                              (const void*)write_kernel<WC_SCHEME_DITHER_INT8, 10, true>,
-                              (const void*)write_kernel<WC_SCHEME_DITHER_INT8_G32, 8, true>};
+        const void* fns[9] = {(const void*)write_kernel<WC_SCHEME_FP8_E4M3, 8, false, 1>,
+                              (const void*)write_kernel<WC_SCHEME_DITHER_INT8, 8, false, 1>,
+                              (const void*)write_kernel<WC_SCHEME_DITHER_INT8, 10, false, 1>,
+                              (const void*)write_kernel<WC_SCHEME_DITHER_INT8_G32, 8, false, 1>,
+                              (const void*)write_kernel<WC_SCHEME_FP8_E4M3, 8, true, 2>,
+                              (const void*)write_kernel<WC_SCHEME_DITHER_INT8, 8, true, 2>,
+                              (const void*)write_kernel<WC_SCHEME_DITHER_INT8, 10, true, 2>,
+                              (const void*)write_kernel<WC_SCHEME_DITHER_INT8_G32, 8, true, 1>,
+                              (const void*)write_kernel<WC_SCHEME_DITHER_INT8_G32, 8, true, 2>};
         for (const void* f : fns) {
             cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout,
                                                  (int)cudaSharedmemCarveoutMaxShared);
@@ -235,20 +236,23 @@ cudaError_t launch_write(const WriteParams& p, int scheme, int bits, cudaStream_
         configured = true;
     }
     const bool per_head = p.n_tok >= kPerHeadMinTokens;
-    const int upc = write_units_per_cta(scheme, per_head);
+    const bool grouped = scheme == WC_SCHEME_DITHER_INT8_G32;
+    const bool two = per_head && (!grouped || (int64_t)p.n_tok * p.num_kv_heads >= kGroupedTwoTaskUnits);
+    const int upc = write_units_per_cta(two ? 2 : 1);
     const dim3 grid = per_head ? dim3((p.n_tok + upc - 1) / upc, p.num_kv_heads)
                                : dim3((p.n_tok * p.num_kv_heads + upc - 1) / upc);
     auto go = [&](auto kernel) { return launch_pdl(kernel, grid, dim3(128), 0, stream, p); };
     if (scheme == WC_SCHEME_FP8_E4M3)
-        return per_head ? go(write_kernel<WC_SCHEME_FP8_E4M3, 8, true>) : go(write_kernel<WC_SCHEME_FP8_E4M3, 8, false>);
-    if (scheme == WC_SCHEME_DITHER_INT8_G32)
-        return per_head ? go(write_kernel<WC_SCHEME_DITHER_INT8_G32, 8, true>)
-                        : go(write_kernel<WC_SCHEME_DITHER_INT8_G32, 8, false>);
+        return two ? go(write_kernel<WC_SCHEME_FP8_E4M3, 8, true, 2>) : go(write_kernel<WC_SCHEME_FP8_E4M3, 8, false, 1>);
+    if (grouped)
+        return two        ? go(write_kernel<WC_SCHEME_DITHER_INT8_G32, 8, true, 2>)
+               : per_head ? go(write_kernel<WC_SCHEME_DITHER_INT8_G32, 8, true, 1>)
+                          : go(write_kernel<WC_SCHEME_DITHER_INT8_G32, 8, false, 1>);
     if (bits == 8)
-        return per_head ? go(write_kernel<WC_SCHEME_DITHER_INT8, 8, true>)
-                        : go(write_kernel<WC_SCHEME_DITHER_INT8, 8, false>);
-    return per_head ? go(write_kernel<WC_SCHEME_DITHER_INT8, 10, true>)
-                    : go(write_kernel<WC_SCHEME_DITHER_INT8, 10, false>);
+        return two ? go(write_kernel<WC_SCHEME_DITHER_INT8, 8, true, 2>)
+                   : go(write_kernel<WC_SCHEME_DITHER_INT8, 8, false, 1>);
+    return two ? go(write_kernel<WC_SCHEME_DITHER_INT8, 10, true, 2>)
+               : go(write_kernel<WC_SCHEME_DITHER_INT8, 10, false, 1>);
 }
 
 }  // namespace wc

@@ -87,12 +87,13 @@ constexpr float kBias = 12582912.0f;
 // Dither word byte (i % 4) placed as the float 1 + j/2^15 (bits 0x3F80jj00).
 __device__ __forceinline__ uint32_t xi_sel(int i) { return 0x7604u | ((uint32_t)(i & 3) << 4); }
 
-// x[i] for a lane-uniform runtime index i in [0, 16), without local memory.
-__device__ __forceinline__ float pick16(const float (&x)[16], int i) {
-    float v = x[0];
+// The i-th of a lane's 16 fp16 values for a runtime index, without local memory.
+__device__ __forceinline__ float pick16(const uint4 (&raw)[2], int i) {
+    const __half* x = reinterpret_cast<const __half*>(raw);
+    __half v = x[0];
 #pragma unroll
     for (int k = 1; k < 16; ++k) v = (i == k) ? x[k] : v;
-    return v;
+    return __half2float(v);
 }
 
 // Bypass set of one KV head in shared memory (grouped scheme, per-head grid):
@@ -161,7 +162,7 @@ __device__ __forceinline__ void write_row(const WriteParams& p, uint4 (&raw)[2],
     }
     if constexpr (kDither) {
         float amax = 0.0f;
-        if constexpr (!kGrouped) {   // on the fp16 pairs (exact; NaN is passed over, as fmaxf does)
+        if (!kGrouped || row != 0) {   // on the fp16 pairs (exact; NaN is passed over, as fmaxf does)
             const __half2* hv = reinterpret_cast<const __half2*>(raw);
             __half2 mx = __hmax2(__habs2(hv[0]), __habs2(hv[1]));
 #pragma unroll
@@ -233,6 +234,13 @@ __device__ __forceinline__ void write_row(const WriteParams& p, uint4 (&raw)[2],
                 return __uint_as_float(0x3F800000u | mant) - kOff;
             }
         };
+        // grouped K rows: a bypassed channel enters as 0, so its code is round(xi) = 0; its
+        // exact value is taken from raw below
+        if (kGrouped && row == 0) {
+#pragma unroll
+            for (int i = 0; i < 16; ++i)
+                if ((bmask >> i) & 1u) x[i] = 0.0f;
+        }
         uint32_t tb[16];   // bits of t = k + kBias: the low byte is the code
         // Fast pass (no clamp): round the fp32 estimate, track its largest
         // distance from the rounded value and, in K warps, accumulate the
@@ -241,13 +249,13 @@ __device__ __forceinline__ void write_row(const WriteParams& p, uint4 (&raw)[2],
         // exactly below (about one warp in fifty, and rows with tiny amax).
         auto fast_pass = [&](auto with_residual) -> float {
             float dev = 0.0f;
-            if constexpr (!kGrouped && kBits == 8) {
+            if constexpr (kBits == 8) {
                 // Channel pairs on the packed fp32x2 path: each lane of __ffma2_rn /
                 // __fadd2_rn rounds like the scalar fmaf / add, so est, t, k and r are
                 // the scalar pass's bits.  est - k and k - xi are taken as fma(-1, k,
                 // est) and fma(-1, xi, k) (exact products, the same roundings), and
                 // r = fma(-s, k - xi, x) is the residual with its sign flipped.  The
-                // squared residuals sum in two chains per half; the 2^-18 margin of
+                // squared residuals sum in two chains per half (grouped: one); the 2^-18 margin of
                 // norm_up_fp16 covers the fp32 error of any summation order.
                 const float2 inv2 = make_float2(inv_s, inv_s), ns2 = make_float2(-s, -s);
                 const float2 m1 = make_float2(-1.0f, -1.0f), c128 = make_float2(128.0f, 128.0f);
@@ -268,9 +276,17 @@ __device__ __forceinline__ void write_row(const WriteParams& p, uint4 (&raw)[2],
                     tb[i] = __float_as_uint(t.x);
                     tb[i + 1] = __float_as_uint(t.y);
                     if constexpr (decltype(with_residual)::value) {
-                        const float2 r = __ffma2_rn(ns2, __ffma2_rn(xi, m1, k), x2);
-                        if (i < 8) alo = __ffma2_rn(r, r, alo);
-                        else ahi = __ffma2_rn(r, r, ahi);
+                        float2 r = __ffma2_rn(ns2, __ffma2_rn(xi, m1, k), x2);
+                        if constexpr (kGrouped) {
+                            if ((bmask >> i) & 1u) r.x = 0.0f;   // exact channels: no residual
+                            if ((bmask >> (i + 1)) & 1u) r.y = 0.0f;
+                            float& sum = i < 8 ? alo.x : ahi.x;   // one chain, as the exact pass sums
+                            sum = fmaf(r.y, r.y, fmaf(r.x, r.x, sum));
+                        } else if (i < 8) {
+                            alo = __ffma2_rn(r, r, alo);
+                        } else {
+                            ahi = __ffma2_rn(r, r, ahi);
+                        }
                     }
                 }
                 if constexpr (decltype(with_residual)::value) {
@@ -371,7 +387,8 @@ __device__ __forceinline__ void write_row(const WriteParams& p, uint4 (&raw)[2],
                 __half* bdst = p.k_bypass + rowidx * (2 * p.num_bypass);
 #pragma unroll
                 for (int i = 0; i < 16; ++i)
-                    if ((bmask >> i) & 1u) bdst[tab->entry[16 * sub + i]] = __float2half_rn(x[i]);
+                    if ((bmask >> i) & 1u) bdst[tab->entry[16 * sub + i]] =
+                            __float2half_rn(__half2float(reinterpret_cast<const __half*>(raw)[i]));   // NaN: the canonical one
                 if (sub == 0)   // an ignored pair stores zeros
                     for (uint32_t bad = tab->bad; bad != 0u; bad &= bad - 1u) {
                         const int t = __ffs(bad) - 1;
@@ -391,13 +408,13 @@ __device__ __forceinline__ void write_row(const WriteParams& p, uint4 (&raw)[2],
                     const int b = p.rope_layout == WC_ROPE_HALF ? j + kHeadDim / 2 : 2 * j + 1;
                     if ((a >> 4) == sub) {
                         const bool again = (seen >> (a & 15)) & 1u;
-                        bdst[2 * t] = __float2half_rn(again ? 0.0f : pick16(x, a & 15));
+                        bdst[2 * t] = __float2half_rn(again ? 0.0f : pick16(raw, a & 15));
                         if (again && live_unit && p.dev_status) atomicOr(p.dev_status, WC_DEV_BAD_PAIR);
                         seen |= 1u << (a & 15);
                     }
                     if ((b >> 4) == sub) {
                         const bool again = (seen >> (b & 15)) & 1u;
-                        bdst[2 * t + 1] = __float2half_rn(again ? 0.0f : pick16(x, b & 15));
+                        bdst[2 * t + 1] = __float2half_rn(again ? 0.0f : pick16(raw, b & 15));
                         seen |= 1u << (b & 15);
                     }
                 }
