@@ -135,51 +135,99 @@ __global__ void __launch_bounds__(128, write_min_blocks(kScheme, kBits)) write_k
     }
 }
 
-// Bypass-pair calibration: a cluster of 8 CTAs of 32 warps per KV head.  Warp
-// w of cluster rank r sums rows 32 r + w + 256 i: one 256-byte row per warp load,
-// lane l squaring channels 4l .. 4l + 3.  Each CTA adds its warps' sums in a
-// fixed order; rank 0 adds the 8 CTAs' sums (distributed shared memory, rank
-// order), adds channels into pairs, and selects a pair iff fewer than m pairs
-// rank above it (larger energy, or equal energy and a lower index).
-constexpr int kSelPairThreads = 1024;
-constexpr int kSelPairCluster = 8;
+// Bypass-pair calibration: a cluster of 8 CTAs of 32 warps per KV head, or of 16 CTAs of 8
+// warps.  Either way 256 chains: chain 32 r + c sums rows 32 r + c + 256 i, and the 32
+// chains of an r are added in the order of c.  The narrow cluster gives a chain to a warp:
+// one 256-byte row per warp load, lane l squaring channels 4l .. 4l + 3.  In the wide one
+// rank r takes the channels 0 .. 63 and rank r + 8 the channels 64 .. 127, and a warp load
+// covers the half rows of four chains, 16 bytes a lane.  Rank 0 adds the sums of the eight
+// r (distributed shared memory, r's order), adds channels into pairs, and selects a pair
+// iff fewer than m pairs rank above it (larger energy, or equal energy and a lower index).
+// Both clusters add the same numbers in the same order.  Bytes in flight bound the narrow
+// one (4 loads a warp: 32 KB an SM, 1.8 TB/s over 32 SMs); the wide one keeps 64 KB an SM in
+// a ring of asynchronous copies on twice the SMs, as deeper batches of loads into registers
+// were split up again by the compiler (8.7).  16384 rows x 4 heads: 9.6 -> 6.7 us.
+constexpr int kSelPairRing = 16;   // wide: copies in flight per lane
 
-__global__ void __cluster_dims__(kSelPairCluster, 1, 1) __launch_bounds__(kSelPairThreads)
+__device__ __forceinline__ void copy16_or_zero(uint4* dst, const __half* src, bool valid) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n\tcp.async.commit_group;"
+                 :: "r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src), "r"(valid ? 16 : 0)
+                 : "memory");
+}
+
+template <bool kWide>
+__global__ void __launch_bounds__(kWide ? 256 : 1024)
     select_pairs_kernel(const __half* __restrict__ k, int n_tok, int num_kv_heads, int rope_layout, int m,
                         int32_t* __restrict__ pairs) {
-    __shared__ float part[kSelPairThreads / 32][kHeadDim];
+    constexpr int kWidth = kWide ? kHeadDim / 2 : kHeadDim;   // channels of a CTA
+    __shared__ float part[32][kHeadDim];
     __shared__ float energy[kHeadDim / 2];
     __shared__ int chosen[kHeadDim / 2];
     cg::cluster_group cluster = cg::this_cluster();
     const int rank = (int)cluster.block_rank();
     const int h = blockIdx.y, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    constexpr int kWarpsPerHead = kSelPairCluster * kSelPairThreads / 32;
-    float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
+    if constexpr (kWide) {
+        const size_t stride = (size_t)num_kv_heads * kHeadDim;
+        const int chain = 4 * warp + (lane >> 3), c0 = 8 * (lane & 7);
+        const __half* src = k + (size_t)h * kHeadDim + (rank >> 3) * kWidth + c0;
+        float a[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+        auto add = [&](uint4 w) {
+            const uint32_t ww[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&ww[i]));
+                a[2 * i] = fmaf(f.x, f.x, a[2 * i]);
+                a[2 * i + 1] = fmaf(f.y, f.y, a[2 * i + 1]);
+            }
+        };
+        extern __shared__ uint4 ring[];   // [kSelPairRing][256]: every thread its own 16 bytes
+        uint4* slot = ring + tid;
+        const int steps = (n_tok + 255) / 256;
+        int t = (rank & 7) * 32 + chain;   // row of the next copy
+        for (int i = 0; i < kSelPairRing; ++i, t += 256) copy16_or_zero(slot + 256 * i, t < n_tok ? src + t * stride : k, t < n_tok);
+#pragma unroll 1
+        for (int s = 0; s < steps; s += kSelPairRing) {
+#pragma unroll
+            for (int i = 0; i < kSelPairRing; ++i, t += 256) {
+                asm volatile("cp.async.wait_group %0;" ::"n"(kSelPairRing - 1) : "memory");
+                const uint4 w = slot[256 * i];
+                __syncwarp();   // the read stands before the copy into the same slot
+                add(w);         // + 0 past the end
+                copy16_or_zero(slot + 256 * i, t < n_tok ? src + t * stride : k, t < n_tok);
+            }
+        }
+        asm volatile("cp.async.wait_all;" ::: "memory");
+#pragma unroll
+        for (int i = 0; i < 8; ++i) part[chain][c0 + i] = a[i];
+    } else {
+        float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
 #pragma unroll 4
-    for (int t = rank * (kSelPairThreads / 32) + warp; t < n_tok; t += kWarpsPerHead) {
-        const uint2 w = __ldg(reinterpret_cast<const uint2*>(k + ((size_t)t * num_kv_heads + h) * kHeadDim) + lane);
-        const float2 f01 = __half22float2(*reinterpret_cast<const __half2*>(&w.x));
-        const float2 f23 = __half22float2(*reinterpret_cast<const __half2*>(&w.y));
-        a0 = fmaf(f01.x, f01.x, a0);
-        a1 = fmaf(f01.y, f01.y, a1);
-        a2 = fmaf(f23.x, f23.x, a2);
-        a3 = fmaf(f23.y, f23.y, a3);
+        for (int t = rank * 32 + warp; t < n_tok; t += 256) {
+            const uint2 w = __ldg(reinterpret_cast<const uint2*>(k + ((size_t)t * num_kv_heads + h) * kHeadDim) + lane);
+            const float2 f01 = __half22float2(*reinterpret_cast<const __half2*>(&w.x));
+            const float2 f23 = __half22float2(*reinterpret_cast<const __half2*>(&w.y));
+            a0 = fmaf(f01.x, f01.x, a0);
+            a1 = fmaf(f01.y, f01.y, a1);
+            a2 = fmaf(f23.x, f23.x, a2);
+            a3 = fmaf(f23.y, f23.y, a3);
+        }
+        part[warp][4 * lane] = a0;
+        part[warp][4 * lane + 1] = a1;
+        part[warp][4 * lane + 2] = a2;
+        part[warp][4 * lane + 3] = a3;
     }
-    part[warp][4 * lane] = a0;
-    part[warp][4 * lane + 1] = a1;
-    part[warp][4 * lane + 2] = a2;
-    part[warp][4 * lane + 3] = a3;
     __syncthreads();
-    if (tid < kHeadDim) {   // this CTA's channel sums in a fixed order (each thread its own column)
+    if (tid < kWidth) {   // this CTA's channel sums in a fixed order (each thread its own column)
         float e = 0.f;
-        for (int w = 0; w < kSelPairThreads / 32; ++w) e += part[w][tid];
+        for (int w = 0; w < 32; ++w) e += part[w][tid];
         part[0][tid] = e;
     }
     cluster.sync();   // every CTA's sums are in its row 0
     if (rank == 0) {
         if (tid < kHeadDim) {
             float e = 0.f;
-            for (int r = 0; r < kSelPairCluster; ++r) e += cluster.map_shared_rank(&part[0][0], r)[tid];
+            for (int r = 0; r < 8; ++r)
+                e += cluster.map_shared_rank(&part[0][0], tid / kWidth * 8 + r)[tid % kWidth];
             part[1][tid] = e;
         }
         __syncthreads();
@@ -208,11 +256,40 @@ __global__ void __cluster_dims__(kSelPairCluster, 1, 1) __launch_bounds__(kSelPa
 
 }  // namespace
 
+template <bool kWide>
+static cudaError_t launch_pairs(const __half* k, int n_tok, int num_kv_heads, int rope_layout, int m, int32_t* pairs,
+                                cudaStream_t stream) {
+    static bool configured = false;   // per process; the attribute is per function
+    if (!configured && kWide) {       // above the portable cluster size
+        cudaError_t e = cudaFuncSetAttribute(select_pairs_kernel<kWide>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+        if (e != cudaSuccess) return e;
+        e = cudaFuncSetAttribute(select_pairs_kernel<kWide>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSelPairRing * 256 * 16);
+        if (e != cudaSuccess) return e;
+        configured = true;
+    }
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(kWide ? 16 : 8, num_kv_heads);
+    cfg.blockDim = dim3(kWide ? 256 : 1024);
+    cfg.dynamicSmemBytes = kWide ? kSelPairRing * 256 * 16 : 0;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = cfg.gridDim.x;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, select_pairs_kernel<kWide>, k, n_tok, num_kv_heads, rope_layout, m, pairs);
+}
+
 cudaError_t launch_select_pairs(const __half* k, int n_tok, int num_kv_heads, int rope_layout, int m, int32_t* pairs,
                                 cudaStream_t stream) {
-    select_pairs_kernel<<<dim3(kSelPairCluster, num_kv_heads), kSelPairThreads, 0, stream>>>(k, n_tok, num_kv_heads,
-                                                                                            rope_layout, m, pairs);
-    return cudaGetLastError();
+    // The wide cluster's copies are 16 bytes; a k that is only 8-byte aligned stays on the
+    // narrow one.  4 heads, us narrow / wide: 1024 rows 3.8 / 4.6, 2048 4.5 / 4.6, 4096
+    // 4.8 / 4.4, 8192 6.3 / 5.3, 32768 15.2 / 9.3.
+    constexpr int kWideRows = 4096;
+    const bool wide = n_tok >= kWideRows && ((uintptr_t)k & 15) == 0;
+    return wide ? launch_pairs<true>(k, n_tok, num_kv_heads, rope_layout, m, pairs, stream)
+                : launch_pairs<false>(k, n_tok, num_kv_heads, rope_layout, m, pairs, stream);
 }
 
 cudaError_t launch_write(const WriteParams& p, int scheme, int bits, cudaStream_t stream) {
