@@ -1447,34 +1447,39 @@ DecodePlan plan_decode(int batch, int num_kv_heads, int max_pages, int num_sms, 
 constexpr int kMergeSpreadSmem = 118784;
 
 // Merge where a unit has only a few partials: the flattened plan (its
-// sequence's cuts) and a split plan of at most kWarpMergeSplits splits (a
-// batch of sequences on the per-token kernel).  One warp per (sequence, query
-// head, 32 output dims) folds all of them in order with the same
-// running-maximum update as merge_kernel, so a CTA of 8 warps serves 8 outputs
-// and needs no block barrier, and a batch's merge is one wave of short warps
-// rather than several waves of CTAs with a block reduction each.
+// sequence's cuts) and a split plan of at most kWarpMergeSplits splits.  kW warps per
+// (sequence, query head, 32 output dims) take every kW-th partial with the same
+// running-maximum update as merge_kernel and add up through shared memory, so a CTA of 8
+// warps serves 8 / kW outputs.  A long sequence in a small batch has up to 38 cuts at 4 KV
+// heads, which one warp folds in five rounds of loads: 2 sequences of 984 pages 24.3 us a
+// decode with kW = 1, 21.2 with 8, sequences of 1975 and 1 pages 28.3 and 21.9.  A batch of
+// many sequences has few cuts each, and more CTAs only start later: 16 sequences of 387
+// pages 44.7 us with kW = 1 or 2, 45.8 with 4; 38 of 52 pages 19.4 with 1, 21.3 with 2.
+// So kW is the largest of 8, 4, 2, 1 that keeps the launch within 32 warps per SM.
 constexpr int kWarpMergeSplits = 8;
 
-template <int kX>
+template <int kX, int kW>
 __global__ void __launch_bounds__(32 * kMergeWarps) merge_warp_kernel(const __grid_constant__ DecodeParams p) {
     grid_dep_launch();   // the next kernel waits for this grid before reading its outputs
     grid_dep_wait();
-    const int lane = threadIdx.x & 31;
-    const long long item = (long long)blockIdx.x * kMergeWarps + (threadIdx.x >> 5);
-    if (item >= (long long)p.batch * p.num_q_heads * (kHeadDim / 32)) return;   // warp-uniform
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, sub = warp % kW;
+    const long long item = (long long)blockIdx.x * (kMergeWarps / kW) + warp / kW;
+    const bool live = item < (long long)p.batch * p.num_q_heads * (kHeadDim / 32);   // warp-uniform
+    if (kW == 1 && !live) return;
     const int chunk = (int)(item % (kHeadDim / 32));
     const int hq = (int)((item / (kHeadDim / 32)) % p.num_q_heads);
     const int b = (int)(item / ((kHeadDim / 32) * p.num_q_heads));
     const int h = hq / p.group, hh = hq % p.group;
     constexpr bool tier_b = (kX & kXTierB) != 0, vside = (kX & kXValue) != 0, repair = (kX & kXRepair) != 0;
 
-    const int nb = (max(0, min(__ldg(p.ctx_lens + b), p.max_pages * kPage)) + kPage - 1) / kPage;
-    int count;
-    const float* base;
-    if (p.pages_per_split > 0) {
+    int count = 0;
+    const float* base = nullptr;
+    if (!live) {
+    } else if (p.pages_per_split > 0) {
         // Split plan: the unit's splits are consecutive; those past the
         // sequence's last page hold no pages (their maximum is -inf) and are
         // not read.
+        const int nb = (clamped_ctx(p, b) + kPage - 1) / kPage;
         count = min(p.splits, (nb + p.pages_per_split - 1) / p.pages_per_split);
         base = p.partials + ((size_t)b * p.num_kv_heads + h) * p.splits * (kMaxGroup * kPartialStride) +
                hh * kPartialStride;
@@ -1485,35 +1490,34 @@ __global__ void __launch_bounds__(32 * kMergeWarps) merge_warp_kernel(const __gr
         // [j R, (j + 1) R), R = ceil(total / shares), in each head, so the unit's
         // segments are those of shares P_b / R .. (P_b + n_b - 1) / R, stored at
         // partials h (shares + batch) + j + b, consecutive.
-        int before = 0, total = 0;
+        uint32_t before = 0, total = 0, nb = 0;   // below 2^31 (the plan's condition)
         for (int i = lane; i < p.batch; i += 32) {
-            const int np = (max(0, min(__ldg(p.ctx_lens + i), p.max_pages * kPage)) + kPage - 1) / kPage;
+            const uint32_t np = (uint32_t)(clamped_ctx(p, i) + kPage - 1) / kPage;
             total += np;
             if (i < b) before += np;
+            if (i == b) nb = np;
         }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            before += __shfl_xor_sync(0xffffffffu, before, o);
-            total += __shfl_xor_sync(0xffffffffu, total, o);
-        }
-        const int shares = max(1, p.splits / p.num_kv_heads);
-        const long long R = max(1LL, ((long long)total + shares - 1) / shares);
-        const long long j0 = before / R;
-        count = nb > 0 ? (int)(((long long)before + nb - 1) / R - j0 + 1) : 0;
+        total = __reduce_add_sync(0xffffffffu, total);
+        before = __reduce_add_sync(0xffffffffu, before);
+        nb = __reduce_add_sync(0xffffffffu, nb);
+        const uint32_t shares = max(1, p.splits / p.num_kv_heads);
+        const uint32_t R = max(1u, (total + shares - 1) / shares);
+        const uint32_t j0 = before / R;
+        count = nb > 0 ? (int)((before + nb - 1) / R - j0 + 1) : 0;
         base = p.partials + ((size_t)h * (shares + p.batch) + (size_t)(j0 + b)) * (kMaxGroup * kPartialStride) +
                hh * kPartialStride;
     }
 
     constexpr int kRows = 8;   // rows loaded per round before any is combined
     float M = -INFINITY, acc = 0.f, L = 0.f, Dn = 0.f, Db = 0.f, Vt = 0.f, Vm = 0.f;
-    for (int s0 = 0; s0 < count; s0 += kRows) {
+    for (int s0 = sub; s0 < count; s0 += kRows * kW) {
         float ms[kRows], v[kRows], ls[kRows], ds[kRows], dbs[kRows], vts[kRows];
 #pragma unroll
         for (int i = 0; i < kRows; ++i) {
             ms[i] = -INFINITY;
             v[i] = ls[i] = ds[i] = dbs[i] = vts[i] = 0.f;
-            if (s0 + i < count) {
-                const float* ps = base + (size_t)(s0 + i) * (kMaxGroup * kPartialStride);
+            if (s0 + i * kW < count) {
+                const float* ps = base + (size_t)(s0 + i * kW) * (kMaxGroup * kPartialStride);
                 ms[i] = __ldcg(ps + kHeadDim);
                 v[i] = __ldcg(ps + 32 * chunk + lane);
                 ls[i] = __ldcg(ps + kHeadDim + 1);
@@ -1543,6 +1547,39 @@ __global__ void __launch_bounds__(32 * kMergeWarps) merge_warp_kernel(const __gr
             Dn = fmaf(w, ds[i], Dn);
             Db = fmaf(w, dbs[i], Db);
             Vt = fmaf(w, vts[i], Vt);
+        }
+    }
+    if constexpr (kW > 1) {
+        __shared__ float red[kMergeWarps][38];
+        red[warp][lane] = acc;
+        if (lane == 0) {
+            red[warp][32] = M;
+            red[warp][33] = L;
+            red[warp][34] = Dn;
+            red[warp][35] = Db;
+            red[warp][36] = Vt;
+            red[warp][37] = Vm;
+        }
+        __syncthreads();
+        if (!live || sub != 0) return;
+#pragma unroll
+        for (int w = 1; w < kW; ++w) {
+            M = fmaxf(M, red[warp + w][32]);
+            Vm = fmaxf(Vm, red[warp + w][37]);
+        }
+        acc = L = Dn = Db = Vt = 0.f;
+        if (M != -INFINITY) {
+#pragma unroll
+            for (int w = 0; w < kW; ++w) {
+                const float* r = red[warp + w];
+                if (r[32] == -INFINITY) continue;
+                const float f = fast_exp2(r[32] - M);
+                acc = fmaf(f, r[lane], acc);
+                L = fmaf(f, r[33], L);
+                Dn = fmaf(f, r[34], Dn);
+                Db = fmaf(f, r[35], Db);
+                Vt = fmaf(f, r[36], Vt);
+            }
         }
     }
     const size_t cell = (size_t)b * p.num_q_heads + hq;
@@ -1590,9 +1627,15 @@ static cudaError_t launch_merge(const DecodeParams& p, cudaStream_t stream) {
         (void)cudaGetLastError();   // a refused hint leaves no sticky error behind
     });
     if (p.pages_per_split == 0 || p.splits <= kWarpMergeSplits) {   // a few partials per unit
-        const long warps = (long)p.batch * p.num_q_heads * (kHeadDim / 32);
-        return launch_pdl(merge_warp_kernel<kX>, dim3((unsigned)((warps + kMergeWarps - 1) / kMergeWarps)),
-                          dim3(32 * kMergeWarps), 0, stream, p);
+        const long items = (long)p.batch * p.num_q_heads * (kHeadDim / 32), room = 32L * num_sms;
+        auto go = [&](auto kernel, int w) {
+            const long per = kMergeWarps / w;
+            return launch_pdl(kernel, dim3((unsigned)((items + per - 1) / per)), dim3(32 * kMergeWarps), 0, stream, p);
+        };
+        if (p.pages_per_split == 0 && items * 8 <= room) return go(merge_warp_kernel<kX, 8>, 8);
+        if (p.pages_per_split == 0 && items * 4 <= room) return go(merge_warp_kernel<kX, 4>, 4);
+        if (p.pages_per_split == 0 && items * 2 <= room) return go(merge_warp_kernel<kX, 2>, 2);
+        return go(merge_warp_kernel<kX, 1>, 1);
     }
     const dim3 grid(kHeadDim / 32, p.num_q_heads, p.batch);
     const long ctas = (long)grid.x * grid.y * grid.z;
