@@ -148,98 +148,125 @@ __device__ __forceinline__ void tma_page(void* dst, const CUtensorMap* map, int 
 // A CTA's work as segments: pages [a, e) of unit (b, h); page stream (warp
 // pair) w of the CTA's n takes pages a + ((w - ph) mod n) + n i.  Split plan: one segment, the
 // CTA's split (possibly empty).  Flattened plan: CTA c serves KV head
-// h = c mod Hkv and takes share j = c / Hkv of the batch's pages laid end to
+// h = c mod Hkv and takes share j = c / Hkv of the batch laid end to
 // end (sequence after sequence), cut at sequence boundaries; the Hkv CTAs of a
 // share read the same pages together (the heads of a page are adjacent in the
-// cache).  ph keeps the streams' round robin running across the cuts, so
-// every stream gets ceil or floor of (hi - lo) / n pages.
+// cache).  A segment costs its pages and a fixed part (query setup, the CTA's merge, the
+// streams' last round), so in the layout kCutPages empty positions follow every sequence
+// with pages but the last: a share that goes on to a next sequence gets that many pages
+// less.  The shares start half of that before multiples of their length, so that
+// nearly equal sequences, one to a share, are not cut for a page or two.  4 KV heads, us a
+// decode: 2 sequences of 987 and 989 pages 21.7 without empty positions and 19.8 with 12
+// (what two take that end with a share), 16 of 280 to 512 pages 45.3 and 43.3 (with 8:
+// 43.9), 38 of 51 and 53 pages 20.0 (22.1 with shares from 0).
+// ph keeps the streams' round robin running across the cuts, so
+// every stream gets ceil or floor of the share's pages / n.
+constexpr uint32_t kCutPages = 12;  
+
 struct WsSeg {
     int b, h, a, e, ph, ctx, np;
-    long long pos;      // flattened position of page a
-    long long lo, hi;   // the CTA's share
+    uint32_t vb, hi;   // flattened plan: sequence b's first position; the share's end
+};
+
+// Positions of a sequence of np pages in the flattened layout, and positions of a share.
+__device__ __forceinline__ uint32_t flat_span(uint32_t np) { return np > 0 ? np + kCutPages : 0u; }
+struct FlatShares {
+    uint32_t total;   // positions, without the empty ones behind the last sequence
+    uint32_t R, off;  // share j: positions [j R - off, (j + 1) R - off); off < R, so share 0 has pages if any has
+    __device__ __forceinline__ FlatShares(uint32_t spans, uint32_t shares) {   // spans: sum of flat_span
+        total = spans - min(spans, kCutPages);
+        off = min(kCutPages / 2, max(1u, (total + shares - 1) / shares) - 1);
+        R = max(1u, (total + off + shares - 1) / shares);
+    }
 };
 
 __device__ __forceinline__ int clamped_ctx(const DecodeParams& p, int b) {
     return max(0, min(__ldg(p.ctx_lens + b), p.max_pages * kPage));
 }
 
-// First segment; called by every thread of the CTA (the flattened plan scans
-// the batch's page counts with two block barriers).  False: no pages.
-template <bool kFlat>
-__device__ __forceinline__ bool ws_first_segment(const DecodeParams& p, WsSeg& sg, int* s_wtot, long long* s_start) {
-    if constexpr (!kFlat) {
-        sg.b = blockIdx.z;
-        sg.h = blockIdx.y;
-        int ctx = __ldg(p.ctx_lens + sg.b);
-        if (ctx < 0 || ctx > p.max_pages * kPage) {
-            if (threadIdx.x == 0 && blockIdx.x == 0 && sg.h == 0) atomicOr(p.status, WC_DEV_BAD_CTX);
-            ctx = max(0, min(ctx, p.max_pages * kPage));
-        }
-        sg.ctx = ctx;
-        sg.np = (ctx + kPage - 1) / kPage;
-        sg.a = blockIdx.x * p.pages_per_split;
-        sg.e = min(sg.a + p.pages_per_split, sg.np);
-        sg.ph = 0;
-        sg.pos = sg.lo = sg.hi = 0;
-        return true;
-    } else {
-        const int nt = blockDim.x, t = threadIdx.x, per = (p.batch + nt - 1) / nt;
-        int loc = 0;
-        bool bad = false;
-        for (int i = 0; i < per; ++i) {
-            const int bb = t * per + i;
-            if (bb < p.batch) {
-                const int cx = __ldg(p.ctx_lens + bb);
-                bad |= cx < 0 || cx > p.max_pages * kPage;
-                loc += (max(0, min(cx, p.max_pages * kPage)) + kPage - 1) / kPage;
-            }
-        }
-        if (bad && blockIdx.x == 0) atomicOr(p.status, WC_DEV_BAD_CTX);
-        int inc = loc;   // inclusive scan over the warp
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int v = __shfl_up_sync(0xffffffffu, inc, o);
-            if ((t & 31) >= o) inc += v;
-        }
-        if ((t & 31) == 31) s_wtot[t >> 5] = inc;
-        __syncthreads();
-        int before = 0, total = 0;
-        for (int w = 0; w < nt / 32; ++w) {
-            const int v = s_wtot[w];
-            total += v;
-            if (w < (t >> 5)) before += v;
-        }
-        const int excl = before + inc - loc;   // pages of the sequences before this thread's
-        const int hk = p.num_kv_heads, shares = max(1, p.splits / hk);
-        const long long R = max(1LL, ((long long)total + shares - 1) / shares);
-        const long long lo = (long long)(blockIdx.x / hk) * R, hi = min((long long)total, lo + R);
-        if (lo < hi && excl <= lo && lo < (long long)excl + loc) {
-            long long acc = excl;   // exactly one thread: the one whose sequences hold lo
-            for (int i = 0; i < per; ++i) {
-                const int bb = t * per + i;
-                if (bb >= p.batch) break;
-                const int np = (clamped_ctx(p, bb) + kPage - 1) / kPage;
-                if (lo < acc + np) {
-                    *s_start = ((long long)bb << 32) | (long long)(lo - acc);
-                    break;
-                }
-                acc += np;
-            }
-        }
-        __syncthreads();
-        if (lo >= hi) return false;
-        const long long st = *s_start;
-        sg.b = (int)(st >> 32);
-        sg.a = (int)(st & 0xffffffffLL);
-        sg.h = blockIdx.x % hk;
-        sg.ctx = clamped_ctx(p, sg.b);
-        sg.np = (sg.ctx + kPage - 1) / kPage;
-        sg.e = (int)min((long long)sg.np, sg.a + (hi - lo));
-        sg.ph = 0;
-        sg.pos = sg.lo = lo;
-        sg.hi = hi;
-        return true;
+// The split plan's segment of this CTA.
+__device__ __forceinline__ void split_segment(const DecodeParams& p, WsSeg& sg) {
+    sg.b = blockIdx.z;
+    sg.h = blockIdx.y;
+    int ctx = __ldg(p.ctx_lens + sg.b);
+    if (ctx < 0 || ctx > p.max_pages * kPage) {
+        if (threadIdx.x == 0 && blockIdx.x == 0 && sg.h == 0) atomicOr(p.status, WC_DEV_BAD_CTX);
+        ctx = max(0, min(ctx, p.max_pages * kPage));
     }
+    sg.ctx = ctx;
+    sg.np = (ctx + kPage - 1) / kPage;
+    sg.a = blockIdx.x * p.pages_per_split;
+    sg.e = min(sg.a + p.pages_per_split, sg.np);
+    sg.ph = 0;
+    sg.vb = sg.hi = 0;
+}
+
+// First segment of the flattened plan; called by every thread of the CTA (a scan of the
+// batch's page counts with two block barriers).  cx: this thread's context length, when the
+// batch has at most a sequence per thread.  False: no pages.  All positions fit
+// in 32 bits (the plan's condition on batch * max_pages, and kCutPages more a sequence).
+struct FlatScratch {
+    uint32_t wtot[32];
+    int b, a, ctx;
+    uint32_t vb;
+};
+__device__ __forceinline__ bool flat_first_segment(const DecodeParams& p, WsSeg& sg, FlatScratch& s, int cx, bool& bad) {
+    const int nt = blockDim.x, t = threadIdx.x, per = (p.batch + nt - 1) / nt, cap = p.max_pages * kPage;
+    auto length = [&](int i) { return per == 1 ? cx : __ldg(p.ctx_lens + t * per + i); };
+    uint32_t loc = 0;
+    bad = false;
+    for (int i = 0; i < per; ++i)
+        if (t * per + i < p.batch) {
+            const int len = length(i);
+            bad |= len < 0 || len > cap;
+            loc += flat_span((uint32_t)(max(0, min(len, cap)) + kPage - 1) / kPage);
+        }
+    uint32_t inc = loc;   // inclusive scan over the warp
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t v = __shfl_up_sync(0xffffffffu, inc, o);
+        if ((t & 31) >= o) inc += v;
+    }
+    if ((t & 31) == 31) s.wtot[t >> 5] = inc;
+    if (t == 0) s.b = -1;
+    __syncthreads();
+    uint32_t before = 0, total = 0;
+    for (int w = 0; w < nt / 32; ++w) {
+        const uint32_t v = s.wtot[w];
+        total += v;
+        if (w < (t >> 5)) before += v;
+    }
+    const uint32_t excl = before + inc - loc;   // positions of the sequences before this thread's
+    const uint32_t hk = p.num_kv_heads, shares = max(1u, p.splits / hk);
+    const FlatShares f(total, shares);
+    const uint32_t j = (uint32_t)blockIdx.x / hk, lo = max(j * f.R, f.off) - f.off, hi = min(f.total, (j + 1) * f.R - f.off);
+    if (lo < hi && excl <= lo + kCutPages && lo < excl + loc) {   // the first page at lo or behind it
+        uint32_t vb = excl;
+        for (int i = 0; i < per && t * per + i < p.batch; ++i) {
+            const int len = max(0, min(length(i), cap));
+            const uint32_t np = (uint32_t)(len + kPage - 1) / kPage;
+            if (np > 0 && vb <= lo + kCutPages && lo < vb + np) {   // one sequence at most
+                s.b = t * per + i;
+                s.a = lo > vb ? (int)(lo - vb) : 0;
+                s.ctx = len;
+                s.vb = vb;
+                break;
+            }
+            vb += flat_span(np);
+        }
+    }
+    __syncthreads();
+    if (s.b < 0 || hi <= s.vb) return false;   // the share lies in empty positions
+    sg.b = s.b;
+    sg.a = s.a;
+    sg.h = (int)((uint32_t)blockIdx.x % hk);
+    sg.ctx = s.ctx;
+    sg.vb = s.vb;
+    sg.hi = hi;
+    sg.np = (sg.ctx + kPage - 1) / kPage;
+    sg.e = (int)min((uint32_t)sg.np, hi - sg.vb);
+    sg.ph = 0;
+    return true;
 }
 
 // Next segment of the flattened plan (the next sequence with pages); false
@@ -247,20 +274,62 @@ __device__ __forceinline__ bool ws_first_segment(const DecodeParams& p, WsSeg& s
 template <int kStreams, bool kFlat>
 __device__ __forceinline__ bool ws_next_segment(const DecodeParams& p, WsSeg& sg) {
     if constexpr (!kFlat) return false;
-    sg.pos += sg.e - sg.a;
-    if (sg.pos >= sg.hi) return false;
+    const int done = sg.ph + (sg.e - sg.a);
     do {   // sequences without pages hold no part of the share
-        if (sg.b + 1 >= p.batch) return false;
+        sg.vb += flat_span(sg.np);
+        if (sg.vb >= sg.hi || sg.b + 1 >= p.batch) return false;
         ++sg.b;
         sg.ctx = clamped_ctx(p, sg.b);
         sg.np = (sg.ctx + kPage - 1) / kPage;
     } while (sg.np == 0);
     sg.a = 0;
-    sg.e = (int)min((long long)sg.np, sg.hi - sg.pos);
-    sg.ph = (int)((sg.pos - sg.lo) % kStreams);
+    sg.e = (int)min((uint32_t)sg.np, sg.hi - sg.vb);
+    sg.ph = done % kStreams;
     return true;
 }
 
+// The flattened plan's first segment, before and after the grid-dependency wait.  While the
+// preceding kernel drains, the plan is made of the context lengths as they stand and
+// warm() may prefetch what it says (hints: read past L1, clamped into range).  After the wait the lengths
+// are read again, and the plan is made anew if one has changed.  bad: a length is out of range.
+template <typename Warm>
+__device__ __forceinline__ bool flat_plan(const DecodeParams& p, WsSeg& sg, FlatScratch& s, Warm warm) {
+    const bool single = p.batch <= (int)blockDim.x, mine = single && (int)threadIdx.x < p.batch;
+    int cx = mine ? __ldcg(p.ctx_lens + threadIdx.x) : 0;
+    bool waited = false, have, bad;
+    for (;;) {
+        if (!single && !waited) {
+            grid_dep_wait();
+            waited = true;
+        }
+        have = flat_first_segment(p, sg, s, cx, bad);
+        if (waited) break;
+        if (have) warm(sg);
+        grid_dep_wait();
+        waited = true;
+        const int now = mine ? __ldg(p.ctx_lens + threadIdx.x) : 0;
+        const bool changed = now != cx;
+        cx = now;
+        if (!__syncthreads_or(changed)) break;
+    }
+    if (bad && blockIdx.x == 0) atomicOr(p.status, WC_DEV_BAD_CTX);
+    return have;
+}
+
+// While the preceding kernel drains: a page's codes, scales and witnesses into L2.  The
+// page-table entry may still be changing, so it serves as an address only (clamped).
+__device__ __forceinline__ void warm_page(const DecodeParams& p, int b, int h, int lp, int scale_bytes) {
+    const int phys = min(max(__ldcg(p.block_table + (size_t)b * p.max_pages + lp), 0), p.num_pages - 1);
+    const size_t z = (size_t)phys * p.num_kv_heads + h;
+    bulk_prefetch_l2(p.k_codes + z * (kPage * kHeadDim), kPage * kHeadDim);
+    bulk_prefetch_l2(p.v_codes + z * (kPage * kHeadDim), kPage * kHeadDim);
+    bulk_prefetch_l2(reinterpret_cast<const uint8_t*>(p.k_scale) + z * scale_bytes, scale_bytes);
+    bulk_prefetch_l2(reinterpret_cast<const uint8_t*>(p.v_scale) + z * scale_bytes, scale_bytes);
+    bulk_prefetch_l2(p.k_witness + z * (kPage * kBands), kPage * kBands * 2);
+}
+__device__ __forceinline__ void warm_queries(const DecodeParams& p, int b, int h) {
+    bulk_prefetch_l2(p.q + ((size_t)b * p.num_q_heads + (size_t)h * p.group) * kHeadDim, p.group * kHeadDim * 2);
+}
 
 // Flattened plan: each warp's walker lives in a shared slot, so that only the
 // current segment's indices take registers in the page loop; lane 0 advances it.

@@ -87,7 +87,19 @@ __global__ void __launch_bounds__(kGwThreads, 1) decode_g32_ws_kernel(const __gr
     fence_barrier_init();
     __syncthreads();   // every barrier is initialised before any warp waits on it
     grid_dep_launch();
-    grid_dep_wait();   // q, page tables and the cache may come from the preceding kernel
+    if constexpr (!kFlat) {
+        // split plan: warm L2 while the preceding kernel drains (hints only, as in warm_page)
+        if (lane == 0 && p.max_pages > 0) {
+            const int lp = blockIdx.x * p.pages_per_split + pw;
+            if (producer) {
+                if (lp < p.max_pages && lp * kPage < __ldcg(p.ctx_lens + blockIdx.z))
+                    warm_page(p, blockIdx.z, blockIdx.y, lp, 128);
+            } else if (pw == 0) {
+                warm_queries(p, blockIdx.z, blockIdx.y);
+            }
+        }
+        grid_dep_wait();   // q, page tables and the cache may come from the preceding kernel
+    }
 
     // split plan: this pair's first page-table entry, loaded alongside the context
     // length (in bounds whatever the length; used only if the pair has pages)
@@ -101,15 +113,22 @@ __global__ void __launch_bounds__(kGwThreads, 1) decode_g32_ws_kernel(const __gr
     bool have;
     WsSeg* my_seg = nullptr;   // flattened plan: this warp's walker, in shared memory
     if constexpr (kFlat) {
-        __shared__ int s_wtot[kGwThreads / 32];
-        __shared__ long long s_start;
+        __shared__ FlatScratch s_flat;
         __shared__ WsSeg s_seg[kGwThreads / 32];
-        have = ws_first_segment<true>(p, sg, s_wtot, &s_start);
+        have = flat_plan(p, sg, s_flat, [&](const WsSeg& hint) {
+            if (lane != 0) return;
+            if (producer) {
+                if (hint.a + pw < hint.e) warm_page(p, hint.b, hint.h, hint.a + pw, 128);
+            } else if (pw == 0) {
+                warm_queries(p, hint.b, hint.h);
+            }
+        });
         my_seg = &s_seg[warp];
         if (lane == 0) *my_seg = sg;
         __syncwarp();
     } else {
-        have = ws_first_segment<false>(p, sg, nullptr, nullptr);
+        split_segment(p, sg);
+        have = true;
     }
 
     if (producer) {

@@ -638,23 +638,15 @@ __global__ void __launch_bounds__(kWsThreads, 1) decode_ws_kernel(const __grid_c
         // addresses (clamped into the cache); the loads bypass L1, which therefore
         // holds no copy that the reads after the wait could hit.
         const int b = blockIdx.z, h = blockIdx.y, p0 = blockIdx.x * p.pages_per_split;
-        const int32_t* bt_row = p.block_table + (size_t)b * p.max_pages;
         if (producer) {
             const int ctx_hint = __ldcg(p.ctx_lens + b);
-            if (p0 + pw < p.max_pages && (p0 + pw) * kPage < ctx_hint) {
-                const int ph_hint = min(max(__ldcg(bt_row + p0 + pw), 0), p.num_pages - 1);
-                const size_t z = (size_t)ph_hint * p.num_kv_heads + h;
-                bulk_prefetch_l2(p.k_codes + z * (kPage * kHeadDim), kPage * kHeadDim);
-                bulk_prefetch_l2(p.v_codes + z * (kPage * kHeadDim), kPage * kHeadDim);
-                bulk_prefetch_l2(p.k_scale + z * kPage, 32);
-                bulk_prefetch_l2(p.v_scale + z * kPage, 32);
-                bulk_prefetch_l2(p.k_witness + z * (kPage * kBands), 256);
-            }
+            if (p0 + pw < p.max_pages && (p0 + pw) * kPage < ctx_hint) warm_page(p, b, h, p0 + pw, 32);
         } else if (pw == 0) {
-            bulk_prefetch_l2(p.q + ((size_t)b * p.num_q_heads + (size_t)h * G) * kHeadDim, G * kHeadDim * 2);
+            warm_queries(p, b, h);
         }
     }
-    grid_dep_wait();   // q, page tables and the cache may come from the preceding kernel
+    // q, page tables and the cache may come from the preceding kernel (the flattened plan waits below)
+    if constexpr (!kFlat) grid_dep_wait();
 
     // Split plan: this pair's first page-table entry and the consumer's query
     // fragment are loaded alongside the context length (both in bounds
@@ -671,15 +663,22 @@ __global__ void __launch_bounds__(kWsThreads, 1) decode_ws_kernel(const __grid_c
     bool have;
     WsSeg* my_seg = nullptr;   // flattened plan: this warp's walker, in shared memory
     if constexpr (kFlat) {
-        __shared__ int s_wtot[kWsThreads / 32];
-        __shared__ long long s_start;
+        __shared__ FlatScratch s_flat;
         __shared__ WsSeg s_seg[kWsThreads / 32];
-        have = ws_first_segment<true>(p, sg, s_wtot, &s_start);
+        have = flat_plan(p, sg, s_flat, [&](const WsSeg& hint) {
+            if (lane != 0) return;
+            if (producer) {
+                if (hint.a + pw < hint.e) warm_page(p, hint.b, hint.h, hint.a + pw, 32);
+            } else if (pw == 0) {
+                warm_queries(p, hint.b, hint.h);
+            }
+        });
         my_seg = &s_seg[warp];
         if (lane == 0) *my_seg = sg;
         __syncwarp();
     } else {
-        have = ws_first_segment<false>(p, sg, nullptr, nullptr);
+        split_segment(p, sg);
+        have = true;
     }
 
     if (producer) {
@@ -823,7 +822,11 @@ __global__ void __launch_bounds__(kWsThreads, 1) decode_ws_kernel(const __grid_c
     auto consume = [&](const WsSeg& cs) {
         const int b = cs.b, h = cs.h, ctx = cs.ctx;
         const bool row_valid = g < G;
-        if constexpr (kFlat) load_q_frag(p, b, h, G, g, c, qw);
+        if constexpr (kFlat) {
+            load_q_frag(p, b, h, G, g, c, qw);
+            if (pw == 0 && lane == 0 && cs.vb + cs.np + kCutPages < cs.hi && b + 1 < p.batch)
+                warm_queries(p, b + 1, h);   // of the next segment (or of a sequence without pages)
+        }
         float qsum = 0.f, part[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
         for (int i = 0; i < 16; ++i) {
@@ -1484,26 +1487,26 @@ __global__ void __launch_bounds__(32 * kMergeWarps) merge_warp_kernel(const __gr
         base = p.partials + ((size_t)b * p.num_kv_heads + h) * p.splits * (kMaxGroup * kPartialStride) +
                hh * kPartialStride;
     } else {
-        // Flattened plan.  The batch's pages lie end to end (sequence b from
-        // P_b = sum_{b' < b} n_b', page counts of the clamped context lengths, as
-        // in the decode); share j of the splits / Hkv shares took positions
-        // [j R, (j + 1) R), R = ceil(total / shares), in each head, so the unit's
-        // segments are those of shares P_b / R .. (P_b + n_b - 1) / R, stored at
-        // partials h (shares + batch) + j + b, consecutive.
-        uint32_t before = 0, total = 0, nb = 0;   // below 2^31 (the plan's condition)
+        // Flattened plan.  The sequences lie end to end, the n_b > 0 pages of sequence b
+        // from P_b on and kCutPages empty positions behind them (lengths clamped, as in the
+        // decode); share j of the splits / Hkv shares took positions
+        // [j R - off, (j + 1) R - off) in each head, so the unit's segments are those of
+        // shares (P_b + off) / R .. (P_b + off + n_b - 1) / R, stored at partials
+        // h (shares + batch) + j + b, consecutive.
+        uint32_t before = 0, total = 0, nb = 0;
         for (int i = lane; i < p.batch; i += 32) {
-            const uint32_t np = (uint32_t)(clamped_ctx(p, i) + kPage - 1) / kPage;
-            total += np;
-            if (i < b) before += np;
+            const uint32_t np = (uint32_t)(clamped_ctx(p, i) + kPage - 1) / kPage, span = flat_span(np);
+            total += span;
+            if (i < b) before += span;
             if (i == b) nb = np;
         }
         total = __reduce_add_sync(0xffffffffu, total);
         before = __reduce_add_sync(0xffffffffu, before);
         nb = __reduce_add_sync(0xffffffffu, nb);
         const uint32_t shares = max(1, p.splits / p.num_kv_heads);
-        const uint32_t R = max(1u, (total + shares - 1) / shares);
-        const uint32_t j0 = before / R;
-        count = nb > 0 ? (int)((before + nb - 1) / R - j0 + 1) : 0;
+        const FlatShares f(total, shares);
+        const uint32_t j0 = (before + f.off) / f.R;
+        count = nb > 0 ? (int)((before + f.off + nb - 1) / f.R - j0 + 1) : 0;
         base = p.partials + ((size_t)h * (shares + p.batch) + (size_t)(j0 + b)) * (kMaxGroup * kPartialStride) +
                hh * kPartialStride;
     }

@@ -1,6 +1,7 @@
 """Batches under the flattened split plan (whose cuts depend on every length) against each
 sequence decoded on its own: one long sequence among short ones, empty ones, lengths
-at the edges of pages and shares, at batch sizes that take every width of the merge."""
+at the edges of pages and shares, at batch sizes that take every width of the merge; and
+contexts that change between a captured step's replays."""
 
 import numpy as np
 import pytest
@@ -67,3 +68,29 @@ def test_flat_batch_matches_its_sequences(batch, hq, hkv, kind, scheme, variant)
         one = decode(q[b:b + 1].contiguous(), table[b:b + 1].contiguous(), ctx[b:b + 1].contiguous())
         for i, (x, y) in enumerate(zip(got, one)):
             assert_close(x[b:b + 1].cpu().numpy(), y.cpu().numpy(), f"output {i} of sequence {b}, {lens[b]} tokens")
+
+
+@pytest.mark.parametrize("scheme", ["int8", "g32"])
+def test_contexts_change_between_replays(scheme):
+    """A captured decode follows the lengths that the preceding kernel of the stream writes."""
+    import paper_2607_28699_gb300 as wc
+    code = wc.SCHEME_DITHER_INT8_G32 if scheme == "g32" else wc.SCHEME_DITHER_INT8
+    full = [900, 33, 2400, 16]
+    desc, table, ctx, q, cache = _batch(full, code, 28, 4)
+    ws = wc.Workspace(desc, 4, table.shape[1])
+    src = ctx.clone()
+    outs = wc.metered_decode_attention(desc, 0, q, table, ctx, cache, ws)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        ctx.copy_(src)
+        wc.metered_decode_attention(desc, 0, q, table, ctx, cache, ws, *outs)
+    for lens in (full, [1, 33, 1999, 5], [0, 0, 2400, 0], [899, 32, 17, 16], full):
+        src.copy_(torch.tensor(lens, dtype=torch.int32))
+        graph.replay()
+        torch.cuda.synchronize()
+        assert wc.read_status(ws) == 0
+        want = wc.metered_decode_attention(desc, 0, q, table, torch.tensor(lens, dtype=torch.int32, device="cuda"), cache,
+                                           wc.Workspace(desc, 4, table.shape[1]))
+        for x, y in zip(outs, want):
+            assert torch.equal(x, y)
