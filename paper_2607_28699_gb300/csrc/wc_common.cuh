@@ -250,6 +250,9 @@ __device__ __forceinline__ void bulk_prefetch_l2(const void* src, uint32_t bytes
     asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(src), "r"(bytes) : "memory");
 }
 
+// The line of p into L2 (a hint; any alignment).
+__device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
+
 // One lane of a converged warp.  Unlike a lane test it keeps the guarded code on
 // the uniform path, which bulk copies take their operands from.
 __device__ __forceinline__ bool elect_one() {

@@ -62,7 +62,7 @@ __global__ void __launch_bounds__(128, write_min_blocks(kScheme, kBits)) write_k
     __shared__ __align__(16) uint8_t xrows[kGrouped ? 4 * 4 * kXRowStride : 16];   // [warp][unit][row]
     __shared__ BypassTable btab;
     grid_dep_launch();    // a dependent decode may be scheduled now: it waits for this whole grid
-    grid_dep_wait();      // inputs may come from the preceding kernel
+    if constexpr (kPerHead) grid_dep_wait();   // inputs may come from the preceding kernel
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const BypassTable* tab = nullptr;
     if constexpr (kGrouped && kPerHead) {   // one KV head per CTA: its bypass set, once
@@ -108,15 +108,22 @@ __global__ void __launch_bounds__(128, write_min_blocks(kScheme, kBits)) write_k
             h = idx - tok * p.num_kv_heads;
         }
     }
+    auto row_src = [&](int row) {   // 0 = K, 1 = V
+        return reinterpret_cast<const uint4*>((row == 0 ? p.k : p.v) + ((size_t)tok * p.num_kv_heads + h) * kHeadDim +
+                                              sub * 16);
+    };
+    if constexpr (!kPerHead) {   // a decode step's write: its rows reach L2 while the preceding kernel drains
+        if (live) prefetch_l2(row_src(warp & 1));
+        grid_dep_wait();
+    }
     const int slot = live ? __ldg(p.slot_mapping + tok) : -1;
     uint4 raw[kTasks][2];
 #pragma unroll
     for (int t = 0; t < kTasks; ++t) {
-        const int row = kTasks == 1 ? (warp & 1) : t;                          // 0 = K, 1 = V
+        const int row = kTasks == 1 ? (warp & 1) : t;
         raw[t][0] = raw[t][1] = make_uint4(0, 0, 0, 0);
         if (live) {
-            const uint4* src = reinterpret_cast<const uint4*>(
-                (row == 0 ? p.k : p.v) + ((size_t)tok * p.num_kv_heads + h) * kHeadDim + sub * 16);
+            const uint4* src = row_src(row);
             raw[t][0] = __ldg(src);
             raw[t][1] = __ldg(src + 1);
         }
