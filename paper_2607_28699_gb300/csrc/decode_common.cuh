@@ -144,6 +144,10 @@ __device__ __forceinline__ void tma_page(void* dst, const CUtensorMap* map, int 
         : "memory");
 }
 
+// Fetches a tensor map ahead of its first copy.
+__device__ __forceinline__ void prefetch_map(const CUtensorMap* map) {
+    asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(map)) : "memory");
+}
 
 // A CTA's work as segments: pages [a, e) of unit (b, h); page stream (warp
 // pair) w of the CTA's n takes pages a + ((w - ph) mod n) + n i.  Split plan: one segment, the

@@ -620,6 +620,10 @@ __global__ void __launch_bounds__(kWsThreads, 1) decode_ws_kernel(const __grid_c
     uint8_t* stages = smem + pw * kWsStages * St::kBytes;
     uint64_t* full = reinterpret_cast<uint64_t*>(smem + Sm::kStages) + pw * 2 * kWsStages;
     uint64_t* empty = full + kWsStages;
+    if (kBits == 10 && threadIdx.x == 32 * kWsPairs) {   // 10-bit: 1.6% off a step and no spills; 8-bit: nothing
+        prefetch_map(&wp.k_map);
+        prefetch_map(&wp.v_map);
+    }
     if (producer && lane == 0)
         for (int s = 0; s < kWsStages; ++s) {
             mbar_init(&full[s], 2);
@@ -1458,17 +1462,23 @@ constexpr int kMergeSpreadSmem = 118784;
 // decode with kW = 1, 21.2 with 8, sequences of 1975 and 1 pages 28.3 and 21.9.  A batch of
 // many sequences has few cuts each, and more CTAs only start later: 16 sequences of 387
 // pages 44.7 us with kW = 1 or 2, 45.8 with 4; 38 of 52 pages 19.4 with 1, 21.3 with 2.
-// So kW is the largest of 8, 4, 2, 1 that keeps the launch within 32 warps per SM.
+// So kW is the largest of 8, 4, 2, 1 that keeps the launch within 24 warps per SM, the
+// three CTAs that fit with the value side's 80 registers (kW = 1, of any size: four).
 constexpr int kWarpMergeSplits = 8;
 
 template <int kX, int kW>
-__global__ void __launch_bounds__(32 * kMergeWarps) merge_warp_kernel(const __grid_constant__ DecodeParams p) {
+__global__ void __launch_bounds__(32 * kMergeWarps, kW == 1 ? 4 : 3) merge_warp_kernel(const __grid_constant__ DecodeParams p) {
     grid_dep_launch();   // the next kernel waits for this grid before reading its outputs
-    grid_dep_wait();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, sub = warp % kW;
     const long long item = (long long)blockIdx.x * (kMergeWarps / kW) + warp / kW;
     const bool live = item < (long long)p.batch * p.num_q_heads * (kHeadDim / 32);   // warp-uniform
     if (kW == 1 && !live) return;
+    // Flattened plan, at most a sequence per lane: the partials are found from the context
+    // lengths as they stand before the wait (hints: read past L1).  After it the lengths are
+    // read again next to the partials, which are folded anew if one has changed.
+    // 2 sequences of 988 pages: 20.0 -> 18.7 us a decode; 16 of 387: 42.6 -> 41.4.
+    const bool hinted = p.pages_per_split == 0 && p.batch <= 32;
+    int cx = hinted && lane < p.batch ? __ldcg(p.ctx_lens + lane) : 0;
     const int chunk = (int)(item % (kHeadDim / 32));
     const int hq = (int)((item / (kHeadDim / 32)) % p.num_q_heads);
     const int b = (int)(item / ((kHeadDim / 32) * p.num_q_heads));
@@ -1477,80 +1487,95 @@ __global__ void __launch_bounds__(32 * kMergeWarps) merge_warp_kernel(const __gr
 
     int count = 0;
     const float* base = nullptr;
-    if (!live) {
-    } else if (p.pages_per_split > 0) {
-        // Split plan: the unit's splits are consecutive; those past the
-        // sequence's last page hold no pages (their maximum is -inf) and are
-        // not read.
-        const int nb = (clamped_ctx(p, b) + kPage - 1) / kPage;
-        count = min(p.splits, (nb + p.pages_per_split - 1) / p.pages_per_split);
-        base = p.partials + ((size_t)b * p.num_kv_heads + h) * p.splits * (kMaxGroup * kPartialStride) +
-               hh * kPartialStride;
-    } else {
-        // Flattened plan.  The sequences lie end to end, the n_b > 0 pages of sequence b
-        // from P_b on and kCutPages empty positions behind them (lengths clamped, as in the
-        // decode); share j of the splits / Hkv shares took positions
-        // [j R - off, (j + 1) R - off) in each head, so the unit's segments are those of
-        // shares (P_b + off) / R .. (P_b + off + n_b - 1) / R, stored at partials
-        // h (shares + batch) + j + b, consecutive.
-        uint32_t before = 0, total = 0, nb = 0;
-        for (int i = lane; i < p.batch; i += 32) {
-            const uint32_t np = (uint32_t)(clamped_ctx(p, i) + kPage - 1) / kPage, span = flat_span(np);
-            total += span;
-            if (i < b) before += span;
-            if (i == b) nb = np;
+    auto find = [&] {
+        if (!live) return;
+        if (p.pages_per_split > 0) {
+            // Split plan: the unit's splits are consecutive; those past the
+            // sequence's last page hold no pages (their maximum is -inf) and are
+            // not read.
+            const int nb = (clamped_ctx(p, b) + kPage - 1) / kPage;
+            count = min(p.splits, (nb + p.pages_per_split - 1) / p.pages_per_split);
+            base = p.partials + ((size_t)b * p.num_kv_heads + h) * p.splits * (kMaxGroup * kPartialStride) +
+                   hh * kPartialStride;
+        } else {
+            // Flattened plan.  The sequences lie end to end, the n_b > 0 pages of sequence b
+            // from P_b on and kCutPages empty positions behind them (lengths clamped, as in the
+            // decode); share j of the splits / Hkv shares took positions
+            // [j R - off, (j + 1) R - off) in each head, so the unit's segments are those of
+            // shares (P_b + off) / R .. (P_b + off + n_b - 1) / R, stored at partials
+            // h (shares + batch) + j + b, consecutive.
+            uint32_t before = 0, total = 0, nb = 0;
+            for (int i = lane; i < p.batch; i += 32) {
+                const int len = hinted ? cx : __ldg(p.ctx_lens + i);
+                const uint32_t np = (uint32_t)(max(0, min(len, p.max_pages * kPage)) + kPage - 1) / kPage;
+                const uint32_t span = flat_span(np);
+                total += span;
+                if (i < b) before += span;
+                if (i == b) nb = np;
+            }
+            total = __reduce_add_sync(0xffffffffu, total);
+            before = __reduce_add_sync(0xffffffffu, before);
+            nb = __reduce_add_sync(0xffffffffu, nb);
+            const uint32_t shares = max(1, p.splits / p.num_kv_heads);
+            const FlatShares f(total, shares);
+            const uint32_t j0 = (before + f.off) / f.R;
+            count = nb > 0 ? (int)((before + f.off + nb - 1) / f.R - j0 + 1) : 0;
+            base = p.partials + ((size_t)h * (shares + p.batch) + (size_t)(j0 + b)) * (kMaxGroup * kPartialStride) +
+                   hh * kPartialStride;
         }
-        total = __reduce_add_sync(0xffffffffu, total);
-        before = __reduce_add_sync(0xffffffffu, before);
-        nb = __reduce_add_sync(0xffffffffu, nb);
-        const uint32_t shares = max(1, p.splits / p.num_kv_heads);
-        const FlatShares f(total, shares);
-        const uint32_t j0 = (before + f.off) / f.R;
-        count = nb > 0 ? (int)((before + f.off + nb - 1) / f.R - j0 + 1) : 0;
-        base = p.partials + ((size_t)h * (shares + p.batch) + (size_t)(j0 + b)) * (kMaxGroup * kPartialStride) +
-               hh * kPartialStride;
-    }
+    };
+    if (hinted) find();
+    grid_dep_wait();
+    const int now = hinted && lane < p.batch ? __ldg(p.ctx_lens + lane) : 0;
+    if (!hinted) find();
 
     constexpr int kRows = 8;   // rows loaded per round before any is combined
     float M = -INFINITY, acc = 0.f, L = 0.f, Dn = 0.f, Db = 0.f, Vt = 0.f, Vm = 0.f;
-    for (int s0 = sub; s0 < count; s0 += kRows * kW) {
-        float ms[kRows], v[kRows], ls[kRows], ds[kRows], dbs[kRows], vts[kRows];
+    for (bool again = hinted;; again = false) {
+        for (int s0 = sub; s0 < count; s0 += kRows * kW) {
+            float ms[kRows], v[kRows], ls[kRows], ds[kRows], dbs[kRows], vts[kRows];
 #pragma unroll
-        for (int i = 0; i < kRows; ++i) {
-            ms[i] = -INFINITY;
-            v[i] = ls[i] = ds[i] = dbs[i] = vts[i] = 0.f;
-            if (s0 + i * kW < count) {
-                const float* ps = base + (size_t)(s0 + i * kW) * (kMaxGroup * kPartialStride);
-                ms[i] = __ldcg(ps + kHeadDim);
-                v[i] = __ldcg(ps + 32 * chunk + lane);
-                ls[i] = __ldcg(ps + kHeadDim + 1);
-                ds[i] = __ldcg(ps + kHeadDim + 2);
-                if (tier_b) dbs[i] = __ldcg(ps + kHeadDim + 3);
-                if (vside) {
-                    vts[i] = __ldcg(ps + kHeadDim + 4);
-                    Vm = fmaxf(Vm, __ldcg(ps + kHeadDim + 5));
+            for (int i = 0; i < kRows; ++i) {
+                ms[i] = -INFINITY;
+                v[i] = ls[i] = ds[i] = dbs[i] = vts[i] = 0.f;
+                if (s0 + i * kW < count) {
+                    const float* ps = base + (size_t)(s0 + i * kW) * (kMaxGroup * kPartialStride);
+                    ms[i] = __ldcg(ps + kHeadDim);
+                    v[i] = __ldcg(ps + 32 * chunk + lane);
+                    ls[i] = __ldcg(ps + kHeadDim + 1);
+                    ds[i] = __ldcg(ps + kHeadDim + 2);
+                    if (tier_b) dbs[i] = __ldcg(ps + kHeadDim + 3);
+                    if (vside) {
+                        vts[i] = __ldcg(ps + kHeadDim + 4);
+                        Vm = fmaxf(Vm, __ldcg(ps + kHeadDim + 5));
+                    }
                 }
             }
-        }
-        float Mr = M;
+            float Mr = M;
 #pragma unroll
-        for (int i = 0; i < kRows; ++i) Mr = fmaxf(Mr, ms[i]);
-        if (Mr == -INFINITY) continue;
-        if (Mr > M) {
-            const float f = (M == -INFINITY) ? 0.f : fast_exp2(M - Mr);
-            acc *= f; L *= f; Dn *= f; Db *= f; Vt *= f;
-            M = Mr;
-        }
+            for (int i = 0; i < kRows; ++i) Mr = fmaxf(Mr, ms[i]);
+            if (Mr == -INFINITY) continue;
+            if (Mr > M) {
+                const float f = (M == -INFINITY) ? 0.f : fast_exp2(M - Mr);
+                acc *= f; L *= f; Dn *= f; Db *= f; Vt *= f;
+                M = Mr;
+            }
 #pragma unroll
-        for (int i = 0; i < kRows; ++i) {
-            if (ms[i] == -INFINITY) continue;
-            const float w = fast_exp2(ms[i] - M);
-            acc = fmaf(w, v[i], acc);
-            L = fmaf(w, ls[i], L);
-            Dn = fmaf(w, ds[i], Dn);
-            Db = fmaf(w, dbs[i], Db);
-            Vt = fmaf(w, vts[i], Vt);
+            for (int i = 0; i < kRows; ++i) {
+                if (ms[i] == -INFINITY) continue;
+                const float w = fast_exp2(ms[i] - M);
+                acc = fmaf(w, v[i], acc);
+                L = fmaf(w, ls[i], L);
+                Dn = fmaf(w, ds[i], Dn);
+                Db = fmaf(w, dbs[i], Db);
+                Vt = fmaf(w, vts[i], Vt);
+            }
         }
+        if (!again || !__any_sync(0xffffffffu, now != cx)) break;
+        cx = now;
+        find();
+        M = -INFINITY;
+        acc = L = Dn = Db = Vt = Vm = 0.f;
     }
     if constexpr (kW > 1) {
         __shared__ float red[kMergeWarps][38];
@@ -1630,7 +1655,7 @@ static cudaError_t launch_merge(const DecodeParams& p, cudaStream_t stream) {
         (void)cudaGetLastError();   // a refused hint leaves no sticky error behind
     });
     if (p.pages_per_split == 0 || p.splits <= kWarpMergeSplits) {   // a few partials per unit
-        const long items = (long)p.batch * p.num_q_heads * (kHeadDim / 32), room = 32L * num_sms;
+        const long items = (long)p.batch * p.num_q_heads * (kHeadDim / 32), room = 24L * num_sms;
         auto go = [&](auto kernel, int w) {
             const long per = kMergeWarps / w;
             return launch_pdl(kernel, dim3((unsigned)((items + per - 1) / per)), dim3(32 * kMergeWarps), 0, stream, p);
