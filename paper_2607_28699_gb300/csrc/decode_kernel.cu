@@ -263,49 +263,63 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) decode_kernel(const __gr
                 const uint32_t A[4] = {wa, wb, wa, wb};
                 mma16816(cb, A, a_hi, a_lo);
             }
-            float y[4], P[4];
-            const bool ok0 = g < nvalid, ok1 = g + 8 < nvalid;
+            float y[4], P[4], cl[4];     // cl: the bounds in log2 units
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
-                const bool ok = (i >> 1) ? ok1 : ok0;
-                y[i] = ok ? dc[i] * kRsdLog2e : -INFINITY;
-                if (!ok) cb[i] = 0.f;                 // tail slots may hold any bits
+                y[i] = dc[i] * kRsdLog2e;
+                cl[i] = cb[i] * kLog2e;
             }
-            float rho[2] = {0.f, 0.f};   // value witness of tokens g, g+8 (0 past the context)
+            float rho[2] = {0.f, 0.f}, vn[2] = {0.f, 0.f};   // value witness of tokens g, g+8 (0 past the context)
             if constexpr (kValue) {
                 const float2 w0 = __half22float2(*reinterpret_cast<const __half2*>(st + kOffVw + 4 * g));
                 const float2 w1 = __half22float2(*reinterpret_cast<const __half2*>(st + kOffVw + 4 * (g + 8)));
-                if (ok0) { rho[0] = w0.x; vmax = fmaxf(vmax, w0.y); }
-                if (ok1) { rho[1] = w1.x; vmax = fmaxf(vmax, w1.y); }
+                rho[0] = w0.x;
+                rho[1] = w1.x;
+                vn[0] = w0.y;
+                vn[1] = w1.y;
             }
-            float mx0 = fmaxf(y[0], y[2]), mx1 = fmaxf(y[1], y[3]);
+            // One warp vote finds everything that an ordinary page does not need: the
+            // context's last page, a logit more than 8 above the reference, a bound of
+            // kHugeLog2 or more (meter_term).  Masks, six shuffles of the maximum and the
+            // second vote on every page cost 2% (32 sequences, two layers: 245.6 -> 240.1 us).
+            const float big = fmaxf(fmaxf(cl[0], cl[1]), fmaxf(cl[2], cl[3]));
+            bool huge = false;
+            if (__any_sync(0xffffffffu, nvalid < kPage || fmaxf(y[0], y[2]) > m_run[0] + 8.0f ||
+                                            fmaxf(y[1], y[3]) > m_run[1] + 8.0f || !(big < kHugeLog2))) {
+                const bool ok0 = g < nvalid, ok1 = g + 8 < nvalid;
 #pragma unroll
-            for (int o = 4; o < 32; o <<= 1) {
-                mx0 = fmaxf(mx0, __shfl_xor_sync(0xffffffffu, mx0, o));
-                mx1 = fmaxf(mx1, __shfl_xor_sync(0xffffffffu, mx1, o));
-            }
-            const bool mv0 = mx0 > m_run[0] + 8.0f, mv1 = mx1 > m_run[1] + 8.0f;
-            if (__any_sync(0xffffffffu, mv0 || mv1)) {
-                const float a0 = mv0 ? (m_run[0] == -INFINITY ? 0.f : fast_exp2(m_run[0] - mx0)) : 1.f;
-                const float a1 = mv1 ? (m_run[1] == -INFINITY ? 0.f : fast_exp2(m_run[1] - mx1)) : 1.f;
-                if (mv0) m_run[0] = mx0;
-                if (mv1) m_run[1] = mx1;
-                l_part[0] *= a0; d_part[0] *= a0;
-                l_part[1] *= a1; d_part[1] *= a1;
-                if constexpr (kValue) { vt_part[0] *= a0; vt_part[1] *= a1; }
+                for (int i = 0; i < 4; ++i)
+                    if (!((i >> 1) ? ok1 : ok0)) {   // tail slots may hold any bits
+                        y[i] = -INFINITY;
+                        cl[i] = 0.f;
+                    }
+                if (!ok0) rho[0] = vn[0] = 0.f;
+                if (!ok1) rho[1] = vn[1] = 0.f;
+                huge = __any_sync(0xffffffffu, fmaxf(fmaxf(cl[0], cl[1]), fmaxf(cl[2], cl[3])) >= kHugeLog2);
+                float mx0 = fmaxf(y[0], y[2]), mx1 = fmaxf(y[1], y[3]);
 #pragma unroll
-                for (int mt = 0; mt < 8; ++mt) {
-                    acc[mt][0] *= a0; acc[mt][2] *= a0;
-                    acc[mt][1] *= a1; acc[mt][3] *= a1;
+                for (int o = 4; o < 32; o <<= 1) {
+                    mx0 = fmaxf(mx0, __shfl_xor_sync(0xffffffffu, mx0, o));
+                    mx1 = fmaxf(mx1, __shfl_xor_sync(0xffffffffu, mx1, o));
+                }
+                const bool mv0 = mx0 > m_run[0] + 8.0f, mv1 = mx1 > m_run[1] + 8.0f;
+                if (__any_sync(0xffffffffu, mv0 || mv1)) {
+                    const float a0 = mv0 ? (m_run[0] == -INFINITY ? 0.f : fast_exp2(m_run[0] - mx0)) : 1.f;
+                    const float a1 = mv1 ? (m_run[1] == -INFINITY ? 0.f : fast_exp2(m_run[1] - mx1)) : 1.f;
+                    if (mv0) m_run[0] = mx0;
+                    if (mv1) m_run[1] = mx1;
+                    l_part[0] *= a0; d_part[0] *= a0;
+                    l_part[1] *= a1; d_part[1] *= a1;
+                    if constexpr (kValue) { vt_part[0] *= a0; vt_part[1] *= a1; }
+#pragma unroll
+                    for (int mt = 0; mt < 8; ++mt) {
+                        acc[mt][0] *= a0; acc[mt][2] *= a0;
+                        acc[mt][1] *= a1; acc[mt][3] *= a1;
+                    }
                 }
             }
+            if constexpr (kValue) vmax = fmaxf(vmax, fmaxf(vn[0], vn[1]));
             float dpg[2] = {0.f, 0.f};   // this page's share of D (kRepair)
-            float cl[4];                 // the bounds in log2 units
-#pragma unroll
-            for (int i = 0; i < 4; ++i) cl[i] = cb[i] * kLog2e;
-            // warp-uniform: a bound of kHugeLog2 or more (meter_term)
-            const bool huge =
-                __any_sync(0xffffffffu, fmaxf(fmaxf(cl[0], cl[1]), fmaxf(cl[2], cl[3])) >= kHugeLog2);
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
                 const int r = i >> 1, e = i & 1;
@@ -351,10 +365,11 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) decode_kernel(const __gr
             const int tv[4] = {2 * c, 2 * c + 1, 2 * c + 8, 2 * c + 9};
             uint4 vq[4];
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                vq[j] = *reinterpret_cast<const uint4*>(kt + kTileRegion + swz(tv[j], g));
-                // an fp8 NaN byte in an unused tail slot would poison P = 0 columns
-                if (tv[j] >= nvalid) vq[j] = make_uint4(0, 0, 0, 0);
+            for (int j = 0; j < 4; ++j) vq[j] = *reinterpret_cast<const uint4*>(kt + kTileRegion + swz(tv[j], g));
+            if (nvalid < kPage) {   // an fp8 NaN byte in an unused tail slot would poison P = 0 columns
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+                    if (tv[j] >= nvalid) vq[j] = make_uint4(0, 0, 0, 0);
             }
 #pragma unroll
             for (int mt = 0; mt < 8; ++mt) {
