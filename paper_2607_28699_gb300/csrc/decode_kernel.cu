@@ -542,13 +542,16 @@ struct WsStage {
 constexpr int kWsBarBytes = kWsPairs * kWsStages * 2 * 8;
 // The CTA merge's buffer [warp][head][kPartialStride]: the stage area in the
 // split plan, one of its own after the barriers in the flattened plan.  There
-// the 10-bit stages (and the walkers' static slots) leave room for two heads' rows
-// at a time.
+// the 10-bit stages (and the walkers' static slots) leave room for four heads at a
+// time, their 128 outputs and six sums apart and without padding (two heads with
+// it: 32 sequences of 8 to 60 pages, 8 x 8 heads, 40.0 -> 37.2 us).
 template <int kBits, bool kFlat>
 struct WsSmem {
     static constexpr int kStages = kWsPairs * kWsStages * WsStage<kBits>::kBytes;
-    static constexpr int kMergeHeads = kFlat && kBits == 10 ? 2 : kMaxGroup;
-    static constexpr int kMergeBytes = kWsPairs * kMergeHeads * kPartialStride * 4;
+    static constexpr bool kDense = kFlat && kBits == 10;
+    static constexpr int kMergeHeads = kDense ? 4 : kMaxGroup;
+    static constexpr int kMergeRow = kDense ? kHeadDim : kPartialStride;   // floats from row to row
+    static constexpr int kMergeBytes = kWsPairs * kMergeHeads * (kDense ? kHeadDim + 6 : kPartialStride) * 4;
     static constexpr int kOffMerge = kFlat ? kStages + kWsBarBytes : 0;
     static constexpr int kBytes = kStages + kWsBarBytes + (kFlat ? kMergeBytes : 0) + 1024;   // + alignment slack
     static_assert(kBytes + (kFlat ? 1024 : 0) <= 232448, "shared memory limit of a CTA, static slots included");
@@ -1179,15 +1182,19 @@ __global__ void __launch_bounds__(kWsThreads, 1) decode_ws_kernel(const __grid_c
         // ---- CTA merge over the consumer warps: one partial per segment --------------------
         // (heads hb .. hb + kMergeHeads - 1 at a time)
         constexpr int kMH = Sm::kMergeHeads;
+        auto merge_row = [&](int w, int hh) { return mbuf + (w * kMH + hh) * Sm::kMergeRow; };
+        auto merge_sums = [&](int w, int hh) {   // m, l, D, Tier-B D, value term, max ||v||
+            return Sm::kDense ? mbuf + kWsPairs * kMH * kHeadDim + (w * kMH + hh) * 6 : merge_row(w, hh) + kHeadDim;
+        };
 #pragma unroll 1
         for (int hb = 0; hb < kMaxGroup; hb += kMH) {
         if (hb >= G) break;
         consumer_sync();   // all consumers are done with their stages and with mbuf's last use
         if (2 * c >= hb && 2 * c < hb + kMH) {
-            float* wb = mbuf + pw * kMH * kPartialStride - hb * kPartialStride;
+            float* wb = mbuf + pw * kMH * Sm::kMergeRow - hb * Sm::kMergeRow;
 #pragma unroll
             for (int e = 0; e < 2; ++e) {
-                float* row = wb + (2 * c + e) * kPartialStride;
+                float* row = wb + (2 * c + e) * Sm::kMergeRow;
                 const float add = kKappaV * spv_part[e] * inv_lam;   // spv is in the lam frame
 #pragma unroll
                 for (int mt = 0; mt < 8; ++mt) {   // m-tile rows g, g + 8: dims 16 mt + g, 16 mt + g + 8
@@ -1195,13 +1202,14 @@ __global__ void __launch_bounds__(kWsThreads, 1) decode_ws_kernel(const __grid_c
                     row[16 * mt + g + 8] = fmaf(acc[mt][e + 2], inv_lam, add);
                 }
                 if (g == 0) {
-                    wb[(2 * c + e) * kPartialStride + kHeadDim + 0] = m_run[e];
-                    wb[(2 * c + e) * kPartialStride + kHeadDim + 1] = l_part[e];
-                    wb[(2 * c + e) * kPartialStride + kHeadDim + 2] = d_part[e];
-                    if constexpr (kTierB) wb[(2 * c + e) * kPartialStride + kHeadDim + 3] = db_part[e];
+                    float* sums = Sm::kDense ? merge_sums(pw, 2 * c + e - hb) : row + kHeadDim;
+                    sums[0] = m_run[e];
+                    sums[1] = l_part[e];
+                    sums[2] = d_part[e];
+                    if constexpr (kTierB) sums[3] = db_part[e];
                     if constexpr (kValue) {
-                        wb[(2 * c + e) * kPartialStride + kHeadDim + 4] = vt_part[e];
-                        wb[(2 * c + e) * kPartialStride + kHeadDim + 5] = vmax;
+                        sums[4] = vt_part[e];
+                        sums[5] = vmax;
                     }
                 }
             }
@@ -1220,7 +1228,7 @@ __global__ void __launch_bounds__(kWsThreads, 1) decode_ws_kernel(const __grid_c
             float M = -INFINITY;
 #pragma unroll
             for (int w = 0; w < kWsPairs; ++w) {
-                mw[w] = mbuf[(w * kMH + hh) * kPartialStride + kHeadDim];
+                mw[w] = merge_sums(w, hh)[0];
                 M = fmaxf(M, mw[w]);
             }
             float4 s4 = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -1229,7 +1237,7 @@ __global__ void __launch_bounds__(kWsThreads, 1) decode_ws_kernel(const __grid_c
             for (int w = 0; w < kWsPairs; ++w) {
                 if (mw[w] == -INFINITY) continue;   // a warp without pages: its values are not read
                 const float wt = fast_exp2(mw[w] - M);
-                const float* src = mbuf + (w * kMH + hh) * kPartialStride + col;
+                const float* src = Sm::kDense && ch >= 32 ? merge_sums(w, hh) + 1 : merge_row(w, hh) + col;
                 if (ch < 32) {
                     const float4 v = *reinterpret_cast<const float4*>(src);
                     s4.x = fmaf(wt, v.x, s4.x); s4.y = fmaf(wt, v.y, s4.y);
@@ -1252,7 +1260,7 @@ __global__ void __launch_bounds__(kWsThreads, 1) decode_ws_kernel(const __grid_c
                 if constexpr (kValue) {
                     float vm = 0.f;
                     for (int w = 0; w < kWsPairs; ++w)
-                        vm = fmaxf(vm, mbuf[(w * kMH + hh) * kPartialStride + kHeadDim + 5]);
+                        vm = fmaxf(vm, merge_sums(w, hh)[5]);
                     dst[kHeadDim + 4] = s4.w;
                     dst[kHeadDim + 5] = vm;
                 }
