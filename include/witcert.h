@@ -184,7 +184,7 @@ size_t wc_workspace_size(const wc_cache_desc* desc, int32_t batch, int32_t max_p
  * underflows fp32 while its bound is huge.
  * The context is split across CTAs (one sequence: every KV head's pages in
  * equal splits; several sequences, whose lengths only the device sees: each
- * CTA serves one KV head and an equal share of the batch's pages laid end to
+ * CTA serves one KV head and a share of the batch's pages laid end to
  * end, cut at sequence boundaries); partial softmax, output and A
  * accumulators are merged under log-sum-exp weights (A is a p~-weighted mean,
  * §6.2.2) by a second kernel, launched as a programmatic dependent of the

@@ -56,7 +56,7 @@ constexpr int kOffVw = 320;              // value witness [16][2] fp16 (value si
 constexpr int kSmallStride = 384;
 constexpr int kSmemBytes = 2 * kTileRegion + kWarps * kStages * kSmallStride + kWarps * kStages * 8 + 1024;
 
-// The per-token kernel's parameters: the code tiles' tensor maps and the call.
+// decode_kernel's parameters: the code tiles' tensor maps and the call.
 struct DkParams {
     CUtensorMap k_map;   // k_codes as [num_pages * Hkv][16][128] bytes, box = one page of one head
     CUtensorMap v_map;
@@ -1433,7 +1433,8 @@ static long split_pages(long units, int max_pages, long slots, long streams) {
     return best_pps;
 }
 
-DecodePlan plan_decode(int batch, int num_kv_heads, int max_pages, int num_sms, int scheme, int bits) {
+DecodePlan plan_decode(int batch, int num_kv_heads, int max_pages, int num_sms, int scheme, int bits,
+                       size_t available) {
     DecodePlan pl;
     const long units = (long)batch * num_kv_heads;
     const long slots = std::max<long>(1, (long)num_sms * ctas_per_sm(scheme));
@@ -1443,29 +1444,47 @@ DecodePlan plan_decode(int batch, int num_kv_heads, int max_pages, int num_sms, 
     long partials = units * pl.splits;
     // A batch of several sequences (lengths unknown to the host, often ragged)
     // takes the flattened plan on the dithered caches: Hkv x floor(SMs / Hkv)
-    // CTAs, all resident, each taking equal shares of one KV head's pages.  fp8
+    // CTAs, all resident, each taking a share of one KV head's pages.  fp8
     // keeps the split plan: its CTAs are scheduled as SMs free up, which already
-    // evens out a ragged batch, and its pages are cheap.
-    const bool flat = batch > 1 && (long long)batch * max_pages < (1LL << 31) && scheme != WC_SCHEME_FP8_E4M3;
-    if (flat) {
-        pl.splits = num_kv_heads * std::max(1, (int)(slots / num_kv_heads));
-        pl.pages_per_split = 0;
-        partials = pl.splits + units;
-    }
+    // evens out a ragged batch, and its pages are cheap.  So do block tables of at most
+    // kShortRounds rounds of pages: a share there has a cut every few rounds.  4 KV heads,
+    // us split / flattened: 32 sequences of 4 pages 6.9 / 9.4, 16 of 5 to 19 8.3 / 10.3, 32 of 4
+    // to 31 12.0 / 13.3, 400 of 10 to 38 111 / 114; 8 KV heads, 32 of 8 to 60 30.4 / 28.3.
+    constexpr long kShortRounds = 5;
+    const bool batched = batch > 1 && (long long)batch * max_pages < (1LL << 31) && scheme != WC_SCHEME_FP8_E4M3;
+    const int shares = std::max(1, (int)(slots / num_kv_heads));
+    const long flat_partials = (long)num_kv_heads * shares + units;
+    auto bytes = [](long n) {
+        return (256 + sizeof(float) * (size_t)n * kMaxGroup * kPartialStride + 255) & ~(size_t)255;
+    };
+    bool flat = batched;
     if (scheme == WC_SCHEME_DITHER_INT8 && bits == 10) {
-        // The 10-bit dither's workspace keeps the size it was first given, for two
-        // CTAs per SM (and, on a batch that left some empty, a partial per warp of
-        // eight): workspaces sized once stay valid, and so does the limit of the
-        // allocation-free call.
+        // The 10-bit dither's workspace is at least the size it was first given, for two
+        // CTAs per SM (and, on a batch that left some empty, a partial per warp of eight).
+        // The flattened plan of a batch whose units fill two CTAs per SM with a split each
+        // needs up to a partial per SM more: in a workspace of the first size, and beyond
+        // the allocation-free call's limit, such a batch takes a split plan.
         const long slots2 = std::max<long>(1, 2L * num_sms), pps2 = split_pages(units, max_pages, slots2, 8);
         const long splits2 = std::max<long>(1, (max_pages + pps2 - 1) / pps2);
         long first = units * splits2;
-        if (flat && first < slots2) first = 8L * num_kv_heads * std::max<long>(1, slots2 / num_kv_heads) + units;
-        partials = std::max(partials, first);
+        if (batched && first < slots2) first = 8L * num_kv_heads * std::max<long>(1, slots2 / num_kv_heads) + units;
+        if (max_pages <= kShortRounds * streams_per_cta(scheme) && partials <= first) flat = false;
+        if (flat && flat_partials > first && bytes(flat_partials) > available) flat = false;
+        if (!flat && partials > first) {
+            pl.pages_per_split = (int)pps2;
+            pl.splits = (int)splits2;
+        }
+        partials = flat ? std::max(first, flat_partials) : first;
+    } else if (batched) {
+        if (max_pages <= kShortRounds * streams_per_cta(scheme) && partials <= flat_partials) flat = false;
+        partials = flat_partials;   // the workspace of either
     }
-    auto align = [](size_t x) { return (x + 255) & ~(size_t)255; };
+    if (flat) {
+        pl.splits = num_kv_heads * shares;
+        pl.pages_per_split = 0;
+    }
     pl.partials_off = 256;
-    pl.total = align(pl.partials_off + sizeof(float) * (size_t)partials * kMaxGroup * kPartialStride);
+    pl.total = bytes(partials);
     return pl;
 }
 

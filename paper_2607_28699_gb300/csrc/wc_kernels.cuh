@@ -67,7 +67,7 @@ struct DecodeParams {
     int32_t batch, max_pages, num_q_heads, num_kv_heads, group, num_pages, layer, rope_layout;
     // pages_per_split == 0 marks the flattened plan (warp-specialized kernel,
     // batch > 1): the grid is `splits` CTAs, a multiple of Hkv; CTA c serves KV
-    // head c mod Hkv with the (c / Hkv)-th equal share of the batch's pages laid
+    // head c mod Hkv with the (c / Hkv)-th share of the batch's pages laid
     // end to end, cut at sequence boundaries into segments.  Share j's segment of
     // sequence b writes partial h (shares + batch) + j + b (unique: along the
     // pages each next segment increments j, b or both), so splits + batch Hkv
@@ -90,7 +90,10 @@ struct DecodePlan {
     size_t partials_off, total;
 };
 
-DecodePlan plan_decode(int batch, int num_kv_heads, int max_pages, int num_sms, int scheme, int bits);
+// available: the workspace's bytes (a smaller plan is taken where the preferred one does
+// not fit and calls with that size have always been accepted); SIZE_MAX: the preferred plan.
+DecodePlan plan_decode(int batch, int num_kv_heads, int max_pages, int num_sms, int scheme, int bits,
+                       size_t available = SIZE_MAX);
 
 // Launch `kernel` on `stream` as a programmatic dependent of the preceding work.
 template <typename Kernel, typename Params>

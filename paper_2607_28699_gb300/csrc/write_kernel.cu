@@ -2,10 +2,9 @@
 // K band-norm residual witness (§6.2.1 write kernel; §4.1 Eq. witness;
 // §4.2 subtractive dither).
 //
-// A warp handles four (token, KV head) units, their K rows and then their V rows, 8
-// lanes per row.  Each lane owns 16 consecutive
-// channels, so it loads 32 B of fp16, stores 16 B of codes, and (for the dither
-// schemes) consumes exactly one Philox4x32-10 call per row and 16 channels.
+// A warp handles four (token, KV head) units, their K rows and then their V rows (few
+// units: one of the two), 8 lanes per row.  Each lane owns 16 consecutive channels, so it
+// loads 32 B of fp16, stores 16 B of codes, and (for the dither schemes) consumes exactly one Philox4x32-10 call per row and 16 channels.
 //
 // Grouped scheme (§6.2.3 "Storage side" and §6.2.5 "Fixed-channel outlier bypass"):
 // one fp16 scale per 32-channel group (a lane pair), the group amax leaving
@@ -45,9 +44,9 @@ constexpr int kPerHeadMinTokens = 16;                     // per-head grid from 
 // Two ways of cutting the units (token, KV head) into 4-unit tasks:
 //  kPerHead: grid (token groups, Hkv), a task = 4 consecutive tokens of one
 //            head, so a warp's code, scale and witness stores are contiguous
-//            runs of consecutive slots (prefill), K and V;
+//            runs of consecutive slots (prefill);
 //  else:     one index over units u = token * Hkv + h, a task = 4 consecutive
-//            units, so a one-token write of up to 8 KV heads is a single CTA
+//            units, K or V, so a one-token write of up to 8 KV heads is a single CTA
 //            (decode steps, where every SM the next decode needs counts).
 // Resident CTAs per SM the register budget is sized for, the best of 5 .. 9 in each case
 // (us at 32768 x 4): 8-bit dither seven at 72 registers 26.9 (six 28.5, eight 28.2, with

@@ -70,6 +70,47 @@ def test_flat_batch_matches_its_sequences(batch, hq, hkv, kind, scheme, variant)
             assert_close(x[b:b + 1].cpu().numpy(), y.cpu().numpy(), f"output {i} of sequence {b}, {lens[b]} tokens")
 
 
+@pytest.mark.parametrize("scheme,bits", [("int8", 8), ("int8", 10), ("g32", 8)])
+@pytest.mark.parametrize("tokens", [16, 128, 129, 480, 481, 640, 641])
+@pytest.mark.parametrize("batch", [2, 33])
+def test_short_block_tables_match_their_sequences(batch, tokens, scheme, bits):
+    """Both sides of the longest block table that a batch splits instead of flattening (30 pages
+    for the grouped cache, 40 otherwise), and of a split's pages."""
+    import paper_2607_28699_gb300 as wc
+    code = wc.SCHEME_DITHER_INT8_G32 if scheme == "g32" else wc.SCHEME_DITHER_INT8
+    lens = [tokens] + [max(1, (tokens * i) // batch) for i in range(1, batch - 1)] + [0]
+    desc, table, ctx, q, cache = _batch(lens, code, 28, 4, bits=bits)
+    got = wc.metered_decode_attention(desc, 0, q, table, ctx, cache, wc.Workspace(desc, batch, table.shape[1]))
+    for b in sorted({0, batch // 2, batch - 1}):
+        one = wc.metered_decode_attention(desc, 0, q[b:b + 1].contiguous(), table[b:b + 1].contiguous(),
+                                          ctx[b:b + 1].contiguous(), cache, wc.Workspace(desc, 1, table.shape[1]))
+        for i, (x, y) in enumerate(zip(got, one)):
+            assert_close(x[b:b + 1].cpu().numpy(), y.cpu().numpy(), f"output {i} of sequence {b}, {lens[b]} tokens")
+
+
+def test_ten_bit_batch_in_a_workspace_of_one_partial_per_unit():
+    """800 units, a split each: the flattened plan needs a partial per SM more than the split
+    plan, which a workspace of that plan's size still gets; a smaller one is refused."""
+    import paper_2607_28699_gb300 as wc
+    lens = [700] + [int(x) for x in np.random.default_rng(4).integers(1, 120, 199)]
+    desc, table, ctx, q, cache = _batch(lens, wc.SCHEME_DITHER_INT8, 8, 4, bits=10)
+    ws = wc.Workspace(desc, 200, table.shape[1])
+    least = (256 + 4 * 800 * 8 * 140 + 255) // 256 * 256
+    assert ws.nbytes > least
+    want = wc.metered_decode_attention(desc, 0, q, table, ctx, cache, ws)
+    small = wc.Workspace(desc, 200, table.shape[1])
+    small.nbytes = least
+    got = wc.metered_decode_attention(desc, 0, q, table, ctx, cache, small)
+    torch.cuda.synchronize()
+    assert not small.view[least:].any()          # nothing written behind the given size
+    for i, (x, y) in enumerate(zip(got, want)):
+        assert_close(x.cpu().numpy(), y.cpu().numpy(), f"output {i}")
+    small.nbytes = least - 256
+    with pytest.raises(wc.WitCertError) as e:
+        wc.metered_decode_attention(desc, 0, q, table, ctx, cache, small)
+    assert e.value.status == 4
+
+
 @pytest.mark.parametrize("scheme", ["int8", "g32"])
 def test_contexts_change_between_replays(scheme):
     """A captured decode follows the lengths that the preceding kernel of the stream writes."""
