@@ -613,7 +613,7 @@ def run_ours(args, rank, world, local):
         "value_side": value_side,
         "repair": repair,
         "grouped": grouped,
-        "roofline": {"kernel": ("decode_ws_kernel" if wl.scheme == 0 and args.dither_bits == 8 else "decode_kernel")
+        "roofline": {"kernel": ("decode_ws_kernel" if wl.scheme == 0 else "decode_kernel")
                                + " + merge_kernel (one metered_decode_attention call)",
                      "bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                      "frac": achieved / peak, "traffic": _traffic(wl.name),

@@ -1,5 +1,5 @@
 """The warp-specialized decode where its halves can go wrong: every group size
-(the CTA merge takes the heads of the 10-bit dither's batches two at a time), page
+(the CTA merge takes the heads of the 10-bit dither's batches four at a time), page
 counts around the eight page streams, both dithers, one sequence and batches."""
 
 import pytest
