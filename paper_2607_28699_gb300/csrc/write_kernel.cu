@@ -4,7 +4,8 @@
 //
 // A warp handles four (token, KV head) units, their K rows and then their V rows (few
 // units: one of the two), 8 lanes per row.  Each lane owns 16 consecutive channels, so it
-// loads 32 B of fp16, stores 16 B of codes, and (for the dither schemes) consumes exactly one Philox4x32-10 call per row and 16 channels.
+// loads 32 B of fp16, stores 16 B of codes, and (for the dither schemes) consumes exactly
+// one Philox4x32-10 call per row and 16 channels.
 //
 // Grouped scheme (§6.2.3 "Storage side" and §6.2.5 "Fixed-channel outlier bypass"):
 // one fp16 scale per 32-channel group (a lane pair), the group amax leaving
