@@ -1508,72 +1508,99 @@ constexpr int kMergeSpreadSmem = 118784;
 // three CTAs that fit with the value side's 80 registers (kW = 1, of any size: four).
 constexpr int kWarpMergeSplits = 8;
 
-template <int kX, int kW>
+// kHint (flattened plan, at most a sequence per lane): the partials are found from the
+// context lengths as they stand before the wait (hints: read past L1).  After it the
+// lengths are read again next to the partials, which are folded anew if one has changed.
+// 2 sequences of 988 pages: 20.0 -> 18.7 us a decode; 16 of 387: 42.6 -> 41.4.  Larger
+// batches and the split plan do without: there the second pass only cost (1000 fp8 sequences
+// of 1 to 4 pages, 28 heads: 91.2 us with it, 87.2 without).
+template <int kX, int kW, bool kHint>
 __global__ void __launch_bounds__(32 * kMergeWarps, kW == 1 ? 4 : 3) merge_warp_kernel(const __grid_constant__ DecodeParams p) {
     grid_dep_launch();   // the next kernel waits for this grid before reading its outputs
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, sub = warp % kW;
     const long long item = (long long)blockIdx.x * (kMergeWarps / kW) + warp / kW;
     const bool live = item < (long long)p.batch * p.num_q_heads * (kHeadDim / 32);   // warp-uniform
-    if (kW == 1 && !live) return;
-    // Flattened plan, at most a sequence per lane: the partials are found from the context
-    // lengths as they stand before the wait (hints: read past L1).  After it the lengths are
-    // read again next to the partials, which are folded anew if one has changed.
-    // 2 sequences of 988 pages: 20.0 -> 18.7 us a decode; 16 of 387: 42.6 -> 41.4.
-    const bool hinted = p.pages_per_split == 0 && p.batch <= 32;
-    int cx = hinted && lane < p.batch ? __ldcg(p.ctx_lens + lane) : 0;
+    if (kHint && kW == 1 && !live) return;
+    int cx = kHint && lane < p.batch ? __ldcg(p.ctx_lens + lane) : 0;
     const int chunk = (int)(item % (kHeadDim / 32));
     const int hq = (int)((item / (kHeadDim / 32)) % p.num_q_heads);
     const int b = (int)(item / ((kHeadDim / 32) * p.num_q_heads));
     const int h = hq / p.group, hh = hq % p.group;
     constexpr bool tier_b = (kX & kXTierB) != 0, vside = (kX & kXValue) != 0, repair = (kX & kXRepair) != 0;
 
+    // A sequence's span in the flattened layout.
+    auto span_of = [&](int len) {
+        return flat_span((uint32_t)(max(0, min(len, p.max_pages * kPage)) + kPage - 1) / kPage);
+    };
+    // Flattened plan.  The sequences lie end to end, the n_b > 0 pages of sequence b
+    // from P_b on and kCutPages empty positions behind them (lengths clamped, as in the
+    // decode); share j of the splits / Hkv shares took positions
+    // [j R - off, (j + 1) R - off) in each head, so the unit's segments are those of
+    // shares (P_b + off) / R .. (P_b + off + n_b - 1) / R, stored at partials
+    // h (shares + batch) + j + b, consecutive.
     int count = 0;
     const float* base = nullptr;
-    auto find = [&] {
-        if (!live) return;
+    auto find_flat = [&](uint32_t before, uint32_t total, uint32_t nb) {
+        const uint32_t shares = max(1, p.splits / p.num_kv_heads);
+        const FlatShares f(total, shares);
+        const uint32_t j0 = (before + f.off) / f.R;
+        count = nb > 0 ? (int)((before + f.off + nb - 1) / f.R - j0 + 1) : 0;
+        base = p.partials + ((size_t)h * (shares + p.batch) + (size_t)(j0 + b)) * (kMaxGroup * kPartialStride) +
+               hh * kPartialStride;
+    };
+    auto find_hinted = [&] {
+        if (kW > 1 && !live) return;
+        const uint32_t span = lane < p.batch ? span_of(cx) : 0u, own = __shfl_sync(0xffffffffu, span, b);
+        find_flat(__reduce_add_sync(0xffffffffu, lane < b ? span : 0u), __reduce_add_sync(0xffffffffu, span),
+                  own > 0 ? own - kCutPages : 0u);
+    };
+    int now = 0;
+    if constexpr (kHint) {
+        find_hinted();
+        grid_dep_wait();
+        now = lane < p.batch ? __ldg(p.ctx_lens + lane) : 0;
+    } else {
+        grid_dep_wait();
         if (p.pages_per_split > 0) {
             // Split plan: the unit's splits are consecutive; those past the
             // sequence's last page hold no pages (their maximum is -inf) and are
             // not read.
+            if (!live) return;   // (a warp per output)
             const int nb = (clamped_ctx(p, b) + kPage - 1) / kPage;
             count = min(p.splits, (nb + p.pages_per_split - 1) / p.pages_per_split);
             base = p.partials + ((size_t)b * p.num_kv_heads + h) * p.splits * (kMaxGroup * kPartialStride) +
                    hh * kPartialStride;
         } else {
-            // Flattened plan.  The sequences lie end to end, the n_b > 0 pages of sequence b
-            // from P_b on and kCutPages empty positions behind them (lengths clamped, as in the
-            // decode); share j of the splits / Hkv shares took positions
-            // [j R - off, (j + 1) R - off) in each head, so the unit's segments are those of
-            // shares (P_b + off) / R .. (P_b + off + n_b - 1) / R, stored at partials
-            // h (shares + batch) + j + b, consecutive.
-            uint32_t before = 0, total = 0, nb = 0;
-            for (int i = lane; i < p.batch; i += 32) {
-                const int len = hinted ? cx : __ldg(p.ctx_lens + i);
-                const uint32_t np = (uint32_t)(max(0, min(len, p.max_pages * kPage)) + kPage - 1) / kPage;
-                const uint32_t span = flat_span(np);
+            // The CTA's threads add up the spans together, up to the sequence of its first
+            // output (a scan by every warp: 1000 sequences of 45 pages, 56 heads, 822 us a
+            // decode; so 722).
+            __shared__ uint32_t sums[2][kMergeWarps];
+            const int b0 = (int)((long long)blockIdx.x * (kMergeWarps / kW) / ((kHeadDim / 32) * p.num_q_heads));
+            uint32_t before = 0, total = 0;
+            for (int i = threadIdx.x; i < p.batch; i += 32 * kMergeWarps) {
+                const uint32_t span = span_of(__ldg(p.ctx_lens + i));
                 total += span;
-                if (i < b) before += span;
-                if (i == b) nb = np;
+                if (i < b0) before += span;
             }
             total = __reduce_add_sync(0xffffffffu, total);
             before = __reduce_add_sync(0xffffffffu, before);
-            nb = __reduce_add_sync(0xffffffffu, nb);
-            const uint32_t shares = max(1, p.splits / p.num_kv_heads);
-            const FlatShares f(total, shares);
-            const uint32_t j0 = (before + f.off) / f.R;
-            count = nb > 0 ? (int)((before + f.off + nb - 1) / f.R - j0 + 1) : 0;
-            base = p.partials + ((size_t)h * (shares + p.batch) + (size_t)(j0 + b)) * (kMaxGroup * kPartialStride) +
-                   hh * kPartialStride;
+            if (lane == 0) {
+                sums[0][warp] = before;
+                sums[1][warp] = total;
+            }
+            __syncthreads();
+            if (kW == 1 && !live) return;
+            if (live) {
+                before = __reduce_add_sync(0xffffffffu, lane < kMergeWarps ? sums[0][lane] : 0u);
+                total = __reduce_add_sync(0xffffffffu, lane < kMergeWarps ? sums[1][lane] : 0u);
+                for (int i = b0; i < b; ++i) before += span_of(__ldg(p.ctx_lens + i));
+                find_flat(before, total, (uint32_t)(clamped_ctx(p, b) + kPage - 1) / kPage);
+            }
         }
-    };
-    if (hinted) find();
-    grid_dep_wait();
-    const int now = hinted && lane < p.batch ? __ldg(p.ctx_lens + lane) : 0;
-    if (!hinted) find();
-
+    }
     constexpr int kRows = 8;   // rows loaded per round before any is combined
     float M = -INFINITY, acc = 0.f, L = 0.f, Dn = 0.f, Db = 0.f, Vt = 0.f, Vm = 0.f;
-    for (bool again = hinted;; again = false) {
+    for (bool again = kHint;; again = false) {
         for (int s0 = sub; s0 < count; s0 += kRows * kW) {
             float ms[kRows], v[kRows], ls[kRows], ds[kRows], dbs[kRows], vts[kRows];
 #pragma unroll
@@ -1615,7 +1642,7 @@ __global__ void __launch_bounds__(32 * kMergeWarps, kW == 1 ? 4 : 3) merge_warp_
         }
         if (!again || !__any_sync(0xffffffffu, now != cx)) break;
         cx = now;
-        find();
+        find_hinted();
         M = -INFINITY;
         acc = L = Dn = Db = Vt = Vm = 0.f;
     }
@@ -1702,10 +1729,17 @@ static cudaError_t launch_merge(const DecodeParams& p, cudaStream_t stream) {
             const long per = kMergeWarps / w;
             return launch_pdl(kernel, dim3((unsigned)((items + per - 1) / per)), dim3(32 * kMergeWarps), 0, stream, p);
         };
-        if (p.pages_per_split == 0 && items * 8 <= room) return go(merge_warp_kernel<kX, 8>, 8);
-        if (p.pages_per_split == 0 && items * 4 <= room) return go(merge_warp_kernel<kX, 4>, 4);
-        if (p.pages_per_split == 0 && items * 2 <= room) return go(merge_warp_kernel<kX, 2>, 2);
-        return go(merge_warp_kernel<kX, 1>, 1);
+        const bool flat = p.pages_per_split == 0;
+        const int w = !flat ? 1 : items * 8 <= room ? 8 : items * 4 <= room ? 4 : items * 2 <= room ? 2 : 1;
+        if (flat && p.batch <= 32)
+            return w == 8   ? go(merge_warp_kernel<kX, 8, true>, 8)
+                   : w == 4 ? go(merge_warp_kernel<kX, 4, true>, 4)
+                   : w == 2 ? go(merge_warp_kernel<kX, 2, true>, 2)
+                            : go(merge_warp_kernel<kX, 1, true>, 1);
+        return w == 8   ? go(merge_warp_kernel<kX, 8, false>, 8)
+               : w == 4 ? go(merge_warp_kernel<kX, 4, false>, 4)
+               : w == 2 ? go(merge_warp_kernel<kX, 2, false>, 2)
+                        : go(merge_warp_kernel<kX, 1, false>, 1);
     }
     const dim3 grid(kHeadDim / 32, p.num_q_heads, p.batch);
     const long ctas = (long)grid.x * grid.y * grid.z;
