@@ -17,15 +17,16 @@
 // logarithmic scale, on which contributions spread), a count per bucket, their
 // prefix sums, and each key's rank inside its bucket by comparison with the bucket's
 // other keys (a handful).  A cell whose fullest bucket holds more than kMaxBucket keys
-// (equal contributions; a range stretched by inf or NaN) is sorted by a bitonic
-// network instead, whose keys stay in registers: exchanges within a thread and within a
-// warp need no shared memory, only those across warps go through it.  Both give the
-// same order, so the sums that follow are the same bits.  Measured, network -> buckets:
-// 784 cells of 2048 pages 57.8 -> 22.2 us (57,000 -> 17,300 warp instructions a cell; what
-// is left waits for barriers and shared memory), 2800 of 512 43.5 -> 16.6, 8400 of 100
-// 120 -> 12.7, 196 of 8192 97.8 -> 30.8.  Twice or four times the buckets: 22.3 and 28.2 us.
+// (many contributions that are zero or equal; a range stretched by inf or NaN) is sorted by
+// stable passes over 7-bit digits instead.  Both give the same order, so the sums that
+// follow are the same bits.
+// Measured, network of compare-exchanges (the only sort before) -> this: 784 cells of 2048
+// pages 58.6 -> 21.3 us, half of their contributions zero 58.7 -> 17.7, all equal 59.3 -> 19.5;
+// 2800 of 512 43.5 -> 18.5; 8400 of 100 119 -> 13.6; 196 of 8192 99 -> 36.  Twice or four times
+// the buckets at 784 x 2048: no faster.
 #include <climits>
 
+#include "dispatch.h"
 #include "wc_kernels.cuh"
 
 namespace wc {
@@ -36,31 +37,27 @@ namespace {
 // consecutive sorted positions, whatever the CTA's size: their order of additions, and
 // with it the count that a borderline tau gives, does not depend on how a table is sorted.
 constexpr int kSumThreads = 512, kSumWarps = kSumThreads / 32;
-// Keys of a bucket that its members are compared with: beyond it the network is faster
-// (a warp's ranking takes as many steps as its fullest bucket).
+// Keys of a bucket that its members are compared with: a warp's ranking takes as many
+// steps as its fullest bucket.
 constexpr int kMaxBucket = 64;
 
 __device__ __forceinline__ float key_value(unsigned long long key) { return __uint_as_float((uint32_t)(key >> 32)); }
 
-// Bitonic compare-exchange seen from element i, whose partner is i ^ j, in the
-// merge of size k: blocks with (i & k) == 0 sort descending (the lower index
-// keeps the larger key), the others ascending.  For j >= KPT and k > j every
-// position a thread holds has the same bits j and k, so one flag serves all.
-__device__ __forceinline__ bool bitonic_takes_max(int i, int j, int k) { return ((i & k) == 0) == ((i & j) == 0); }
-
-__device__ __forceinline__ unsigned long long pick(bool take_max, unsigned long long mine, unsigned long long other) {
-    return take_max ? (mine > other ? mine : other) : (mine < other ? mine : other);
-}
-
 // A CTA of T threads sorts K keys per thread; KS: positions per thread of the sums.
 // T grows with the table (K = 4 up to 4096 pages), so that a small cell costs few warps
 // and barriers: 2800 cells of 512 pages took 24.8 us with 512 threads, 16.2 with 256.
+// Threads per SM that the register budget leaves room for: all 2048 with one or two keys a
+// thread, 1536 with four (at most 40 registers: 2800 cells of 512 pages 18.5 us, without it 23.9),
+// 1024 with more.
+constexpr int min_ctas(int T, int K) {
+    const int n = (K <= 2 ? 2048 : K <= 4 ? 1536 : 1024) / T;
+    return n < 1 ? 1 : n > 32 ? 32 : n;
+}
 template <int T, int K, int KS>
-__global__ void __launch_bounds__(T) repair_select_kernel(const __grid_constant__ RepairParams p) {
+__global__ void __launch_bounds__(T, min_ctas(T, K)) repair_select_kernel(const __grid_constant__ RepairParams p) {
     constexpr int N = T * K;      // sorted length: the block table, padded to a power of two
-    constexpr int W = 32 * K;     // positions held by one warp
     constexpr int kSelWarps = T / 32;
-    extern __shared__ __align__(16) unsigned long long xs[];   // [N] keys; exchange buffer of the network
+    extern __shared__ __align__(16) unsigned long long xs[];   // [N] keys
     uint32_t* cnt = reinterpret_cast<uint32_t*>(xs + N);      // [N] keys per bucket, then the buckets' ends
     __shared__ uint32_t warp_lo[kSelWarps], warp_hi[kSelWarps], warp_sum[kSelWarps];
     __shared__ float warp_tot[kSumWarps];
@@ -84,18 +81,21 @@ __global__ void __launch_bounds__(T) repair_select_kernel(const __grid_constant_
     const int n = (ctx + kPage - 1) / kPage;
 
     // ---- C_j = d_j 2^(m_j - M) / L; thread t takes pages t, t + T, ... (any order does) --
+    // A page that contributes nothing is not sorted: nothing remains after the pages that
+    // do, so that with tau >= 0 the list ends before it.
+    const bool zeros = !(p.tau >= 0.f);   // every page is listed, these in page order behind the others
     unsigned long long key[K];
     auto page_of = [&](int r) { return tid + r * T; };
 #pragma unroll
     for (int r = 0; r < K; ++r) {
         const int j = page_of(r);
         const float2 t = j < p.max_pages ? terms[j] : make_float2(-INFINITY, 0.f);
-        key[r] = 0ull;   // padding: below every page (C = +0, index bits 0)
+        key[r] = 0ull;   // not sorted
         if (j < n) {
             float cj = (nm.y > 0.f && t.y != 0.f) ? __fdiv_rn(t.y * exp2f(t.x - nm.x), nm.y) : 0.f;
             if (cj <= 0.f) cj = 0.f;   // -0 ranks as +0; NaN stays and ranks first
             if (p.contrib) p.contrib[cell * p.max_pages + j] = cj;
-            key[r] = ((unsigned long long)__float_as_uint(cj) << 32) | (0xFFFFFFFFu - (uint32_t)j);
+            if (cj != 0.f || zeros) key[r] = ((unsigned long long)__float_as_uint(cj) << 32) | (0xFFFFFFFFu - (uint32_t)j);
         }
     }
 
@@ -107,16 +107,15 @@ __global__ void __launch_bounds__(T) repair_select_kernel(const __grid_constant_
     };
 
     // ---- descending sort into xs (kept cells: nothing is paged in, any order does) ------
-    bool network = false;
     if (!kept) {
-        uint32_t lo = 0xFFFFFFFFu, hi = 0u;   // range of the pages' contribution bits
+        uint32_t lo = 0xFFFFFFFFu, hi = 0u;   // the contributions' bits: least, largest finite
 #pragma unroll
         for (int r = 0; r < K; ++r) {
             cnt[page_of(r)] = 0u;
-            if (page_of(r) < n) {
+            if (key[r] != 0ull) {
                 const uint32_t bits = (uint32_t)(key[r] >> 32);
                 lo = min(lo, bits);
-                hi = max(hi, bits);
+                hi = max(hi, bits < 0x7F800000u ? bits : 0u);
             }
         }
         lo = __reduce_min_sync(0xffffffffu, lo);
@@ -126,17 +125,20 @@ __global__ void __launch_bounds__(T) repair_select_kernel(const __grid_constant_
             warp_hi[warp] = hi;
         }
         __syncthreads();
-#pragma unroll
-        for (int w = 0; w < kSelWarps; ++w) {
-            lo = min(lo, warp_lo[w]);
-            hi = max(hi, warp_hi[w]);
+        if (kSelWarps > 1) {   // lane w takes warp w's (kSelWarps is a power of two)
+            lo = __reduce_min_sync(0xffffffffu, warp_lo[lane % kSelWarps]);
+            hi = __reduce_max_sync(0xffffffffu, warp_hi[lane % kSelWarps]);
         }
-        // bucket 0 holds the largest keys; the shift is the least that gives N buckets
-        const int shift = max(0, 32 - __clz(n > 0 ? hi - lo : 0u) - (31 - __clz(N)));
-        auto bucket = [&](unsigned long long k) { return (hi - (uint32_t)(k >> 32)) >> shift; };
+        // bucket 0 holds the largest keys (inf and NaN with the largest finite ones); the shift
+        // is the least that gives N buckets
+        const int shift = max(0, 32 - __clz(hi > lo ? hi - lo : 0u) - (31 - __clz(N)));
+        auto bucket = [&](unsigned long long k) {
+            const uint32_t bits = (uint32_t)(k >> 32);
+            return bits < hi ? (hi - bits) >> shift : 0u;
+        };
 #pragma unroll
         for (int r = 0; r < K; ++r)
-            if (page_of(r) < n) atomicAdd(&cnt[bucket(key[r])], 1u);
+            if (key[r] != 0ull) atomicAdd(&cnt[bucket(key[r])], 1u);
         __syncthreads();
         uint32_t sum = 0u, most = 0u;   // exclusive prefix sums; thread t takes buckets [t K, t K + K)
 #pragma unroll
@@ -152,10 +154,11 @@ __global__ void __launch_bounds__(T) repair_select_kernel(const __grid_constant_
             if (lane >= o) inc += v;
         }
         if (lane == 31) warp_sum[warp] = inc;
-        network = __syncthreads_or(most > kMaxBucket);   // block-uniform
-        if (!network) {
-            uint32_t first = inc - sum;
-            for (int w = 0; w < warp; ++w) first += warp_sum[w];
+        const bool buckets = !__syncthreads_or(most > kMaxBucket);   // block-uniform
+        const uint32_t of_warp = lane < kSelWarps ? warp_sum[lane] : 0u;
+        uint32_t first = inc - sum + __reduce_add_sync(0xffffffffu, lane < warp ? of_warp : 0u);
+        const int n_sorted = (int)__reduce_add_sync(0xffffffffu, of_warp);
+        if (buckets) {
 #pragma unroll
             for (int r = 0; r < K; ++r) {
                 const uint32_t x = cnt[base + r];
@@ -165,13 +168,13 @@ __global__ void __launch_bounds__(T) repair_select_kernel(const __grid_constant_
             __syncthreads();
 #pragma unroll
             for (int r = 0; r < K; ++r)   // grouped by bucket; cnt then holds each bucket's end
-                if (page_of(r) < n) xs[atomicAdd(&cnt[bucket(key[r])], 1u)] = key[r];
+                if (key[r] != 0ull) xs[atomicAdd(&cnt[bucket(key[r])], 1u)] = key[r];
             __syncthreads();
             uint32_t rank[(K + 1) / 2];   // two to a word (positions below 16384)
 #pragma unroll
             for (int r = 0; r < K; ++r) {
                 uint32_t k = 0u;   // the bucket's first position plus its larger keys
-                if (page_of(r) < n) {
+                if (key[r] != 0ull) {
                     const uint32_t bk = bucket(key[r]), last = cnt[bk];
                     k = bk > 0 ? cnt[bk - 1] : 0u;
                     for (uint32_t i = k, e = last; i < e; ++i) k += xs[i] > key[r] ? 1u : 0u;
@@ -181,53 +184,95 @@ __global__ void __launch_bounds__(T) repair_select_kernel(const __grid_constant_
             }
             __syncthreads();
 #pragma unroll
-            for (int r = 0; r < K; ++r) {   // padding keeps its own places behind the pages
-                const int k = page_of(r) < n ? (int)((rank[r / 2] >> (16 * (r & 1))) & 0xFFFFu) : page_of(r);
-                xs[spot(k)] = key[r];
+            for (int r = 0; r < K; ++r) {
+                if (key[r] != 0ull) xs[spot((int)((rank[r / 2] >> (16 * (r & 1))) & 0xFFFFu))] = key[r];
+                if (page_of(r) >= n_sorted) xs[spot(page_of(r))] = 0ull;
             }
-        }
-    }
-    if (network) {
-        // exchange layout: position i at word i ^ sw(i / K), as in spot(); an exchange
-        // partner i ^ j (j >= 32 K) flips only bits >= 5 of the thread index, which sw
-        // does not read
-        const int sw = K >= 16 ? (tid & 15) : (((tid * K) >> 4) & (K - 1));
-        for (int k = 2; k <= N; k <<= 1) {
-            for (int j = k >> 1; j >= W; j >>= 1) {   // partner in another warp
-                const bool tm = bitonic_takes_max(base, j, k);
+        } else {
+            // Stable passes over the digits of top - bits, from the lowest: the keys start in
+            // page order, so equal contributions stay in it.  A warp holds 32 K consecutive
+            // positions; within a warp a key's place among its digit's keys is a count of lanes
+            // by ballots, across warps the prefix sums of the counts per (digit, warp).
+            constexpr int kDigit = K >= 4 ? 7 : K == 2 ? 6 : 5, kBins = 1 << kDigit;
+            constexpr int kPer = kBins / 32;   // counts per thread: kBins per warp
+            static_assert(kPer <= K, "the counts fit in cnt");
+            auto slot = [](int d, int w) { return d * kSelWarps + ((w + d) & (kSelWarps - 1)); };   // spreads the banks
+            auto place = [&](int r) { return (warp * K + r) * 32 + lane; };
+            uint32_t top = 0u;   // the largest, inf and NaN included
 #pragma unroll
-                for (int r = 0; r < K; ++r) xs[(base + r) ^ sw] = key[r];
+            for (int r = 0; r < K; ++r) {
+                top = max(top, (uint32_t)(key[r] >> 32));
+                xs[page_of(r)] = key[r];
+            }
+            top = __reduce_max_sync(0xffffffffu, top);
+            if (lane == 0) warp_hi[warp] = top;
+            __syncthreads();
+            top = __reduce_max_sync(0xffffffffu, warp_hi[lane % kSelWarps]);
+#pragma unroll
+            for (int r = 0; r < K; ++r) key[r] = xs[place(r)];
+            const int length = 32 - __clz(top - lo);
+            for (int d0 = 0; d0 == 0 || d0 < length; d0 += kDigit) {   // the first also moves the sorted to the front
+                auto digit = [&](int r) { return (int)(((top - (uint32_t)(key[r] >> 32)) >> d0) & (kBins - 1)); };
+                for (int i = tid; i < kBins * kSelWarps; i += T) cnt[i] = 0u;
                 __syncthreads();
+                uint32_t nth[(K + 1) / 2];   // two to a word
 #pragma unroll
-                for (int r = 0; r < K; ++r) key[r] = pick(tm, key[r], xs[((base + r) ^ j) ^ sw]);
-                __syncthreads();
-            }
-            for (int j = min(k >> 1, W >> 1); j >= K; j >>= 1) {   // partner in this warp
-                const bool tm = bitonic_takes_max(base, j, k);
-                const int lm = j / K;
+                for (int r = 0; r < K; ++r) {
+                    const bool valid = key[r] != 0ull;
+                    const int d = digit(r);
+                    uint32_t peers = __ballot_sync(0xffffffffu, valid);
 #pragma unroll
-                for (int r = 0; r < K; ++r) key[r] = pick(tm, key[r], __shfl_xor_sync(0xffffffffu, key[r], lm));
-            }
-#pragma unroll
-            for (int j = K >> 1; j > 0; j >>= 1) {   // partner in this thread
-                if (j <= (k >> 1)) {
-#pragma unroll
-                    for (int r = 0; r < K; ++r)
-                        if ((r & j) == 0) {
-                            const bool desc = ((base + r) & k) == 0;
-                            const unsigned long long a = key[r], c = key[r | j];
-                            if ((a < c) == desc) {
-                                key[r] = c;
-                                key[r | j] = a;
-                            }
-                        }
+                    for (int i = 0; i < kDigit; ++i) {
+                        const bool bit = (d >> i) & 1;
+                        const uint32_t set = __ballot_sync(0xffffffffu, bit);
+                        peers &= bit ? set : ~set;
+                    }
+                    uint32_t* c = cnt + slot(d, warp);
+                    const uint32_t k = valid ? *c + __popc(peers & ((1u << lane) - 1u)) : 0u;
+                    __syncwarp();
+                    if (valid && (peers >> lane) == 1u) *c = k + 1u;   // the last of the digit's lanes
+                    __syncwarp();
+                    if (r & 1) nth[r / 2] |= k << 16;
+                    else nth[r / 2] = k;
                 }
-            }
-        }
-    }
-    if (kept || network) {   // kept: page order, the order its sums have always had
+                __syncthreads();
+                uint32_t tot = 0u;   // thread t takes the counts [t kPer, t kPer + kPer) in (digit, warp) order
+                auto count = [&](int i) -> uint32_t& {
+                    const int e = tid * kPer + i;
+                    return cnt[slot(e / kSelWarps, e % kSelWarps)];
+                };
 #pragma unroll
-        for (int r = 0; r < K; ++r) xs[spot(kept ? page_of(r) : base + r)] = key[r];
+                for (int i = 0; i < kPer; ++i) tot += count(i);
+                uint32_t to = tot;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const uint32_t v = __shfl_up_sync(0xffffffffu, to, o);
+                    if (lane >= o) to += v;
+                }
+                if (lane == 31) warp_sum[warp] = to;
+                __syncthreads();
+                uint32_t start = to - tot + __reduce_add_sync(0xffffffffu, lane < warp ? warp_sum[lane] : 0u);
+#pragma unroll
+                for (int i = 0; i < kPer; ++i) {
+                    const uint32_t x = count(i);
+                    count(i) = start;
+                    start += x;
+                }
+                __syncthreads();
+#pragma unroll
+                for (int r = 0; r < K; ++r)
+                    if (key[r] != 0ull) xs[cnt[slot(digit(r), warp)] + ((nth[r / 2] >> (16 * (r & 1))) & 0xFFFFu)] = key[r];
+                __syncthreads();
+#pragma unroll
+                for (int r = 0; r < K; ++r) key[r] = place(r) < n_sorted ? xs[place(r)] : 0ull;
+            }
+            __syncthreads();
+#pragma unroll
+            for (int r = 0; r < K; ++r) xs[spot(place(r))] = key[r];
+        }
+    } else {   // page order, the order a kept cell's sums have always had
+#pragma unroll
+        for (int r = 0; r < K; ++r) xs[spot(page_of(r))] = key[r];
     }
     __syncthreads();
 
@@ -278,8 +323,7 @@ __global__ void __launch_bounds__(T) repair_select_kernel(const __grid_constant_
     cand = __reduce_min_sync(0xffffffffu, cand);
     if (lane == 0) warp_min[warp] = cand;
     __syncthreads();
-    int kmin = INT_MAX;
-    for (int w = 0; w < kSelWarps; ++w) kmin = min(kmin, warp_min[w]);
+    const int kmin = __reduce_min_sync(0xffffffffu, warp_min[lane % kSelWarps]);
     const int kstar = kept ? 0 : min(kmin, n);   // every page when no prefix is enough
     if (kstar >= n) {
         if (tid == 0) r_at_k = 0.f;
@@ -327,13 +371,23 @@ cudaError_t launch_select(const RepairParams& p, cudaStream_t stream) {
 cudaError_t launch_repair_select(const RepairParams& p, cudaStream_t stream) {
     static_assert(kRepairMaxPages == 16 * 1024, "the largest instance holds 16 keys per thread");
     if (p.batch == 0) return cudaSuccess;
-    // the least power of two that holds the table; KS = keys per thread of 512
-    if (p.max_pages <= 128) return launch_select<32, 4, 1>(p, stream);
-    if (p.max_pages <= 256) return launch_select<64, 4, 1>(p, stream);
-    if (p.max_pages <= 512) return launch_select<128, 4, 1>(p, stream);
-    if (p.max_pages <= 1024) return launch_select<256, 4, 2>(p, stream);
+    // the least power of two that holds the table; KS = positions per thread of 512
+    const int64_t cells = (int64_t)p.batch * p.num_q_heads;
+    if (p.max_pages <= 32) return launch_select<32, 1, 1>(p, stream);
+    if (p.max_pages <= 64)
+        return repair_wide(cells, 64) ? launch_select<64, 1, 1>(p, stream) : launch_select<32, 2, 1>(p, stream);
+    if (p.max_pages <= 128)
+        return repair_wide(cells, 128) ? launch_select<128, 1, 1>(p, stream) : launch_select<64, 2, 1>(p, stream);
+    if (p.max_pages <= 256)
+        return repair_wide(cells, 256)  ? launch_select<256, 1, 1>(p, stream)
+               : repair_wide(cells, 64) ? launch_select<128, 2, 1>(p, stream) : launch_select<64, 4, 1>(p, stream);
+    if (p.max_pages <= 512)
+        return repair_wide(cells, 256) ? launch_select<256, 2, 1>(p, stream) : launch_select<128, 4, 1>(p, stream);
+    if (p.max_pages <= 1024)
+        return repair_wide(cells, 512) ? launch_select<512, 2, 2>(p, stream) : launch_select<256, 4, 2>(p, stream);
     if (p.max_pages <= 2048) return launch_select<512, 4, 4>(p, stream);
-    if (p.max_pages <= 4096) return launch_select<1024, 4, 8>(p, stream);
+    if (p.max_pages <= 4096)
+        return repair_wide(cells, 1024) ? launch_select<1024, 4, 8>(p, stream) : launch_select<512, 8, 8>(p, stream);
     if (p.max_pages <= 8192) return launch_select<1024, 8, 16>(p, stream);
     return launch_select<1024, 16, 32>(p, stream);
 }
