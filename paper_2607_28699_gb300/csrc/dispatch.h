@@ -8,6 +8,24 @@
 
 namespace wc {
 
+// ---- write: one or two tasks (rows of 4 units) per warp -------------------------------------
+// From this many tokens on the grid runs per KV head.
+constexpr int kPerHeadMinTokens = 16;
+
+// Two: the K and the V rows of the same units in one warp.  The grouped row routine is the
+// longest: until its two-task CTAs fill the SMs (6 x 152 of 16 units), one task per warp is
+// done sooner (tokens x 8 heads, us one / two tasks: 100 3.8 / 4.5, 600 5.2 / 6.7, 1200 6.8 /
+// 8.5).  With the 10-bit dither's two Philox calls a row it is while the one-task CTAs fit the
+// SMs at once (7 x 152 of 8 units; one / two tasks, several writes in a row: 64 2.9 / 3.5, 512
+// 3.9 / 5.4, 1000 4.6 / 6.2; a write by itself: 1000 6.3 / 7.0, 1500 8.1 / 7.6).
+constexpr int64_t kGroupedTwoTaskUnits = 16384, kTenBitTwoTaskUnits = 7 * 152 * 8 + 1;
+constexpr bool write_two_tasks(int scheme, int bits, int64_t n_tok, int64_t num_kv_heads) {
+    return n_tok >= kPerHeadMinTokens &&
+           (scheme == WC_SCHEME_DITHER_INT8_G32             ? n_tok * num_kv_heads >= kGroupedTwoTaskUnits
+            : scheme == WC_SCHEME_DITHER_INT8 && bits == 10 ? n_tok * num_kv_heads >= kTenBitTwoTaskUnits
+                                                            : true);
+}
+
 // ---- repair selection: threads per cell -----------------------------------------------------
 // A wide CTA has fewer positions a thread and ends sooner, a narrow one needs fewer warps and
 // barriers per cell; the wide one wins while the cells' threads take at most half of the

@@ -20,6 +20,7 @@
 // 128-byte shared row per unit, so quantization runs in channel order.
 #include <cooperative_groups.h>
 
+#include "dispatch.h"
 #include "write_row.cuh"
 
 namespace cg = cooperative_groups;
@@ -36,11 +37,6 @@ namespace {
 // and heads against K and V rows in separate warps (us): 8-bit dither 31.1 -> 26.4, 10-bit
 // 39.7 -> 36.3, fp8 18.1 -> 15.7, grouped 50.1 -> 44.9 (55.4 before its packed pass).
 constexpr int write_units_per_cta(int tasks) { return 2 * 4 * tasks; }
-// The grouped row routine is the longest: until its two-task CTAs fill the SMs (6 x 152 of
-// 16 units), one task per warp is done sooner (tokens x 8 heads, us one / two tasks: 100
-// 3.8 / 4.5, 600 5.2 / 6.7, 1200 6.8 / 8.5).
-constexpr int kGroupedTwoTaskUnits = 16384;
-constexpr int kPerHeadMinTokens = 16;                     // per-head grid from this many tokens on
 
 // Two ways of cutting the units (token, KV head) into 4-unit tasks:
 //  kPerHead: grid (token groups, Hkv), a task = 4 consecutive tokens of one
@@ -51,13 +47,15 @@ constexpr int kPerHeadMinTokens = 16;                     // per-head grid from 
 //            (decode steps, where every SM the next decode needs counts).
 // Resident CTAs per SM the register budget is sized for, the best of 5 .. 9 in each case
 // (us at 32768 x 4): 8-bit dither seven at 72 registers 26.9 (six 28.5, eight 28.2, with
-// 36 bytes of spill), 10-bit six 35.7 (seven 36.3), grouped six 44.9 (seven 44.1 with 84
-// bytes of spill, which costs the 2047 x 8 write 10%), fp8 eight 15.3 (ten 15.7).
-__host__ __device__ constexpr int write_min_blocks(int scheme, int bits) {
-    return scheme == WC_SCHEME_FP8_E4M3 ? 8 : scheme == WC_SCHEME_DITHER_INT8_G32 || bits == 10 ? 6 : 7;
+// 36 bytes of spill), 10-bit six 35.7 (seven 36.5), grouped six 44.3 with 56 bytes of spill
+// (seven 44.1 with 84, which costs the 2047 x 8 write 10%), fp8 eight 15.3 (ten 15.7).  One
+// task per warp: seven, so that the small writes that take it are one wave (1000 x 8: grouped
+// 5.6, six 6.3).
+__host__ __device__ constexpr int write_min_blocks(int scheme, int bits, int tasks) {
+    return scheme == WC_SCHEME_FP8_E4M3 ? 8 : tasks == 2 && (scheme == WC_SCHEME_DITHER_INT8_G32 || bits == 10) ? 6 : 7;
 }
 template <int kScheme, int kBits, bool kPerHead, int kTasks>
-__global__ void __launch_bounds__(128, write_min_blocks(kScheme, kBits)) write_kernel(const __grid_constant__ WriteParams p) {
+__global__ void __launch_bounds__(128, write_min_blocks(kScheme, kBits, kTasks)) write_kernel(const __grid_constant__ WriteParams p) {
     constexpr bool kGrouped = kScheme == WC_SCHEME_DITHER_INT8_G32;
     __shared__ __align__(16) uint8_t xrows[kGrouped ? 4 * 4 * kXRowStride : 16];   // [warp][unit][row]
     __shared__ BypassTable btab;
@@ -303,15 +301,16 @@ cudaError_t launch_write(const WriteParams& p, int scheme, int bits, cudaStream_
     if (p.n_tok == 0) return cudaSuccess;
     static bool configured = false;   // same carveout as the decode kernels: no L1/shared reconfiguration
     if (!configured) {
-        const void* fns[9] = {(const void*)write_kernel<WC_SCHEME_FP8_E4M3, 8, false, 1>,
-                              (const void*)write_kernel<WC_SCHEME_DITHER_INT8, 8, false, 1>,
-                              (const void*)write_kernel<WC_SCHEME_DITHER_INT8, 10, false, 1>,
-                              (const void*)write_kernel<WC_SCHEME_DITHER_INT8_G32, 8, false, 1>,
-                              (const void*)write_kernel<WC_SCHEME_FP8_E4M3, 8, true, 2>,
-                              (const void*)write_kernel<WC_SCHEME_DITHER_INT8, 8, true, 2>,
-                              (const void*)write_kernel<WC_SCHEME_DITHER_INT8, 10, true, 2>,
-                              (const void*)write_kernel<WC_SCHEME_DITHER_INT8_G32, 8, true, 1>,
-                              (const void*)write_kernel<WC_SCHEME_DITHER_INT8_G32, 8, true, 2>};
+        const void* fns[10] = {(const void*)write_kernel<WC_SCHEME_FP8_E4M3, 8, false, 1>,
+                               (const void*)write_kernel<WC_SCHEME_DITHER_INT8, 8, false, 1>,
+                               (const void*)write_kernel<WC_SCHEME_DITHER_INT8, 10, false, 1>,
+                               (const void*)write_kernel<WC_SCHEME_DITHER_INT8_G32, 8, false, 1>,
+                               (const void*)write_kernel<WC_SCHEME_FP8_E4M3, 8, true, 2>,
+                               (const void*)write_kernel<WC_SCHEME_DITHER_INT8, 8, true, 2>,
+                               (const void*)write_kernel<WC_SCHEME_DITHER_INT8, 10, true, 1>,
+                               (const void*)write_kernel<WC_SCHEME_DITHER_INT8, 10, true, 2>,
+                               (const void*)write_kernel<WC_SCHEME_DITHER_INT8_G32, 8, true, 1>,
+                               (const void*)write_kernel<WC_SCHEME_DITHER_INT8_G32, 8, true, 2>};
         for (const void* f : fns) {
             cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout,
                                                  (int)cudaSharedmemCarveoutMaxShared);
@@ -320,23 +319,23 @@ cudaError_t launch_write(const WriteParams& p, int scheme, int bits, cudaStream_
         configured = true;
     }
     const bool per_head = p.n_tok >= kPerHeadMinTokens;
-    const bool grouped = scheme == WC_SCHEME_DITHER_INT8_G32;
-    const bool two = per_head && (!grouped || (int64_t)p.n_tok * p.num_kv_heads >= kGroupedTwoTaskUnits);
+    const bool two = write_two_tasks(scheme, bits, p.n_tok, p.num_kv_heads);
     const int upc = write_units_per_cta(two ? 2 : 1);
     const dim3 grid = per_head ? dim3((p.n_tok + upc - 1) / upc, p.num_kv_heads)
                                : dim3((p.n_tok * p.num_kv_heads + upc - 1) / upc);
     auto go = [&](auto kernel) { return launch_pdl(kernel, grid, dim3(128), 0, stream, p); };
     if (scheme == WC_SCHEME_FP8_E4M3)
         return two ? go(write_kernel<WC_SCHEME_FP8_E4M3, 8, true, 2>) : go(write_kernel<WC_SCHEME_FP8_E4M3, 8, false, 1>);
-    if (grouped)
+    if (scheme == WC_SCHEME_DITHER_INT8_G32)
         return two        ? go(write_kernel<WC_SCHEME_DITHER_INT8_G32, 8, true, 2>)
                : per_head ? go(write_kernel<WC_SCHEME_DITHER_INT8_G32, 8, true, 1>)
                           : go(write_kernel<WC_SCHEME_DITHER_INT8_G32, 8, false, 1>);
     if (bits == 8)
         return two ? go(write_kernel<WC_SCHEME_DITHER_INT8, 8, true, 2>)
                    : go(write_kernel<WC_SCHEME_DITHER_INT8, 8, false, 1>);
-    return two ? go(write_kernel<WC_SCHEME_DITHER_INT8, 10, true, 2>)
-               : go(write_kernel<WC_SCHEME_DITHER_INT8, 10, false, 1>);
+    return two        ? go(write_kernel<WC_SCHEME_DITHER_INT8, 10, true, 2>)
+           : per_head ? go(write_kernel<WC_SCHEME_DITHER_INT8, 10, true, 1>)
+                      : go(write_kernel<WC_SCHEME_DITHER_INT8, 10, false, 1>);
 }
 
 }  // namespace wc

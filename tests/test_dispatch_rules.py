@@ -13,6 +13,7 @@ SOURCE = r"""
 #include "dispatch.h"
 extern "C" {
 int repair_wide(long cells, int threads) { return wc::repair_wide(cells, threads); }
+int write_two_tasks(int scheme, int bits, long n_tok, long heads) { return wc::write_two_tasks(scheme, bits, n_tok, heads); }
 }
 """
 
@@ -31,3 +32,12 @@ def lib(tmp_path_factory):
 def test_repair_ctas_are_wide_while_the_chip_is_half_full(lib, cells, threads, wide):
     """One warp per small cell left a few cells with long chains: 28 of 128 pages took 7.5 us, 4.8 before."""
     assert lib.repair_wide(ctypes.c_long(cells), threads) == wide
+
+
+@pytest.mark.parametrize("scheme,bits,n_tok,heads,two", [
+    (0, 8, 15, 8, 0), (0, 8, 16, 8, 1), (1, 8, 16, 1, 1),
+    (0, 10, 15, 64, 0), (0, 10, 700, 8, 0), (0, 10, 1064, 8, 0), (0, 10, 1065, 8, 1), (0, 10, 8512, 1, 0), (0, 10, 32768, 4, 1),
+    (2, 8, 2047, 8, 0), (2, 8, 2048, 8, 1), (2, 8, 131072, 1, 1)])
+def test_write_tasks(lib, scheme, bits, n_tok, heads, two):
+    """700 x 8 tokens and heads at 10 bits: 5.8 us with two tasks, 4.6 with one."""
+    assert lib.write_two_tasks(scheme, bits, ctypes.c_long(n_tok), ctypes.c_long(heads)) == two
