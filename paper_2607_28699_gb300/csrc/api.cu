@@ -529,6 +529,18 @@ CtxGetCurrentFn ctx_get_current() {
     return fn;
 }
 
+}  // namespace
+
+cudaError_t wc::current_context(int* device, void** context) {
+    *context = nullptr;
+    const cudaError_t e = cudaGetDevice(device);
+    if (e != cudaSuccess) return e;
+    if (CtxGetCurrentFn get = ctx_get_current()) (void)get(context);
+    return cudaSuccess;
+}
+
+namespace {
+
 std::mutex g_noalloc_mu;
 void* g_noalloc_ptr[kNoAllocMaxDevices] = {};
 void* g_noalloc_ctx[kNoAllocMaxDevices] = {};

@@ -671,15 +671,8 @@ __global__ void __launch_bounds__(kGwThreads, 1) decode_g32_ws_kernel(const __gr
 
 template <int kX>
 cudaError_t launch_g32_ws(const DecodeParams& p, cudaStream_t stream) {
-    static bool configured = false;   // per process; the attributes are per function
-    if (!configured) {
-        cudaError_t e = cudaFuncSetAttribute(decode_g32_ws_kernel<kX>, cudaFuncAttributeMaxDynamicSharedMemorySize, kGwSmemFlat);
-        if (e != cudaSuccess) return e;
-        e = cudaFuncSetAttribute(decode_g32_ws_kernel<kX>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                 (int)cudaSharedmemCarveoutMaxShared);
-        if (e != cudaSuccess) return e;
-        configured = true;
-    }
+    static PerDevice<Configured, cudaError_t> configured;
+    if (cudaError_t e = configure(configured, decode_g32_ws_kernel<kX>, kGwSmemFlat)) return e;
     G32Params gp;
     gp.p = p;
     if (!encode_page_map(&gp.k_map, p.k_codes, p.num_pages, p.num_kv_heads) ||

@@ -1710,18 +1710,20 @@ __global__ void __launch_bounds__(32 * kMergeWarps, kW == 1 ? 4 : 3) merge_warp_
 
 template <int kX>
 static cudaError_t launch_merge(const DecodeParams& p, cudaStream_t stream) {
-    static std::once_flag once;
-    static int num_sms = 0;   // 0: the spread request is not used
-    std::call_once(once, [] {
+    static PerDevice<int, cudaError_t> state;
+    int num_sms = 0;   // 0: the spread request is not used
+    (void)per_device(state, num_sms, [](int& sms) {
         int dev = 0, n = 0;
+        sms = 0;
         if (cudaGetDevice(&dev) == cudaSuccess &&
             cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess &&
             cudaFuncSetAttribute(merge_kernel<kX>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMergeSpreadSmem) ==
                 cudaSuccess)
-            num_sms = n;
+            sms = n;
         (void)cudaFuncSetAttribute(merge_kernel<kX>, cudaFuncAttributePreferredSharedMemoryCarveout,
                                    (int)cudaSharedmemCarveoutMaxShared);
         (void)cudaGetLastError();   // a refused hint leaves no sticky error behind
+        return cudaSuccess;
     });
     if (p.pages_per_split == 0 || p.splits <= kWarpMergeSplits) {   // a few partials per unit
         const long items = (long)p.batch * p.num_q_heads * (kHeadDim / 32), room = 24L * num_sms;
@@ -1755,17 +1757,8 @@ cudaError_t launch_merge_x(const DecodeParams& p, int x, cudaStream_t stream) {
 
 template <int kX>
 static cudaError_t launch_fp8(const DecodeParams& p, cudaStream_t stream) {
-    static bool configured = false;   // per process; the attributes are per function
-    if (!configured) {
-        cudaError_t e = cudaFuncSetAttribute(decode_kernel<kX>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
-        if (e != cudaSuccess) return e;
-        // the library's kernels all prefer the largest shared-memory carveout,
-        // so consecutive launches do not reconfigure the L1 / shared split
-        e = cudaFuncSetAttribute(decode_kernel<kX>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                 (int)cudaSharedmemCarveoutMaxShared);
-        if (e != cudaSuccess) return e;
-        configured = true;
-    }
+    static PerDevice<Configured, cudaError_t> configured;
+    if (cudaError_t e = configure(configured, decode_kernel<kX>, kSmemBytes)) return e;
     DkParams dp;
     dp.p = p;
     if (!encode_page_map(&dp.k_map, p.k_codes, p.num_pages, p.num_kv_heads) ||
@@ -1813,16 +1806,8 @@ bool encode_page_map(CUtensorMap* map, const void* codes, int num_pages, int num
 template <int kBits, int kX>
 static cudaError_t launch_ws(const DecodeParams& p, cudaStream_t stream) {
     constexpr int kSmem = WsSmem<kBits, (kX & kXFlat) != 0>::kBytes;
-    static bool configured = false;
-    if (!configured) {
-        cudaError_t e = cudaFuncSetAttribute(decode_ws_kernel<kBits, kX>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             kSmem);
-        if (e != cudaSuccess) return e;
-        e = cudaFuncSetAttribute(decode_ws_kernel<kBits, kX>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                 (int)cudaSharedmemCarveoutMaxShared);
-        if (e != cudaSuccess) return e;
-        configured = true;
-    }
+    static PerDevice<Configured, cudaError_t> configured;
+    if (cudaError_t e = configure(configured, decode_ws_kernel<kBits, kX>, kSmem)) return e;
     WsParams wp;
     wp.p = p;
     if constexpr ((kX & kXAppend) != 0) {   // the cache as the write path sees it

@@ -85,13 +85,8 @@ __global__ void __launch_bounds__(kGateThreads) gate_kernel(const float* __restr
 cudaError_t launch_gate(const float* meter_raw, const float* value_term, const float* v_max, int n_cells, int group,
                         float tau, float tau_v, uint8_t* keep_q, uint8_t* keep_kv, int32_t* n_kept,
                         cudaStream_t stream) {
-    static bool configured = false;   // same carveout as the decode kernels
-    if (!configured) {
-        cudaError_t e = cudaFuncSetAttribute(gate_kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                             (int)cudaSharedmemCarveoutMaxShared);
-        if (e != cudaSuccess) return e;
-        configured = true;
-    }
+    static PerDevice<Configured, cudaError_t> configured;
+    if (cudaError_t e = configure(configured, gate_kernel, 0)) return e;
     // a programmatic dependent of the preceding kernel (the decode's merge): its CTA
     // becomes resident while that grid drains and waits for it (griddepcontrol.wait)
     cudaLaunchConfig_t cfg = {};

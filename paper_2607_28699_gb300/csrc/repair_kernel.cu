@@ -351,17 +351,9 @@ __global__ void __launch_bounds__(T, min_ctas(T, K)) repair_select_kernel(const 
 
 template <int T, int K, int KS>
 cudaError_t launch_select(const RepairParams& p, cudaStream_t stream) {
-    static bool configured = false;
     constexpr size_t smem = (size_t)T * K * (sizeof(unsigned long long) + sizeof(uint32_t));
-    if (!configured) {
-        cudaError_t e = cudaFuncSetAttribute(repair_select_kernel<T, K, KS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)smem);
-        if (e != cudaSuccess) return e;
-        e = cudaFuncSetAttribute(repair_select_kernel<T, K, KS>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                 (int)cudaSharedmemCarveoutMaxShared);
-        if (e != cudaSuccess) return e;
-        configured = true;
-    }
+    static PerDevice<Configured, cudaError_t> configured;
+    if (cudaError_t e = configure(configured, repair_select_kernel<T, K, KS>, smem)) return e;
     repair_select_kernel<T, K, KS><<<dim3(p.num_q_heads, p.batch), T, smem, stream>>>(p);
     return cudaGetLastError();
 }

@@ -3,6 +3,7 @@
 
 #include <cuda_runtime.h>
 
+#include "per_device.h"
 #include "wc_common.cuh"
 
 namespace wc {
@@ -94,6 +95,34 @@ struct DecodePlan {
 // not fit and calls with that size have always been accepted); SIZE_MAX: the preferred plan.
 DecodePlan plan_decode(int batch, int num_kv_heads, int max_pages, int num_sms, int scheme, int bits,
                        size_t available = SIZE_MAX);
+
+// The current device and its context (null until the runtime has made one current here).
+cudaError_t current_context(int* device, void** context);
+
+// What make(value) sets up for the current device context, once for each (per_device.h).
+template <typename T, typename Make>
+inline cudaError_t per_device(PerDevice<T, cudaError_t>& state, T& value, Make make) {
+    int device = 0;
+    void* context = nullptr;
+    if (cudaError_t e = current_context(&device, &context)) return e;
+    return state.get(device, context, value, make);
+}
+
+// The attributes of a kernel's launches: its dynamic shared memory (0: not raised), and the
+// largest shared-memory carveout, which all the library's kernels prefer, so that consecutive
+// launches do not reconfigure the L1 / shared split.
+struct Configured {};
+template <typename Kernel>
+inline cudaError_t configure(PerDevice<Configured, cudaError_t>& state, Kernel* kernel, size_t smem) {
+    Configured c;
+    return per_device(state, c, [&](Configured&) {
+        cudaError_t e = smem > 0 ? cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)
+                                 : cudaSuccess;
+        if (e != cudaSuccess) return e;
+        return cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                    (int)cudaSharedmemCarveoutMaxShared);
+    });
+}
 
 // Launch `kernel` on `stream` as a programmatic dependent of the preceding work.
 template <typename Kernel, typename Params>

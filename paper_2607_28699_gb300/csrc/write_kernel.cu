@@ -264,13 +264,15 @@ __global__ void __launch_bounds__(kWide ? 256 : 1024)
 template <bool kWide>
 static cudaError_t launch_pairs(const __half* k, int n_tok, int num_kv_heads, int rope_layout, int m, int32_t* pairs,
                                 cudaStream_t stream) {
-    static bool configured = false;   // per process; the attribute is per function
-    if (!configured && kWide) {       // above the portable cluster size
-        cudaError_t e = cudaFuncSetAttribute(select_pairs_kernel<kWide>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-        if (e != cudaSuccess) return e;
-        e = cudaFuncSetAttribute(select_pairs_kernel<kWide>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSelPairRing * 256 * 16);
-        if (e != cudaSuccess) return e;
-        configured = true;
+    if (kWide) {   // above the portable cluster size
+        static PerDevice<Configured, cudaError_t> configured;
+        Configured c;
+        const cudaError_t set = per_device(configured, c, [](Configured&) {
+            cudaError_t e = cudaFuncSetAttribute(select_pairs_kernel<kWide>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+            if (e != cudaSuccess) return e;
+            return cudaFuncSetAttribute(select_pairs_kernel<kWide>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSelPairRing * 256 * 16);
+        });
+        if (set != cudaSuccess) return set;
     }
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(kWide ? 16 : 8, num_kv_heads);
@@ -299,8 +301,9 @@ cudaError_t launch_select_pairs(const __half* k, int n_tok, int num_kv_heads, in
 
 cudaError_t launch_write(const WriteParams& p, int scheme, int bits, cudaStream_t stream) {
     if (p.n_tok == 0) return cudaSuccess;
-    static bool configured = false;   // same carveout as the decode kernels: no L1/shared reconfiguration
-    if (!configured) {
+    static PerDevice<Configured, cudaError_t> configured;   // same carveout as the decode kernels: no L1/shared reconfiguration
+    Configured c;
+    const cudaError_t set = per_device(configured, c, [](Configured&) {
         const void* fns[10] = {(const void*)write_kernel<WC_SCHEME_FP8_E4M3, 8, false, 1>,
                                (const void*)write_kernel<WC_SCHEME_DITHER_INT8, 8, false, 1>,
                                (const void*)write_kernel<WC_SCHEME_DITHER_INT8, 10, false, 1>,
@@ -316,8 +319,9 @@ cudaError_t launch_write(const WriteParams& p, int scheme, int bits, cudaStream_
                                                  (int)cudaSharedmemCarveoutMaxShared);
             if (e != cudaSuccess) return e;
         }
-        configured = true;
-    }
+        return cudaSuccess;
+    });
+    if (set != cudaSuccess) return set;
     const bool per_head = p.n_tok >= kPerHeadMinTokens;
     const bool two = write_two_tasks(scheme, bits, p.n_tok, p.num_kv_heads);
     const int upc = write_units_per_cta(two ? 2 : 1);
