@@ -263,17 +263,7 @@ __global__ void __launch_bounds__(kWide ? 256 : 1024)
 
 template <bool kWide>
 static cudaError_t launch_pairs(const __half* k, int n_tok, int num_kv_heads, int rope_layout, int m, int32_t* pairs,
-                                cudaStream_t stream) {
-    if (kWide) {   // above the portable cluster size
-        static PerDevice<Configured, cudaError_t> configured;
-        Configured c;
-        const cudaError_t set = per_device(configured, c, [](Configured&) {
-            cudaError_t e = cudaFuncSetAttribute(select_pairs_kernel<kWide>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-            if (e != cudaSuccess) return e;
-            return cudaFuncSetAttribute(select_pairs_kernel<kWide>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSelPairRing * 256 * 16);
-        });
-        if (set != cudaSuccess) return set;
-    }
+                                cudaStream_t stream, int* resident = nullptr) {   // resident: asked instead of a launch
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(kWide ? 16 : 8, num_kv_heads);
     cfg.blockDim = dim3(kWide ? 256 : 1024);
@@ -285,16 +275,32 @@ static cudaError_t launch_pairs(const __half* k, int n_tok, int num_kv_heads, in
     attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
+    if (resident) return cudaOccupancyMaxActiveClusters(resident, select_pairs_kernel<kWide>, &cfg);
     return cudaLaunchKernelEx(&cfg, select_pairs_kernel<kWide>, k, n_tok, num_kv_heads, rope_layout, m, pairs);
+}
+
+// Wide clusters resident at once on the current device; 0 where they cannot be launched.
+static int wide_pair_clusters() {
+    static PerDevice<int, cudaError_t> state;
+    int n = 0;
+    const cudaError_t known = per_device(state, n, [](int& clusters) {
+        auto kernel = select_pairs_kernel<true>;
+        clusters = 0;
+        if (cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||   // above 8
+            cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSelPairRing * 256 * 16) != cudaSuccess ||
+            launch_pairs<true>(nullptr, 0, 1, WC_ROPE_HALF, 0, nullptr, nullptr, &clusters) != cudaSuccess) {
+            clusters = 0;
+            (void)cudaGetLastError();   // the narrow cluster serves instead
+        }
+        return cudaSuccess;
+    });
+    return known == cudaSuccess ? n : 0;
 }
 
 cudaError_t launch_select_pairs(const __half* k, int n_tok, int num_kv_heads, int rope_layout, int m, int32_t* pairs,
                                 cudaStream_t stream) {
-    // The wide cluster's copies are 16 bytes; a k that is only 8-byte aligned stays on the
-    // narrow one.  4 heads, us narrow / wide: 1024 rows 3.8 / 4.6, 2048 4.5 / 4.6, 4096
-    // 4.8 / 4.4, 8192 6.3 / 5.3, 32768 15.2 / 9.3.
-    constexpr int kWideRows = 4096;
-    const bool wide = n_tok >= kWideRows && ((uintptr_t)k & 15) == 0;
+    const bool wide = pairs_wide(n_tok, ((uintptr_t)k & 15) == 0, num_kv_heads,
+                                 n_tok >= kWidePairRows ? wide_pair_clusters() : 0);
     return wide ? launch_pairs<true>(k, n_tok, num_kv_heads, rope_layout, m, pairs, stream)
                 : launch_pairs<false>(k, n_tok, num_kv_heads, rope_layout, m, pairs, stream);
 }

@@ -14,6 +14,7 @@ SOURCE = r"""
 extern "C" {
 int repair_wide(long cells, int threads) { return wc::repair_wide(cells, threads); }
 int write_two_tasks(int scheme, int bits, long n_tok, long heads) { return wc::write_two_tasks(scheme, bits, n_tok, heads); }
+int pairs_wide(int n_tok, int aligned, int heads, int resident) { return wc::pairs_wide(n_tok, aligned != 0, heads, resident); }
 }
 """
 
@@ -41,3 +42,11 @@ def test_repair_ctas_are_wide_while_the_chip_is_half_full(lib, cells, threads, w
 def test_write_tasks(lib, scheme, bits, n_tok, heads, two):
     """700 x 8 tokens and heads at 10 bits: 5.8 us with two tasks, 4.6 with one."""
     assert lib.write_two_tasks(scheme, bits, ctypes.c_long(n_tok), ctypes.c_long(heads)) == two
+
+
+@pytest.mark.parametrize("n_tok,aligned,heads,resident,wide", [
+    (4095, 1, 4, 14, 0), (4096, 1, 4, 14, 1), (4096, 0, 4, 14, 0), (4096, 1, 14, 14, 1), (4096, 1, 15, 14, 0),
+    (65536, 1, 32, 14, 0),                     # more clusters than fit at once: 93 us, 80 narrow
+    (65536, 1, 1, 0, 0), (65536, 1, 8, 4, 0)])   # a device that cannot place them: the narrow cluster serves
+def test_pair_clusters_are_wide_while_resident(lib, n_tok, aligned, heads, resident, wide):
+    assert lib.pairs_wide(n_tok, aligned, heads, resident) == wide
