@@ -197,7 +197,9 @@ size_t wc_workspace_size(const wc_cache_desc* desc, int32_t batch, int32_t max_p
         fail(WC_ERR_CUDA, "no current CUDA device to size the workspace for");
         return 0;
     }
-    return wc::plan_decode(batch, desc->num_kv_heads, max_pages, sms, desc->scheme, desc->dither_bits).total;
+    return wc::plan_decode(batch, desc->num_kv_heads, max_pages, sms, desc->scheme, desc->dither_bits,
+                           desc->num_q_heads / desc->num_kv_heads, false)
+        .total;
 }
 
 // Metered decode with a caller workspace; meter_b != NULL also asks for the
@@ -266,7 +268,8 @@ static wc_status decode_with_workspace(const wc_cache_desc* desc, int32_t layer,
     int sms = 0;
     if (current_sm_count(&sms) != 0) return fail(WC_ERR_CUDA, "cannot query the current device");
     const wc::DecodePlan pl =
-        wc::plan_decode(batch, desc->num_kv_heads, max_pages, sms, desc->scheme, desc->dither_bits, workspace_bytes);
+        wc::plan_decode(batch, desc->num_kv_heads, max_pages, sms, desc->scheme, desc->dither_bits,
+                        desc->num_q_heads / desc->num_kv_heads, k_new != nullptr, workspace_bytes);
     if (workspace_bytes < pl.total)
         return fail(WC_ERR_WORKSPACE, "workspace has %zu bytes, needs %zu", workspace_bytes, pl.total);
     uint8_t* ws = static_cast<uint8_t*>(workspace);
@@ -588,7 +591,8 @@ extern "C" wc_status wc_metered_decode_attention_noalloc(
     int sms = 0;
     if (current_sm_count(&sms) != 0) return fail(WC_ERR_CUDA, "cannot query the current device");
     const wc::DecodePlan pl =
-        wc::plan_decode(batch, desc->num_kv_heads, max_pages, sms, desc->scheme, desc->dither_bits, kNoAllocScratchBytes);
+        wc::plan_decode(batch, desc->num_kv_heads, max_pages, sms, desc->scheme, desc->dither_bits,
+                        desc->num_q_heads / desc->num_kv_heads, false, kNoAllocScratchBytes);
     if (pl.total > kNoAllocScratchBytes)
         return fail(WC_ERR_UNSUPPORTED,
                     "this decode needs %zu bytes of scratch but the built-in scratch holds %zu; "

@@ -1401,93 +1401,6 @@ __global__ void __launch_bounds__(32 * kMergeWarps) merge_kernel(const __grid_co
 
 }  // namespace
 
-// Resident decode CTAs per SM: the dithered kernels take a whole SM, the fp8
-// kernel two CTAs.
-static int ctas_per_sm(int scheme) { return scheme == WC_SCHEME_FP8_E4M3 ? kMinBlocks : 1; }
-
-// Page streams per CTA: warps, or warp pairs.
-static long streams_per_cta(int scheme) { return scheme == WC_SCHEME_DITHER_INT8_G32 ? kG32PageStreams : 8; }
-
-// Split plan.  A CTA's n page streams each take every n-th page of its split,
-// so a split of P pages costs ceil(P / n) page steps, and a wave of resident
-// CTAs adds a fixed prologue / epilogue of about one and a half page steps.
-// The split count minimises
-//     waves * (ceil(pages_per_split / n) + 1.5),   waves = ceil(CTAs / resident CTAs),
-// so a grid never spills a small remainder into an extra wave; splits keep at
-// least n pages (one per stream).  Ties go to fewer splits (less to merge).
-static long split_pages(long units, int max_pages, long slots, long streams) {
-    constexpr long kWaveCost2 = 3;    // per-wave fixed cost, in half page steps
-    const long max_splits = std::max<long>(1, std::min<long>(max_pages / streams, 4 * slots));
-    long best_pps = std::max(max_pages, 1), best_cost = -1;
-    for (long sp = 1; sp <= max_splits; ++sp) {
-        const long pps = (max_pages + sp - 1) / sp;
-        const long splits = (max_pages + pps - 1) / pps;
-        if (splits != sp) continue;   // same plan as a smaller split count
-        const long waves = (splits * units + slots - 1) / slots;
-        const long cost = waves * (2 * ((pps + streams - 1) / streams) + kWaveCost2);
-        if (best_cost < 0 || cost < best_cost) {
-            best_cost = cost;
-            best_pps = pps;
-        }
-    }
-    return best_pps;
-}
-
-DecodePlan plan_decode(int batch, int num_kv_heads, int max_pages, int num_sms, int scheme, int bits,
-                       size_t available) {
-    DecodePlan pl;
-    const long units = (long)batch * num_kv_heads;
-    const long slots = std::max<long>(1, (long)num_sms * ctas_per_sm(scheme));
-    const long best_pps = split_pages(units, max_pages, slots, streams_per_cta(scheme));
-    pl.pages_per_split = (int)best_pps;
-    pl.splits = (int)std::max<long>(1, (max_pages + best_pps - 1) / best_pps);
-    long partials = units * pl.splits;
-    // A batch of several sequences (lengths unknown to the host, often ragged)
-    // takes the flattened plan on the dithered caches: Hkv x floor(SMs / Hkv)
-    // CTAs, all resident, each taking a share of one KV head's pages.  fp8
-    // keeps the split plan: its CTAs are scheduled as SMs free up, which already
-    // evens out a ragged batch, and its pages are cheap.  So do block tables of at most
-    // kShortRounds rounds of pages: a share there has a cut every few rounds.  4 KV heads,
-    // us split / flattened: 32 sequences of 4 pages 6.9 / 9.4, 16 of 5 to 19 8.3 / 10.3, 32 of 4
-    // to 31 12.0 / 13.3, 400 of 10 to 38 111 / 114; 8 KV heads, 32 of 8 to 60 30.4 / 28.3.
-    constexpr long kShortRounds = 5;
-    const bool batched = batch > 1 && (long long)batch * max_pages < (1LL << 31) && scheme != WC_SCHEME_FP8_E4M3;
-    const int shares = std::max(1, (int)(slots / num_kv_heads));
-    const long flat_partials = (long)num_kv_heads * shares + units;
-    auto bytes = [](long n) {
-        return (256 + sizeof(float) * (size_t)n * kMaxGroup * kPartialStride + 255) & ~(size_t)255;
-    };
-    bool flat = batched;
-    if (scheme == WC_SCHEME_DITHER_INT8 && bits == 10) {
-        // The 10-bit dither's workspace is at least the size it was first given, for two
-        // CTAs per SM (and, on a batch that left some empty, a partial per warp of eight).
-        // The flattened plan of a batch whose units fill two CTAs per SM with a split each
-        // needs up to a partial per SM more: in a workspace of the first size, and beyond
-        // the allocation-free call's limit, such a batch takes a split plan.
-        const long slots2 = std::max<long>(1, 2L * num_sms), pps2 = split_pages(units, max_pages, slots2, 8);
-        const long splits2 = std::max<long>(1, (max_pages + pps2 - 1) / pps2);
-        long first = units * splits2;
-        if (batched && first < slots2) first = 8L * num_kv_heads * std::max<long>(1, slots2 / num_kv_heads) + units;
-        if (max_pages <= kShortRounds * streams_per_cta(scheme) && partials <= first) flat = false;
-        if (flat && flat_partials > first && bytes(flat_partials) > available) flat = false;
-        if (!flat && partials > first) {
-            pl.pages_per_split = (int)pps2;
-            pl.splits = (int)splits2;
-        }
-        partials = flat ? std::max(first, flat_partials) : first;
-    } else if (batched) {
-        if (max_pages <= kShortRounds * streams_per_cta(scheme) && partials <= flat_partials) flat = false;
-        partials = flat_partials;   // the workspace of either
-    }
-    if (flat) {
-        pl.splits = num_kv_heads * shares;
-        pl.pages_per_split = 0;
-    }
-    pl.partials_off = 256;
-    pl.total = bytes(partials);
-    return pl;
-}
-
 // The merge is launched early (programmatic dependent) and its CTAs become
 // resident on the SMs the decode grid frees first.  When the merge grid fits
 // in one wave, each CTA also reserves more than half of an SM's shared memory

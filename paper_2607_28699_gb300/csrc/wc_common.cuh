@@ -5,13 +5,9 @@
 #include <stdint.h>
 
 #include "../../include/witcert.h"
+#include "sizes.h"
 
 namespace wc {
-
-constexpr int kHeadDim = 128;
-constexpr int kPage = 16;
-constexpr int kBands = 8;
-constexpr int kMaxGroup = 8;
 
 // Philox4x32-10 (Salmon et al., SC'11): round constants of the published
 // algorithm.

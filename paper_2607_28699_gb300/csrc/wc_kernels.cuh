@@ -3,6 +3,7 @@
 
 #include <cuda_runtime.h>
 
+#include "dispatch.h"
 #include "per_device.h"
 #include "wc_common.cuh"
 
@@ -77,25 +78,6 @@ struct DecodeParams {
     PhiloxKeys keys;
 };
 
-// Per (query head, split) partial: acc[128] | m | l | D | Tier-B D | value
-// term | max ||v|| | pad.  140 floats: in the CTA merge's shared buffer the
-// rows of the heads one warp instruction touches then start in distinct bank
-// groups (12 words apart modulo 32; 136 would put two heads on each group).
-constexpr int kPartialStride = kHeadDim + 12;
-
-// Workspace layout (bytes): [0, 256) status word, then the partials
-// (256-byte aligned).
-struct DecodePlan {
-    int splits;            // flattened plan: the grid's CTAs
-    int pages_per_split;   // 0: the flattened plan
-    size_t partials_off, total;
-};
-
-// available: the workspace's bytes (a smaller plan is taken where the preferred one does
-// not fit and calls with that size have always been accepted); SIZE_MAX: the preferred plan.
-DecodePlan plan_decode(int batch, int num_kv_heads, int max_pages, int num_sms, int scheme, int bits,
-                       size_t available = SIZE_MAX);
-
 // The current device and its context (null until the runtime has made one current here).
 cudaError_t current_context(int* device, void** context);
 
@@ -158,9 +140,6 @@ struct RepairParams {
 // Largest block-table width the selection handles (its sort holds one cell's
 // pages in shared memory).
 constexpr int kRepairMaxPages = 16384;
-// Page streams (producer / consumer warp pairs) per CTA of the grouped-scheme
-// decode; the split planner sizes splits by it.
-constexpr int kG32PageStreams = 6;
 
 cudaError_t launch_write(const WriteParams& p, int scheme, int bits, cudaStream_t stream);
 cudaError_t launch_decode(const DecodeParams& p, int scheme, int bits, cudaStream_t stream);
