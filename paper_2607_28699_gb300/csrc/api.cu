@@ -313,6 +313,7 @@ static wc_status decode_with_workspace(const wc_cache_desc* desc, int32_t layer,
     p.rope_layout = desc->rope_layout;
     p.splits = pl.splits;
     p.pages_per_split = pl.pages_per_split;
+    p.two_per_sm = pl.two_per_sm;
     p.keys = wc::make_philox_keys(desc->seed);
     cudaError_t e = wc::launch_decode(p, desc->scheme, desc->dither_bits, static_cast<cudaStream_t>(stream));
     return e == cudaSuccess ? WC_OK : cuda_fail(e, "decode kernel launch");
@@ -632,6 +633,7 @@ extern "C" wc_status wc_metered_decode_attention_noalloc(
     p.rope_layout = desc->rope_layout;
     p.splits = pl.splits;
     p.pages_per_split = pl.pages_per_split;
+    p.two_per_sm = pl.two_per_sm;
     p.keys = wc::make_philox_keys(desc->seed);
     cudaError_t e = wc::launch_decode(p, desc->scheme, desc->dither_bits, static_cast<cudaStream_t>(stream));
     return e == cudaSuccess ? WC_OK : cuda_fail(e, "decode kernel launch");

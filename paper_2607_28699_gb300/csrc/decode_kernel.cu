@@ -6,7 +6,8 @@
 // merged across context splits under log-sum-exp weights (A is a p~-weighted
 // mean, so it merges exactly like the output; §6.2.2).
 //
-// Two kernels.  decode_kernel (fp8-e4m3): grid (splits, Hkv, batch), 8 warps per
+// Two kernels.  decode_kernel (fp8-e4m3, and the 10-bit dither's batches of many short
+// sequences): grid (splits, Hkv, batch), 8 warps per
 // CTA, two CTAs per SM; each warp owns a 3-stage ring of page buffers in shared
 // memory that one of its lanes fills ahead of use: the K and V code tiles (2 KiB
 // each) by tensor-map TMA with the 128-byte swizzle (so the 16-byte reads of a warp
@@ -51,10 +52,13 @@ constexpr int kStageBytes = 4416;        // copy bytes: K codes | V codes | K sc
 // each, written by tensor-map TMA with the 128-byte swizzle (1024-byte aligned
 // regions), then each stage's scales and witness, then the barriers.
 constexpr int kTileRegion = kWarps * kStages * 2048;
-constexpr int kOffW = 64;                // within a stage's small part
+constexpr int kOffKs = 0, kOffVs = 32, kOffW = 64;   // within a stage's small part
 constexpr int kOffVw = 320;              // value witness [16][2] fp16 (value side)
 constexpr int kSmallStride = 384;
-constexpr int kSmemBytes = 2 * kTileRegion + kWarps * kStages * kSmallStride + kWarps * kStages * 8 + 1024;
+constexpr int kOffQ = 2 * kTileRegion + kWarps * kStages * kSmallStride + kWarps * kStages * 8;   // query fragment (kQShared)
+constexpr int kQBytes = 16 * 32 * 4;
+constexpr int kSmemBytes = kOffQ + kQBytes + 1024;
+static_assert(kOffQ % 16 == 0 && 2 * (kSmemBytes + 1024) <= 228 * 1024, "two CTAs per SM");
 
 // decode_kernel's parameters: the code tiles' tensor maps and the call.
 struct DkParams {
@@ -101,9 +105,11 @@ __device__ __forceinline__ void load_q_frag(const DecodeParams& p, int b, int h,
     }
 }
 
-template <int kX>
+// kInt8: the dithered INT8 cache with the 10-bit dither; otherwise fp8-e4m3.
+template <bool kInt8, int kX>
 __global__ void __launch_bounds__(kThreads, kMinBlocks) decode_kernel(const __grid_constant__ DkParams dp) {
-    constexpr bool kValue = (kX & kXValue) != 0, kRepair = (kX & kXRepair) != 0;
+    constexpr bool kTierB = (kX & kXTierB) != 0, kValue = (kX & kXValue) != 0, kRepair = (kX & kXRepair) != 0;
+    static_assert(kInt8 || !kTierB, "Tier B needs the dither");
     const DecodeParams& p = dp.p;
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     uint8_t* smem = smem_raw + ((1024 - (smem_addr(smem_raw) & 1023)) & 1023);
@@ -139,6 +145,18 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) decode_kernel(const __gr
     }
     int ctx = __ldg(p.ctx_lens + b);
     load_q_frag(p, b, h, G, g, c, qw);
+    // Tier B and the value side of the dithered cache read the query fragment (the same in every
+    // warp) from shared memory page by page: with its 16 registers held through the PV products
+    // they spill (3% of a call; the plain and the repair variant do not gain).
+    constexpr bool kQShared = kInt8 && (kTierB || kValue);
+    uint4* q_s = reinterpret_cast<uint4*>(smem + kOffQ) + lane;
+    if constexpr (kQShared) {
+        if (warp == 0) {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) q_s[32 * i] = make_uint4(qw[4 * i], qw[4 * i + 1], qw[4 * i + 2], qw[4 * i + 3]);
+        }
+        __syncthreads();
+    }
     if (ctx < 0 || ctx > p.max_pages * kPage) {
         if (threadIdx.x == 0 && split == 0 && h == 0) atomicOr(p.status, WC_DEV_BAD_CTX);
         ctx = max(0, min(ctx, p.max_pages * kPage));
@@ -160,9 +178,13 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) decode_kernel(const __gr
         uint8_t* st = my_small + s * kSmallStride;
         const int z = phys * p.num_kv_heads + h;
         const size_t ph = (size_t)z;
-        mbar_arrive_expect_tx(bar, (2048 + 2048 + 256) + (kValue ? 64 : 0));
+        mbar_arrive_expect_tx(bar, (kInt8 ? kStageBytes : 2048 + 2048 + 256) + (kValue ? 64 : 0));
         tma_page(my_k + s * 2048, &dp.k_map, z, bar);
         tma_page(my_k + kTileRegion + s * 2048, &dp.v_map, z, bar);
+        if constexpr (kInt8) {
+            bulk_g2s(st + kOffKs, p.k_scale + ph * kPage, 32, bar);
+            bulk_g2s(st + kOffVs, p.v_scale + ph * kPage, 32, bar);
+        }
         bulk_g2s(st + kOffW, p.k_witness + ph * (kPage * kBands), 256, bar);
         if constexpr (kValue) bulk_g2s(st + kOffVw, p.v_witness + ph * (kPage * 2), 64, bar);
     };
@@ -175,12 +197,31 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) decode_kernel(const __gr
 
     // ---- band norms and the bound operand ----------------------------------------
     uint32_t a_hi = 0, a_lo = 0;   // B operand of the bound: a[head g][bands 2c, 2c+1]
+    float alpha0 = 0.f, alpha1 = 0.f, zoff0 = 0.f, zoff1 = 0.f;   // of the softmax heads 2c, 2c+1
+    constexpr float kKappa = DitherConst<10>::kappa;
+    constexpr uint32_t kSubV = 0x647F647Fu;                       // 1152 - 1 (u8x2_minus)
     {
-        float part[4] = {0.f, 0.f, 0.f, 0.f};
+        float part[4] = {0.f, 0.f, 0.f, 0.f}, qsum = 0.f;
 #pragma unroll
         for (int i = 0; i < 16; ++i) {
             const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&qw[i]));
+            if constexpr (kInt8) qsum += f.x + f.y;
             part[i >> 2] = fmaf(f.x, f.x, fmaf(f.y, f.y, part[i >> 2]));   // channels 32c + 8(i>>2) .. +7
+        }
+        if constexpr (kInt8) {   // kappa * sum(q)
+            qsum += __shfl_xor_sync(0xffffffffu, qsum, 1);
+            qsum += __shfl_xor_sync(0xffffffffu, qsum, 2);
+            zoff0 = kKappa * __shfl_sync(0xffffffffu, qsum, 8 * c);
+            zoff1 = kKappa * __shfl_sync(0xffffffffu, qsum, 8 * c + 4);
+        }
+        if constexpr (kTierB) {   // §4.2: u_t = alpha s_t with alpha = sqrt(2 log(2S/delta) ||q||^2 / (12 d))
+            float qn2 = part[0] + part[1] + part[2] + part[3];   // ||q_g||^2 over channels 32c .. 32c+31
+            qn2 += __shfl_xor_sync(0xffffffffu, qn2, 1);
+            qn2 += __shfl_xor_sync(0xffffffffu, qn2, 2);
+            const float lg = p.tb_log_2_over_delta + logf((float)max(ctx, 1));   // log(2S / delta)
+            const float al = sqrtf(2.0f * lg * qn2 * (1.0f / (12.0f * kHeadDim)));
+            alpha0 = __shfl_sync(0xffffffffu, al, 8 * c);
+            alpha1 = __shfl_sync(0xffffffffu, al, 8 * c + 4);
         }
         float band_a, band_b;   // squared norms of bands 2c and 2c+1 of head g
         if (p.rope_layout == WC_ROPE_HALF) {
@@ -215,7 +256,14 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) decode_kernel(const __gr
     float acc[8][4];
 #pragma unroll
     for (int i = 0; i < 8; ++i) acc[i][0] = acc[i][1] = acc[i][2] = acc[i][3] = 0.f;
-    constexpr int kLamExp = 6;       // P * 2^kLamExp stays below 2^14 (fp16)
+    float db_part[2] = {0.f, 0.f};   // Tier-B meter (kTierB)
+    float spv_part[2] = {0.f, 0.f};  // sum P s_v (kInt8)
+    // P * s_v * 2^lam_exp stays below 2^14 (fp16): s_v * 2^lam_exp < 2^6 (fp8: s_v = 1).  It only
+    // decreases; sv_lim = 2^(6 - lam_exp) is the scale at which it must, FLT_MIN until the
+    // first positive scale.
+    int lam_exp = kInt8 ? INT_MIN : 6;
+    float sv_lim = 1.17549435e-38f;
+    const uint32_t c1 = (uint32_t)p.layer * 65536u + (uint32_t)h;   // Philox counter word (kInt8)
     bool failed = false;
     int consumed = 0;
 
@@ -241,6 +289,13 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) decode_kernel(const __gr
             // rows g and g+8 are tokens g and g+8; dc[0..3] =
             // (tok g, head 2c), (tok g, 2c+1), (tok g+8, 2c), (tok g+8, 2c+1)
             float dc[4] = {0.f, 0.f, 0.f, 0.f};
+            if constexpr (kQShared) {
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const uint4 v = q_s[32 * i];
+                    qw[4 * i] = v.x; qw[4 * i + 1] = v.y; qw[4 * i + 2] = v.z; qw[4 * i + 3] = v.w;
+                }
+            }
 #pragma unroll
             for (int gp = 0; gp < 2; ++gp) {                 // channels 32c + 16gp .. +15
                 const uint4 ka = *reinterpret_cast<const uint4*>(kt + swz(g, 2 * c + gp));
@@ -249,10 +304,45 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) decode_kernel(const __gr
                 for (int kk = 0; kk < 4; ++kk) {
                     const int ks = 4 * gp + kk;              // channels 32c + 4ks .. +3
                     const uint32_t wa = word_of(ka, kk), wb = word_of(kb, kk);
-                    const uint32_t A[4] = {e4m3x2_to_h2(wa), e4m3x2_to_h2(wb), e4m3x2_to_h2(wa >> 16),
-                                           e4m3x2_to_h2(wb >> 16)};
+                    uint32_t A[4];
+                    if constexpr (kInt8) {
+                        const uint32_t xa = wa ^ 0x80808080u, xb = wb ^ 0x80808080u;
+                        A[0] = s8x2_to_h2(xa, kSel01);
+                        A[1] = s8x2_to_h2(xb, kSel01);
+                        A[2] = s8x2_to_h2(xa, kSel23);
+                        A[3] = s8x2_to_h2(xb, kSel23);
+                    } else {
+                        A[0] = e4m3x2_to_h2(wa);
+                        A[1] = e4m3x2_to_h2(wb);
+                        A[2] = e4m3x2_to_h2(wa >> 16);
+                        A[3] = e4m3x2_to_h2(wb >> 16);
+                    }
                     mma16816(dc, A, qw[2 * ks], qw[2 * ks + 1]);
                 }
+            }
+            float sk[2] = {1.f, 1.f}, sv[2] = {1.f, 1.f};   // scales of tokens g, g+8
+            if constexpr (kInt8) {
+                float dd[4] = {0.f, 0.f, 0.f, 0.f};          // h' . q
+#pragma unroll
+                for (int gi = 0; gi < 4; ++gi) {             // a Philox call covers 8 channels
+                    const uint4 da = philox((uint32_t)phys * kPage + g, c1, (uint32_t)(4 * c + gi), 0u, p.keys);
+                    const uint4 db = philox((uint32_t)phys * kPage + g + 8, c1, (uint32_t)(4 * c + gi), 0u, p.keys);
+#pragma unroll
+                    for (int kk = 0; kk < 2; ++kk) {
+                        const int ks = 2 * gi + kk;
+                        const uint32_t H[4] = {h10(word_of(da, 2 * kk)), h10(word_of(db, 2 * kk)),
+                                               h10(word_of(da, 2 * kk + 1)), h10(word_of(db, 2 * kk + 1))};
+                        mma16816(dd, H, qw[2 * ks], qw[2 * ks + 1]);
+                    }
+                }
+#pragma unroll
+                for (int i = 0; i < 4; ++i) dc[i] = dc[i] - dd[i] + ((i & 1) ? zoff1 : zoff0);
+                const __half* ks = reinterpret_cast<const __half*>(st + kOffKs);
+                const __half* vs = reinterpret_cast<const __half*>(st + kOffVs);
+                sk[0] = __half2float(ks[g]);
+                sk[1] = __half2float(ks[g + 8]);
+                sv[0] = __half2float(vs[g]);
+                sv[1] = __half2float(vs[g + 8]);
             }
 
             // ---------------- logits, bound, softmax ------------------------------
@@ -264,28 +354,26 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) decode_kernel(const __gr
                 mma16816(cb, A, a_hi, a_lo);
             }
             float y[4], P[4], cl[4];     // cl: the bounds in log2 units
+            auto ub = [&](int i) { return ((i & 1) ? alpha1 : alpha0) * sk[i >> 1] * kLog2e; };   // Tier B's
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
-                y[i] = dc[i] * kRsdLog2e;
+                y[i] = kInt8 ? dc[i] * (sk[i >> 1] * kRsdLog2e) : dc[i] * kRsdLog2e;
                 cl[i] = cb[i] * kLog2e;
             }
-            float rho[2] = {0.f, 0.f}, vn[2] = {0.f, 0.f};   // value witness of tokens g, g+8 (0 past the context)
-            if constexpr (kValue) {
-                const float2 w0 = __half22float2(*reinterpret_cast<const __half2*>(st + kOffVw + 4 * g));
-                const float2 w1 = __half22float2(*reinterpret_cast<const __half2*>(st + kOffVw + 4 * (g + 8)));
-                rho[0] = w0.x;
-                rho[1] = w1.x;
-                vn[0] = w0.y;
-                vn[1] = w1.y;
-            }
             // One warp vote finds everything that an ordinary page does not need: the
-            // context's last page, a logit more than 8 above the reference, a bound of
-            // kHugeLog2 or more (meter_term).  Masks, six shuffles of the maximum and the
-            // second vote on every page cost 2% (32 sequences, two layers: 245.6 -> 240.1 us).
-            const float big = fmaxf(fmaxf(cl[0], cl[1]), fmaxf(cl[2], cl[3]));
+            // context's last page, a logit more than 8 above the reference, a V scale above the
+            // P scale's limit, a bound of kHugeLog2 or more (meter_term).  Masks, six shuffles of
+            // the maximum and the second vote on every page cost up to 2% (32 sequences of 1000
+            // pages, 56 heads: 175.1 -> 172.9 us).
+            auto largest = [&] {
+                float m = fmaxf(fmaxf(cl[0], cl[1]), fmaxf(cl[2], cl[3]));
+                if constexpr (kTierB) m = fmaxf(m, fmaxf(fmaxf(ub(0), ub(1)), fmaxf(ub(2), ub(3))));
+                return m;
+            };
             bool huge = false;
             if (__any_sync(0xffffffffu, nvalid < kPage || fmaxf(y[0], y[2]) > m_run[0] + 8.0f ||
-                                            fmaxf(y[1], y[3]) > m_run[1] + 8.0f || !(big < kHugeLog2))) {
+                                            fmaxf(y[1], y[3]) > m_run[1] + 8.0f || !(largest() < kHugeLog2) ||
+                                            (kInt8 && fmaxf(sv[0], sv[1]) >= sv_lim))) {
                 const bool ok0 = g < nvalid, ok1 = g + 8 < nvalid;
 #pragma unroll
                 for (int i = 0; i < 4; ++i)
@@ -293,9 +381,9 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) decode_kernel(const __gr
                         y[i] = -INFINITY;
                         cl[i] = 0.f;
                     }
-                if (!ok0) rho[0] = vn[0] = 0.f;
-                if (!ok1) rho[1] = vn[1] = 0.f;
-                huge = __any_sync(0xffffffffu, fmaxf(fmaxf(cl[0], cl[1]), fmaxf(cl[2], cl[3])) >= kHugeLog2);
+                if (!ok0) sv[0] = sk[0] = 0.f;
+                if (!ok1) sv[1] = sk[1] = 0.f;
+                huge = __any_sync(0xffffffffu, largest() >= kHugeLog2);
                 float mx0 = fmaxf(y[0], y[2]), mx1 = fmaxf(y[1], y[3]);
 #pragma unroll
                 for (int o = 4; o < 32; o <<= 1) {
@@ -310,6 +398,8 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) decode_kernel(const __gr
                     if (mv1) m_run[1] = mx1;
                     l_part[0] *= a0; d_part[0] *= a0;
                     l_part[1] *= a1; d_part[1] *= a1;
+                    if constexpr (kTierB) { db_part[0] *= a0; db_part[1] *= a1; }
+                    if constexpr (kInt8) { spv_part[0] *= a0; spv_part[1] *= a1; }
                     if constexpr (kValue) { vt_part[0] *= a0; vt_part[1] *= a1; }
 #pragma unroll
                     for (int mt = 0; mt < 8; ++mt) {
@@ -317,8 +407,30 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) decode_kernel(const __gr
                         acc[mt][1] *= a1; acc[mt][3] *= a1;
                     }
                 }
+                if constexpr (kInt8) {
+                    const float smax = fmaxf(sv[0], sv[1]);
+                    if (__any_sync(0xffffffffu, smax >= sv_lim)) {
+                        const float wmax = __int_as_float(__reduce_max_sync(0xffffffffu, __float_as_int(smax)));
+                        const int want = 6 - (((__float_as_int(wmax) >> 23) & 0xFF) - 126);   // wmax < 2^(6 - want)
+                        if (lam_exp != INT_MIN) {   // want < lam_exp here
+                            const float f = pow2(want - lam_exp);
+#pragma unroll
+                            for (int mt = 0; mt < 8; ++mt)
+#pragma unroll
+                                for (int e2 = 0; e2 < 4; ++e2) acc[mt][e2] *= f;
+                        }
+                        lam_exp = want;
+                        sv_lim = pow2(6 - lam_exp);
+                    }
+                }
             }
-            if constexpr (kValue) vmax = fmaxf(vmax, fmaxf(vn[0], vn[1]));
+            float rho[2] = {0.f, 0.f};   // value witness of tokens g, g+8 (0 past the context)
+            if constexpr (kValue) {
+                const float2 w0 = __half22float2(*reinterpret_cast<const __half2*>(st + kOffVw + 4 * g));
+                const float2 w1 = __half22float2(*reinterpret_cast<const __half2*>(st + kOffVw + 4 * (g + 8)));
+                if (g < nvalid) { rho[0] = w0.x; vmax = fmaxf(vmax, w0.y); }
+                if (g + 8 < nvalid) { rho[1] = w1.x; vmax = fmaxf(vmax, w1.y); }
+            }
             float dpg[2] = {0.f, 0.f};   // this page's share of D (kRepair)
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
@@ -329,17 +441,20 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) decode_kernel(const __gr
                     const float em1 = fast_exp2(cl[i]) - 1.f;
                     d_part[e] = fmaf(pe, em1, d_part[e]);
                     if constexpr (kRepair) dpg[e] = fmaf(pe, em1, dpg[e]);
+                    if constexpr (kTierB) db_part[e] = fmaf(pe, fast_exp2(ub(i)) - 1.f, db_part[e]);
                 }
                 if constexpr (kValue) vt_part[e] = fmaf(pe, rho[r], vt_part[e]);
-                P[i] = pe;
+                P[i] = kInt8 ? pe * sv[r] : pe;
+                if constexpr (kInt8) spv_part[e] += P[i];
             }
             if (huge) {
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
                     const int e = i & 1;
-                    const float dt = meter_term(y[i] - m_run[e], cl[i]);
+                    const float t = y[i] - m_run[e], dt = meter_term(t, cl[i]);
                     d_part[e] += dt;
                     if constexpr (kRepair) dpg[e] += dt;
+                    if constexpr (kTierB) db_part[e] += meter_term(t, ub(i));
                 }
             }
             if constexpr (kRepair) emit_page_terms(p, b, h, G, lp, g, c, dpg, m_run);
@@ -349,7 +464,7 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) decode_kernel(const __gr
             // transposed with movmatrix into (P[tok 2c][head g], P[tok 2c+1][head g]).
             uint32_t bp0, bp1, bl0, bl1;
             {
-                const float lam = pow2(kLamExp);
+                const float lam = pow2(kInt8 && lam_exp == INT_MIN ? 0 : lam_exp);
                 const float x0 = P[0] * lam, x1 = P[1] * lam, x2 = P[2] * lam, x3 = P[3] * lam;
                 const uint32_t h01 = pack_h2(x0, x1), h23 = pack_h2(x2, x3);
                 const float2 r01 = __half22float2(*reinterpret_cast<const __half2*>(&h01));
@@ -362,11 +477,24 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) decode_kernel(const __gr
             }
 
             // ---------------- PV: acc[dim][head] ------------------------------------
+            // The MMA truncates its sums: with the dither, whose terms nearly cancel, a page's are
+            // taken from zero and added rounded (codes and dither apart: together they need
+            // registers that are not there).
+            auto add_pv = [&](int mt, const uint32_t (&A)[4]) {
+                float page_sum[4] = {0.f, 0.f, 0.f, 0.f};
+                float(&sum)[4] = kInt8 ? page_sum : acc[mt];
+                mma16816(sum, A, bp0, bp1);
+                mma16816(sum, A, bl0, bl1);
+                if constexpr (kInt8) {
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) acc[mt][i] += page_sum[i];
+                }
+            };
             const int tv[4] = {2 * c, 2 * c + 1, 2 * c + 8, 2 * c + 9};
             uint4 vq[4];
 #pragma unroll
             for (int j = 0; j < 4; ++j) vq[j] = *reinterpret_cast<const uint4*>(kt + kTileRegion + swz(tv[j], g));
-            if (nvalid < kPage) {   // an fp8 NaN byte in an unused tail slot would poison P = 0 columns
+            if (!kInt8 && nvalid < kPage) {   // an fp8 NaN byte in an unused tail slot would poison P = 0 columns
 #pragma unroll
                 for (int j = 0; j < 4; ++j)
                     if (tv[j] >= nvalid) vq[j] = make_uint4(0, 0, 0, 0);
@@ -377,12 +505,38 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) decode_kernel(const __gr
                 uint32_t A[4];
 #pragma unroll
                 for (int pr = 0; pr < 2; ++pr) {
-                    const uint32_t X = prmt(word_of(vq[2 * pr], wi), word_of(vq[2 * pr + 1], wi), sel_interleave(pos));
-                    A[2 * pr] = e4m3x2_to_h2(X);
-                    A[2 * pr + 1] = e4m3x2_to_h2(X >> 16);
+                    if constexpr (kInt8) {
+                        const uint32_t X = prmt(word_of(vq[2 * pr], wi) ^ 0x80808080u,
+                                                word_of(vq[2 * pr + 1], wi) ^ 0x80808080u, sel_interleave(pos));
+                        A[2 * pr] = u8x2_minus(X, kSel01, kSubV);   // code + 1
+                        A[2 * pr + 1] = u8x2_minus(X, kSel23, kSubV);
+                    } else {
+                        const uint32_t X = prmt(word_of(vq[2 * pr], wi), word_of(vq[2 * pr + 1], wi), sel_interleave(pos));
+                        A[2 * pr] = e4m3x2_to_h2(X);
+                        A[2 * pr + 1] = e4m3x2_to_h2(X >> 16);
+                    }
                 }
-                mma16816(acc[mt], A, bp0, bp1);
-                mma16816(acc[mt], A, bl0, bl1);
+                add_pv(mt, A);
+            }
+            if constexpr (kInt8) {   // - H^T P^T
+#pragma unroll
+                for (int hf = 0; hf < 2; ++hf) {
+                    uint4 dv[4];
+#pragma unroll
+                    for (int j = 0; j < 4; ++j)
+                        dv[j] = philox((uint32_t)phys * kPage + tv[j], c1, (uint32_t)(2 * g + hf), 1u, p.keys);
+#pragma unroll
+                    for (int mm = 0; mm < 4; ++mm) {
+                        uint32_t H[4];
+#pragma unroll
+                        for (int pr = 0; pr < 2; ++pr) {
+                            const uint32_t wa = word_of(dv[2 * pr], mm), wb = word_of(dv[2 * pr + 1], mm);
+                            H[2 * pr] = h10(prmt(wa, wb, 0x5410u)) | 0x80008000u;
+                            H[2 * pr + 1] = h10(prmt(wa, wb, 0x7632u)) | 0x80008000u;
+                        }
+                        add_pv(4 * hf + mm, H);
+                    }
+                }
             }
         } else if constexpr (kRepair) {
             emit_skipped_page(p, b, h, G, lp, lane);
@@ -408,6 +562,8 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) decode_kernel(const __gr
         for (int e = 0; e < 2; ++e) {
             l_part[e] += __shfl_xor_sync(0xffffffffu, l_part[e], o);
             d_part[e] += __shfl_xor_sync(0xffffffffu, d_part[e], o);
+            if constexpr (kTierB) db_part[e] += __shfl_xor_sync(0xffffffffu, db_part[e], o);
+            if constexpr (kInt8) spv_part[e] += __shfl_xor_sync(0xffffffffu, spv_part[e], o);
             if constexpr (kValue) vt_part[e] += __shfl_xor_sync(0xffffffffu, vt_part[e], o);
         }
     if constexpr (kValue)
@@ -416,23 +572,26 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) decode_kernel(const __gr
     float* mbuf = reinterpret_cast<float*>(smem);   // [warp][head][kPartialStride]
     {
         float* wb = mbuf + warp * kMaxGroup * kPartialStride;
-        const float inv_lam = pow2(-kLamExp);
+        const float inv_lam = pow2(kInt8 && lam_exp == INT_MIN ? 0 : -lam_exp);
 #pragma unroll
         for (int e = 0; e < 2; ++e) {
             float* row = wb + (2 * c + e) * kPartialStride + 16 * g;   // dims 16g .. 16g+15
+            const float add = (kKappa - 1.0f) * spv_part[e];           // xi = h' - kappa, the codes raised by 1 (fp8: 0)
+            auto out = [&](float x) { return kInt8 ? fmaf(x, inv_lam, add) : x * inv_lam; };
 #pragma unroll
             for (int q4 = 0; q4 < 4; ++q4) {
                 float4 v;
-                v.x = acc[2 * q4][e] * inv_lam;
-                v.y = acc[2 * q4][e + 2] * inv_lam;
-                v.z = acc[2 * q4 + 1][e] * inv_lam;
-                v.w = acc[2 * q4 + 1][e + 2] * inv_lam;
+                v.x = out(acc[2 * q4][e]);
+                v.y = out(acc[2 * q4][e + 2]);
+                v.z = out(acc[2 * q4 + 1][e]);
+                v.w = out(acc[2 * q4 + 1][e + 2]);
                 *reinterpret_cast<float4*>(row + 4 * q4) = v;
             }
             if (g == 0) {
                 wb[(2 * c + e) * kPartialStride + kHeadDim + 0] = m_run[e];
                 wb[(2 * c + e) * kPartialStride + kHeadDim + 1] = l_part[e];
                 wb[(2 * c + e) * kPartialStride + kHeadDim + 2] = d_part[e];
+                if constexpr (kTierB) wb[(2 * c + e) * kPartialStride + kHeadDim + 3] = db_part[e];
                 if constexpr (kValue) {
                     wb[(2 * c + e) * kPartialStride + kHeadDim + 4] = vt_part[e];
                     wb[(2 * c + e) * kPartialStride + kHeadDim + 5] = vmax;
@@ -467,6 +626,7 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) decode_kernel(const __gr
             } else {
                 s.x = fmaf(wt, src[0], s.x);   // l
                 s.y = fmaf(wt, src[1], s.y);   // D
+                if constexpr (kTierB) s.z = fmaf(wt, src[2], s.z);   // Tier-B D
                 if constexpr (kValue) s.w = fmaf(wt, src[3], s.w);   // value term
             }
         }
@@ -477,6 +637,7 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) decode_kernel(const __gr
             dst[kHeadDim] = M;
             dst[kHeadDim + 1] = s.x;
             dst[kHeadDim + 2] = s.y;
+            if constexpr (kTierB) dst[kHeadDim + 3] = s.z;
             if constexpr (kValue) {
                 float vm = 0.f;
                 for (int w = 0; w < kWarps; ++w)
@@ -1668,17 +1829,17 @@ cudaError_t launch_merge_x(const DecodeParams& p, int x, cudaStream_t stream) {
          : x == kXRepair ? launch_merge<kXRepair>(p, stream) : launch_merge<0>(p, stream);
 }
 
-template <int kX>
-static cudaError_t launch_fp8(const DecodeParams& p, cudaStream_t stream) {
+template <bool kInt8, int kX>
+static cudaError_t launch_two_per_sm(const DecodeParams& p, cudaStream_t stream) {
     static PerDevice<Configured, cudaError_t> configured;
-    if (cudaError_t e = configure(configured, decode_kernel<kX>, kSmemBytes)) return e;
+    if (cudaError_t e = configure(configured, decode_kernel<kInt8, kX>, kSmemBytes)) return e;
     DkParams dp;
     dp.p = p;
     if (!encode_page_map(&dp.k_map, p.k_codes, p.num_pages, p.num_kv_heads) ||
         !encode_page_map(&dp.v_map, p.v_codes, p.num_pages, p.num_kv_heads))
         return cudaErrorInvalidValue;
     const dim3 grid(p.splits, p.num_kv_heads, p.batch);
-    cudaError_t e = launch_pdl(decode_kernel<kX>, grid, dim3(kThreads), kSmemBytes, stream, dp);
+    cudaError_t e = launch_pdl(decode_kernel<kInt8, kX>, grid, dim3(kThreads), kSmemBytes, stream, dp);
     if (e != cudaSuccess) return e;
     // the merge is a programmatic dependent too: its CTAs are scheduled while
     // the decode grid drains and wait (griddepcontrol.wait) for all of it
@@ -1770,8 +1931,13 @@ cudaError_t launch_decode(const DecodeParams& p, int scheme, int bits, cudaStrea
     const bool flat = p.pages_per_split == 0;
     if (scheme == WC_SCHEME_FP8_E4M3)   // always the split plan (plan_decode)
         return flat           ? cudaErrorNotSupported
-             : x == kXValue  ? launch_fp8<kXValue>(p, stream)
-             : x == kXRepair ? launch_fp8<kXRepair>(p, stream) : launch_fp8<0>(p, stream);
+             : x == kXValue  ? launch_two_per_sm<false, kXValue>(p, stream)
+             : x == kXRepair ? launch_two_per_sm<false, kXRepair>(p, stream) : launch_two_per_sm<false, 0>(p, stream);
+    if (p.two_per_sm)                   // 10-bit dither, split plan (plan_decode)
+        return flat || bits != 10    ? cudaErrorNotSupported
+             : x == kXTierB  ? launch_two_per_sm<true, kXTierB>(p, stream)
+             : x == kXValue  ? launch_two_per_sm<true, kXValue>(p, stream)
+             : x == kXRepair ? launch_two_per_sm<true, kXRepair>(p, stream) : launch_two_per_sm<true, 0>(p, stream);
     if (p.stall_page >= 0)   // failure-detection test (checked by the caller: 8-bit dither, no extras)
         return bits == 8 && !flat && x == 0 ? launch_ws<8, kXStall>(p, stream) : cudaErrorNotSupported;
     if (bits == 8) return flat ? launch_ws_x<8, kXFlat>(p, x, stream) : launch_ws_x<8, 0>(p, x, stream);

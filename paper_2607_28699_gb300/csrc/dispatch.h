@@ -54,6 +54,7 @@ constexpr bool repair_wide(int64_t cells, int threads) { return cells * threads 
 struct DecodePlan {
     int splits;            // flattened plan: the grid's CTAs
     int pages_per_split;   // 0: the flattened plan
+    bool two_per_sm;       // 10-bit dither: the kernel with two CTAs per SM (split plan)
     size_t partials_off, total;
 };
 
@@ -97,6 +98,23 @@ constexpr bool short_table_flat(long units, int num_sms, int scheme, int bits, i
            (append ? units > num_sms : units >= 4L * num_sms && group <= (units >= 10L * num_sms ? 5 : 3));
 }
 
+// The 10-bit dither has two kernels: warp pairs, one CTA per SM (a page's dither is drawn beside
+// the consuming warp), and two CTAs of 8 warps per SM (drawn by the warp itself: slower pages, but
+// one CTA's prologue and merge under the other's pages).  The second is the faster one where its
+// CTAs fill the SMs (units >= 2 x 152) with tables so short that a unit's fixed part counts, on
+// the split plan: a CTA starts when another ends, which evens out lengths while the tables are a
+// small part of an SM's work.  us, pairs / two per SM, equal lengths | a quarter of the table
+// and up | one long sequence among short ones:
+//   38 sequences x 8 KV heads, 20 pages 24.3 / 21.5 | 24.2 / 21.3 | 17.9 / 16.7, 40 36.7 / 34.4 | 33.5 / 31.7 | 20.4 / 24.6
+//   76 x 8, 41 pages 73.4 / 66.8 | 53.8 / 55.1 | 29.9 / 26.8, 60 95.2 / 91.2 | 75.0 / 81.1 | 35.0 / 33.9
+//   300 x 4, 80 pages 250 / 231 | 185 / 176 | 79.5 / 60.8, 120 352 / 332 | 249 / 250 | 95.0 / 76.0
+//   1000 x 4, 5 pages 195 / 127 | 176 / 117 | 169 / 103
+constexpr long kTwoPerSmPages = 24;   // of the table, per unit that an SM's two CTAs each take
+constexpr bool ten_bit_two_per_sm(long units, int max_pages, int num_sms) {
+    const long slots2 = 2L * num_sms;
+    return units >= slots2 && max_pages * slots2 <= kTwoPerSmPages * units;
+}
+
 // available: the workspace's bytes (a smaller plan is taken where the preferred one does
 // not fit and calls with that size have always been accepted); SIZE_MAX: the preferred plan.
 // The size does not depend on group and append.
@@ -108,6 +126,7 @@ inline DecodePlan plan_decode(int batch, int num_kv_heads, int max_pages, int nu
     const long slots = std::max<long>(1, (long)num_sms * (scheme == WC_SCHEME_FP8_E4M3 ? 2 : 1));
     const long streams = scheme == WC_SCHEME_DITHER_INT8_G32 ? kG32PageStreams : kPageStreams;
     const long best_pps = split_pages(units, max_pages, slots, streams);
+    pl.two_per_sm = false;
     pl.pages_per_split = (int)best_pps;
     pl.splits = (int)std::max<long>(1, (max_pages + best_pps - 1) / best_pps);
     long partials = units * pl.splits;
@@ -130,18 +149,21 @@ inline DecodePlan plan_decode(int batch, int num_kv_heads, int max_pages, int nu
         // CTAs per SM (and, on a batch that left some empty, a partial per warp of eight).
         // The flattened plan of a batch whose units fill two CTAs per SM with a split each
         // needs up to a partial per SM more: in a workspace of the first size, and beyond
-        // the allocation-free call's limit, such a batch takes a split plan.
+        // the allocation-free call's limit, such a batch takes the two CTAs per SM.
         const long slots2 = std::max<long>(1, 2L * num_sms), pps2 = split_pages(units, max_pages, slots2, 8);
         const long splits2 = std::max<long>(1, (max_pages + pps2 - 1) / pps2);
         long first = units * splits2;
         if (batched && first < slots2) first = 8L * num_kv_heads * std::max<long>(1, slots2 / num_kv_heads) + units;
         if (short_table && partials <= first) flat = false;
-        if (flat && flat_partials > first && bytes(flat_partials) > available) flat = false;
-        if (!flat && partials > first) {
+        const long most = flat ? std::max(first, flat_partials) : first;   // the workspace of either kernel
+        pl.two_per_sm = ten_bit_two_per_sm(units, max_pages, num_sms) ||
+                        (flat ? most > first && bytes(most) > available : partials > first);
+        if (pl.two_per_sm) {
+            flat = false;
             pl.pages_per_split = (int)pps2;
             pl.splits = (int)splits2;
         }
-        partials = flat ? std::max(first, flat_partials) : first;
+        partials = bytes(most) <= available ? most : first;
     } else if (batched) {
         if (short_table && partials <= flat_partials) flat = false;
         partials = flat_partials;   // the workspace of either

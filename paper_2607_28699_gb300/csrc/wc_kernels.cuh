@@ -75,6 +75,7 @@ struct DecodeParams {
     // pages each next segment increments j, b or both), so splits + batch Hkv
     // partials suffice.
     int32_t splits, pages_per_split;
+    int32_t two_per_sm = 0;   // 10-bit dither: DecodePlan::two_per_sm
     PhiloxKeys keys;
 };
 

@@ -14,7 +14,7 @@ SOURCE = r"""
 extern "C" {
 void plan(int batch, int heads, int max_pages, int scheme, int bits, int group, int append, long available, long* out) {
     const wc::DecodePlan p = wc::plan_decode(batch, heads, max_pages, 152, scheme, bits, group, append != 0, (size_t)available);
-    out[0] = p.splits, out[1] = p.pages_per_split, out[2] = (long)p.total;
+    out[0] = p.splits, out[1] = p.pages_per_split, out[2] = (long)p.total, out[3] = p.two_per_sm;
 }
 int repair_wide(long cells, int threads) { return wc::repair_wide(cells, threads); }
 int write_two_tasks(int scheme, int bits, long n_tok, long heads) { return wc::write_two_tasks(scheme, bits, n_tok, heads); }
@@ -57,7 +57,7 @@ def test_pair_clusters_are_wide_while_resident(lib, n_tok, aligned, heads, resid
 
 
 def _plan(lib, batch, heads, max_pages, scheme=0, bits=8, group=1, append=0, available=-1):
-    out = (ctypes.c_long * 3)()
+    out = (ctypes.c_long * 4)()
     lib.plan(batch, heads, max_pages, scheme, bits, group, append, ctypes.c_long(available), out)
     return list(out)
 
@@ -80,7 +80,34 @@ def test_workspace_does_not_depend_on_the_variant(lib):
                 for pages in (1, 5, 30, 31, 40, 41, 500):
                     plans = [_plan(lib, batch, heads, pages, scheme, bits, g, a) for g in (1, 3, 4, 5, 8) for a in (0, 1)]
                     assert len({p[2] for p in plans}) == 1
-                    for splits, pps, total in plans:
+                    for splits, pps, total, _ in plans:
                         partials = splits + batch * heads if pps == 0 else splits * batch * heads
                         assert 256 + partials * 8 * 140 * 4 <= total
                         assert pps == 0 or splits * pps >= pages
+
+
+@pytest.mark.parametrize("batch,heads,max_pages,two", [
+    (37, 8, 5, 0), (38, 8, 5, 1), (38, 8, 24, 1), (38, 8, 25, 0), (76, 8, 48, 1), (76, 8, 49, 0), (300, 4, 94, 1), (300, 4, 95, 0),
+    (400, 4, 38, 1), (1000, 1, 16, 1), (1000, 8, 4, 1), (16, 4, 20, 0), (32, 8, 5, 0), (1, 304, 24, 1)])
+def test_ten_bit_short_sequences_take_two_ctas_per_sm(lib, batch, heads, max_pages, two):
+    """400 sequences of 2 pages over 4 KV heads: 70 us on warp pairs with one CTA per SM, 47 with two."""
+    splits, pps, total, got = _plan(lib, batch, heads, max_pages, 0, 10)
+    assert got == two
+    assert not two or pps > 0
+    for scheme, bits in ((0, 8), (1, 8), (2, 8)):
+        assert _plan(lib, batch, heads, max_pages, scheme, bits)[3] == 0
+
+
+def test_ten_bit_plans_fit_what_they_are_given(lib):
+    """A workspace of the size the 10-bit dither was first given holds whatever plan it then gets."""
+    for batch in (2, 16, 76, 100, 200, 400, 1000):
+        for heads in (1, 2, 4, 8):
+            for pages in (1, 5, 20, 41, 60, 100, 400, 2048):
+                want = _plan(lib, batch, heads, pages, 0, 10)
+                small = _plan(lib, batch, heads, pages, 0, 10, available=0)
+                assert small[2] <= want[2]
+                again = _plan(lib, batch, heads, pages, 0, 10, available=small[2])
+                assert again == small
+                for splits, pps, total, two in (want, small):
+                    partials = splits + batch * heads if pps == 0 else splits * batch * heads
+                    assert 256 + partials * 8 * 140 * 4 <= total
