@@ -360,6 +360,18 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) decode_kernel(const __gr
                 y[i] = kInt8 ? dc[i] * (sk[i >> 1] * kRsdLog2e) : dc[i] * kRsdLog2e;
                 cl[i] = cb[i] * kLog2e;
             }
+            // The value witness of tokens g, g+8 (0 past the context): fp8 loads it ahead of the
+            // vote, the dithered cache, which has no registers to spare, behind it.
+            float rho[2] = {0.f, 0.f}, vn[2] = {0.f, 0.f};
+            auto load_vw = [&] {
+                const float2 w0 = __half22float2(*reinterpret_cast<const __half2*>(st + kOffVw + 4 * g));
+                const float2 w1 = __half22float2(*reinterpret_cast<const __half2*>(st + kOffVw + 4 * (g + 8)));
+                rho[0] = w0.x;
+                rho[1] = w1.x;
+                vn[0] = w0.y;
+                vn[1] = w1.y;
+            };
+            if constexpr (kValue && !kInt8) load_vw();
             // One warp vote finds everything that an ordinary page does not need: the
             // context's last page, a logit more than 8 above the reference, a V scale above the
             // P scale's limit, a bound of kHugeLog2 or more (meter_term).  Masks, six shuffles of
@@ -381,8 +393,8 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) decode_kernel(const __gr
                         y[i] = -INFINITY;
                         cl[i] = 0.f;
                     }
-                if (!ok0) sv[0] = sk[0] = 0.f;
-                if (!ok1) sv[1] = sk[1] = 0.f;
+                if (!ok0) sv[0] = sk[0] = rho[0] = vn[0] = 0.f;
+                if (!ok1) sv[1] = sk[1] = rho[1] = vn[1] = 0.f;
                 huge = __any_sync(0xffffffffu, largest() >= kHugeLog2);
                 float mx0 = fmaxf(y[0], y[2]), mx1 = fmaxf(y[1], y[3]);
 #pragma unroll
@@ -424,13 +436,12 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) decode_kernel(const __gr
                     }
                 }
             }
-            float rho[2] = {0.f, 0.f};   // value witness of tokens g, g+8 (0 past the context)
-            if constexpr (kValue) {
-                const float2 w0 = __half22float2(*reinterpret_cast<const __half2*>(st + kOffVw + 4 * g));
-                const float2 w1 = __half22float2(*reinterpret_cast<const __half2*>(st + kOffVw + 4 * (g + 8)));
-                if (g < nvalid) { rho[0] = w0.x; vmax = fmaxf(vmax, w0.y); }
-                if (g + 8 < nvalid) { rho[1] = w1.x; vmax = fmaxf(vmax, w1.y); }
+            if constexpr (kValue && kInt8) {
+                load_vw();
+                if (g >= nvalid) rho[0] = vn[0] = 0.f;
+                if (g + 8 >= nvalid) rho[1] = vn[1] = 0.f;
             }
+            if constexpr (kValue) vmax = fmaxf(vmax, fmaxf(vn[0], vn[1]));
             float dpg[2] = {0.f, 0.f};   // this page's share of D (kRepair)
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
