@@ -185,14 +185,14 @@ struct FlatShares {
 };
 
 __device__ __forceinline__ int clamped_ctx(const DecodeParams& p, int b) {
-    return max(0, min(__ldg(p.ctx_lens + b), p.max_pages * kPage));
+    return max(0, min(load_dep(p.ctx_lens + b), p.max_pages * kPage));
 }
 
 // The split plan's segment of this CTA.
 __device__ __forceinline__ void split_segment(const DecodeParams& p, WsSeg& sg) {
     sg.b = blockIdx.z;
     sg.h = blockIdx.y;
-    int ctx = __ldg(p.ctx_lens + sg.b);
+    int ctx = load_dep(p.ctx_lens + sg.b);
     if (ctx < 0 || ctx > p.max_pages * kPage) {
         if (threadIdx.x == 0 && blockIdx.x == 0 && sg.h == 0) atomicOr(p.status, WC_DEV_BAD_CTX);
         ctx = max(0, min(ctx, p.max_pages * kPage));
@@ -216,7 +216,7 @@ struct FlatScratch {
 };
 __device__ __forceinline__ bool flat_first_segment(const DecodeParams& p, WsSeg& sg, FlatScratch& s, int cx, bool& bad) {
     const int nt = blockDim.x, t = threadIdx.x, per = (p.batch + nt - 1) / nt, cap = p.max_pages * kPage;
-    auto length = [&](int i) { return per == 1 ? cx : __ldg(p.ctx_lens + t * per + i); };
+    auto length = [&](int i) { return per == 1 ? cx : load_dep(p.ctx_lens + t * per + i); };
     uint32_t loc = 0;
     bad = false;
     for (int i = 0; i < per; ++i)
@@ -311,7 +311,7 @@ __device__ __forceinline__ bool flat_plan(const DecodeParams& p, WsSeg& sg, Flat
         if (have) warm(sg);
         grid_dep_wait();
         waited = true;
-        const int now = mine ? __ldg(p.ctx_lens + threadIdx.x) : 0;
+        const int now = mine ? load_dep(p.ctx_lens + threadIdx.x) : 0;
         const bool changed = now != cx;
         cx = now;
         if (!__syncthreads_or(changed)) break;

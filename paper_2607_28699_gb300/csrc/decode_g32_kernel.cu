@@ -106,7 +106,7 @@ __global__ void __launch_bounds__(kGwThreads, 1) decode_g32_ws_kernel(const __gr
     int phys_first = -1;
     if constexpr (!kFlat) {
         if (producer && p.max_pages > 0)
-            phys_first = __ldg(p.block_table + (size_t)blockIdx.z * p.max_pages +
+            phys_first = load_dep(p.block_table + (size_t)blockIdx.z * p.max_pages +
                                min((int)blockIdx.x * p.pages_per_split + pw, p.max_pages - 1));
     }
     WsSeg sg;
@@ -148,7 +148,7 @@ __global__ void __launch_bounds__(kGwThreads, 1) decode_g32_ws_kernel(const __gr
             const int32_t* bt_row = p.block_table + (size_t)b * p.max_pages;
             int first;
             const int n_seg = ws_seg_pages<kGwPairs>(cs, pw, first);
-            int phys_next = kFlat ? (n_seg > 0 ? __ldg(bt_row + first) : -1) : phys_first;
+            int phys_next = kFlat ? (n_seg > 0 ? load_dep(bt_row + first) : -1) : phys_first;
             for (int i = 0; i < n_seg; ++i, ++k) {
                 const int lp = first + kGwPairs * i;
                 const int s = k % kGwStages;
@@ -161,7 +161,7 @@ __global__ void __launch_bounds__(kGwThreads, 1) decode_g32_ws_kernel(const __gr
                     }
                 }
                 const int phys = phys_next;
-                if (i + 1 < n_seg) phys_next = __ldg(bt_row + lp + kGwPairs);
+                if (i + 1 < n_seg) phys_next = load_dep(bt_row + lp + kGwPairs);
                 const bool ok = phys >= 0 && phys < p.num_pages;
                 uint8_t* st = stages + s * kGwStageBytes;
                 if (elect_one()) {   // not a lane test: the copies' operands stay on the uniform path
@@ -228,12 +228,12 @@ __global__ void __launch_bounds__(kGwThreads, 1) decode_g32_ws_kernel(const __gr
         uint32_t qw[16];   // head g, channels 16ks + 4c + 2hh, +1 in word 2ks + hh (storage order)
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-            const uint4 v = row_valid ? __ldg(reinterpret_cast<const uint4*>(qrow + 32 * c) + i) : make_uint4(0, 0, 0, 0);
+            const uint4 v = row_valid ? load_dep(reinterpret_cast<const uint4*>(qrow + 32 * c) + i) : make_uint4(0, 0, 0, 0);
             qn[4 * i] = v.x; qn[4 * i + 1] = v.y; qn[4 * i + 2] = v.z; qn[4 * i + 3] = v.w;
         }
 #pragma unroll
         for (int ks = 0; ks < 8; ++ks) {
-            const uint2 v = row_valid ? __ldg(reinterpret_cast<const uint2*>(qrow + 16 * ks + 4 * c)) : make_uint2(0, 0);
+            const uint2 v = row_valid ? load_dep(reinterpret_cast<const uint2*>(qrow + 16 * ks + 4 * c)) : make_uint2(0, 0);
             qw[2 * ks] = v.x;
             qw[2 * ks + 1] = v.y;
         }
@@ -247,7 +247,7 @@ __global__ void __launch_bounds__(kGwThreads, 1) decode_g32_ws_kernel(const __gr
         uint32_t qb[4] = {0u, 0u, 0u, 0u};
         uint32_t seen_lo = 0u, seen_hi = 0u;   // pair indices met so far: a repeated pair is ignored
         for (int t = 0; t < m; ++t) {
-            const int j = __ldg(prs + t);
+            const int j = load_dep(prs + t);
             const bool again = j >= 0 && j < kHeadDim / 2 && (((j < 32 ? seen_lo : seen_hi) >> (j & 31)) & 1u);
             if (j < 0 || j >= kHeadDim / 2 || again) {
                 if (threadIdx.x == 0 && blockIdx.x == 0) atomicOr(p.status, WC_DEV_BAD_PAIR);
@@ -263,8 +263,8 @@ __global__ void __launch_bounds__(kGwThreads, 1) decode_g32_ws_kernel(const __gr
             if (((da >> 2) & 3) == c) pmask |= 1u << (4 * (da >> 4) + (da & 3));
             if (((db >> 2) & 3) == c) pmask |= 1u << (4 * (db >> 4) + (db & 3));
             if ((t & 3) == c && row_valid) {   // pair t = 4 (t >> 2) + c: entries 2t, 2t + 1 of tile t >> 2
-                const unsigned short qa = __ldg(reinterpret_cast<const unsigned short*>(qrow) + da);
-                const unsigned short qbv = __ldg(reinterpret_cast<const unsigned short*>(qrow) + db);
+                const unsigned short qa = load_dep(reinterpret_cast<const unsigned short*>(qrow) + da);
+                const unsigned short qbv = load_dep(reinterpret_cast<const unsigned short*>(qrow) + db);
                 const uint32_t w = (uint32_t)qa | ((uint32_t)qbv << 16);
                 const int tile = t >> 2;
                 qb[0] = tile == 0 ? w : qb[0];

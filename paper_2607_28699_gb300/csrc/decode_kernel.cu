@@ -100,7 +100,7 @@ __device__ __forceinline__ void load_q_frag(const DecodeParams& p, int b, int h,
         p.q + ((size_t)b * p.num_q_heads + (size_t)h * G + (row_valid ? g : 0)) * kHeadDim + 32 * c);
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-        const uint4 v = row_valid ? __ldg(qsrc + i) : make_uint4(0, 0, 0, 0);
+        const uint4 v = row_valid ? load_dep(qsrc + i) : make_uint4(0, 0, 0, 0);
         qw[4 * i] = v.x; qw[4 * i + 1] = v.y; qw[4 * i + 2] = v.z; qw[4 * i + 3] = v.w;
     }
 }
@@ -141,9 +141,9 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) decode_kernel(const __gr
 #pragma unroll
     for (int k = 0; k < kStages; ++k) {
         const int lp = p0 + warp + kWarps * k;
-        ring[k] = lp < lim ? __ldg(bt_row + lp) : -1;
+        ring[k] = lp < lim ? load_dep(bt_row + lp) : -1;
     }
-    int ctx = __ldg(p.ctx_lens + b);
+    int ctx = load_dep(p.ctx_lens + b);
     load_q_frag(p, b, h, G, g, c, qw);
     // Tier B and the value side of the dithered cache read the query fragment (the same in every
     // warp) from shared memory page by page: with its 16 registers held through the PV products
@@ -270,7 +270,7 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) decode_kernel(const __gr
     for (int k = 0; k < n_my; ++k) {
         const int lp = p0 + warp + kWarps * k;   // this page
         // the page-table entry of the page issued at the end of the iteration
-        const int phys_issue = (k + kStages < n_my) ? __ldg(bt_row + lp + kWarps * kStages) : -1;
+        const int phys_issue = (k + kStages < n_my) ? load_dep(bt_row + lp + kWarps * kStages) : -1;
         const int phys = ring[0];
         const bool page_ok = phys >= 0 && phys < p.num_pages;
         const bool landed = mbar_wait_bounded(&bars[k % kStages], (uint32_t)((k / kStages) & 1));
@@ -756,7 +756,7 @@ struct WsParams {
 // generic-proxy stores are fenced against the async-proxy copies that follow.
 __device__ __forceinline__ void append_new_token(const WsParams& wp, int b, int h, int phys, int ctx, int lane) {
     const DecodeParams& p = wp.p;
-    const int slot = __ldg(p.slot_new + b);
+    const int slot = load_dep(p.slot_new + b);
     if (slot < 0) return;   // warp-uniform: no new token for this sequence
     if (slot != phys * kPage + (ctx - 1) % kPage) {
         if (lane == 0) atomicOr(p.status, WC_DEV_BAD_APPEND);
@@ -767,10 +767,10 @@ __device__ __forceinline__ void append_new_token(const WsParams& wp, int b, int 
     const size_t off = ((size_t)b * p.num_kv_heads + h) * kHeadDim + sub * 16;
     uint4 rk[2] = {make_uint4(0, 0, 0, 0), make_uint4(0, 0, 0, 0)}, rv[2] = {rk[0], rk[1]};
     if (live) {
-        rk[0] = __ldg(reinterpret_cast<const uint4*>(p.k_new + off));
-        rk[1] = __ldg(reinterpret_cast<const uint4*>(p.k_new + off) + 1);
-        rv[0] = __ldg(reinterpret_cast<const uint4*>(p.v_new + off));
-        rv[1] = __ldg(reinterpret_cast<const uint4*>(p.v_new + off) + 1);
+        rk[0] = load_dep(reinterpret_cast<const uint4*>(p.k_new + off));
+        rk[1] = load_dep(reinterpret_cast<const uint4*>(p.k_new + off) + 1);
+        rv[0] = load_dep(reinterpret_cast<const uint4*>(p.v_new + off));
+        rv[1] = load_dep(reinterpret_cast<const uint4*>(p.v_new + off) + 1);
     }
     write_row<WC_SCHEME_DITHER_INT8, 8>(wp.w, rk, slot, live, h, 0, sub, nullptr, nullptr);
     write_row<WC_SCHEME_DITHER_INT8, 8>(wp.w, rv, slot, live, h, 1, sub, nullptr, nullptr);
@@ -849,7 +849,7 @@ __global__ void __launch_bounds__(kWsThreads, 1) decode_ws_kernel(const __grid_c
     uint32_t qw[16];
     if constexpr (!kFlat) {
         if (producer && p.max_pages > 0)
-            phys_first = __ldg(p.block_table + (size_t)blockIdx.z * p.max_pages +
+            phys_first = load_dep(p.block_table + (size_t)blockIdx.z * p.max_pages +
                                min((int)blockIdx.x * p.pages_per_split + pw, p.max_pages - 1));
         if (!producer) load_q_frag(p, blockIdx.z, blockIdx.y, G, g, c, qw);
     }
@@ -899,7 +899,7 @@ __global__ void __launch_bounds__(kWsThreads, 1) decode_ws_kernel(const __grid_c
             const int32_t* bt_row = p.block_table + (size_t)b * p.max_pages;
             int first;
             const int n_seg = ws_seg_pages<kWsPairs>(cs, pw, first);
-            int phys_next = kFlat ? (n_seg > 0 ? __ldg(bt_row + first) : -1) : phys_first;
+            int phys_next = kFlat ? (n_seg > 0 ? load_dep(bt_row + first) : -1) : phys_first;
             if constexpr (kAppend) {
                 // The stream that stages the sequence's last page in this segment stores
                 // the new token before the segment's first page (not inside the page
@@ -907,7 +907,7 @@ __global__ void __launch_bounds__(kWsThreads, 1) decode_ws_kernel(const __grid_c
                 // carries no write code.  Its copies are issued after the token's stores.
                 const int lpl = npages - 1;
                 if (n_seg > 0 && lpl >= first && (lpl - first) % kWsPairs == 0 && lpl < cs.e) {
-                    const int phl = __ldg(bt_row + lpl);
+                    const int phl = load_dep(bt_row + lpl);
                     if (phl >= 0 && phl < p.num_pages) append_new_token(wp, b, h, phl, ctx, lane);
                 }
             }
@@ -923,7 +923,7 @@ __global__ void __launch_bounds__(kWsThreads, 1) decode_ws_kernel(const __grid_c
                     }
                 }
                 const int phys = phys_next;
-                if (i + 1 < n_seg) phys_next = __ldg(bt_row + lp + kWsPairs);
+                if (i + 1 < n_seg) phys_next = load_dep(bt_row + lp + kWsPairs);
                 const bool ok = phys >= 0 && phys < p.num_pages;
                 uint8_t* st = stages + s * St::kBytes;
                 if constexpr (kStall) {   // failure-detection test: this page is never staged
@@ -1643,7 +1643,7 @@ __global__ void __launch_bounds__(32 * kMergeWarps, kW == 1 ? 4 : 3) merge_warp_
     if constexpr (kHint) {
         find_hinted();
         grid_dep_wait();
-        now = lane < p.batch ? __ldg(p.ctx_lens + lane) : 0;
+        now = lane < p.batch ? load_dep(p.ctx_lens + lane) : 0;
     } else {
         grid_dep_wait();
         if (p.pages_per_split > 0) {
@@ -1663,7 +1663,7 @@ __global__ void __launch_bounds__(32 * kMergeWarps, kW == 1 ? 4 : 3) merge_warp_
             const int b0 = (int)((long long)blockIdx.x * (kMergeWarps / kW) / ((kHeadDim / 32) * p.num_q_heads));
             uint32_t before = 0, total = 0;
             for (int i = threadIdx.x; i < p.batch; i += 32 * kMergeWarps) {
-                const uint32_t span = span_of(__ldg(p.ctx_lens + i));
+                const uint32_t span = span_of(load_dep(p.ctx_lens + i));
                 total += span;
                 if (i < b0) before += span;
             }
@@ -1678,7 +1678,7 @@ __global__ void __launch_bounds__(32 * kMergeWarps, kW == 1 ? 4 : 3) merge_warp_
             if (live) {
                 before = __reduce_add_sync(0xffffffffu, lane < kMergeWarps ? sums[0][lane] : 0u);
                 total = __reduce_add_sync(0xffffffffu, lane < kMergeWarps ? sums[1][lane] : 0u);
-                for (int i = b0; i < b; ++i) before += span_of(__ldg(p.ctx_lens + i));
+                for (int i = b0; i < b; ++i) before += span_of(load_dep(p.ctx_lens + i));
                 find_flat(before, total, (uint32_t)(clamped_ctx(p, b) + kPage - 1) / kPage);
             }
         }

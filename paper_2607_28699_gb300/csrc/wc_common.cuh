@@ -284,6 +284,12 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity
 // has completed and its memory is visible (a no-op for ordinary launches).
 __device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+// An input that the preceding kernel may have written, read after grid_dep_wait(): an ordinary
+// load, which the wait's memory clobber holds back.  The read-only path (ld.global.nc) is for data
+// that no one writes while the kernel runs, and a kernel launched early runs beside its
+// predecessor.  (Before the wait, hints are read past L1 by __ldcg.)
+template <typename T>
+__device__ __forceinline__ T load_dep(const T* p) { return *p; }
 
 __device__ __forceinline__ float fast_exp2(float x) {
     float y;

@@ -148,7 +148,7 @@ __device__ __forceinline__ void write_row(const WriteParams& p, uint4 (&raw)[2],
         } else if (row == 0) {
             const int32_t* pr = p.bypass_pairs + (size_t)h * p.num_bypass;
             for (int t = 0; t < p.num_bypass; ++t) {
-                const int j = __ldg(pr + t);
+                const int j = load_dep(pr + t);
                 if (j < 0 || j >= kHeadDim / 2) {
                     if (live_unit && sub == 0 && p.dev_status) atomicOr(p.dev_status, WC_DEV_BAD_PAIR);
                     continue;
@@ -399,7 +399,7 @@ __device__ __forceinline__ void write_row(const WriteParams& p, uint4 (&raw)[2],
                 __half* bdst = p.k_bypass + rowidx * (2 * p.num_bypass);
                 uint32_t seen = 0;   // this lane's channels stored already: a repeated pair stores zeros
                 for (int t = 0; t < p.num_bypass; ++t) {
-                    const int j = __ldg(pr + t);
+                    const int j = load_dep(pr + t);
                     if (j < 0 || j >= kHeadDim / 2) {   // an ignored pair stores zeros
                         if (sub == 0) bdst[2 * t] = bdst[2 * t + 1] = __float2half_rn(0.0f);
                         continue;
