@@ -152,10 +152,15 @@ def _ptr(t: Optional[torch.Tensor]):
     return t.data_ptr()
 
 
+# Not part of torch's public interface: a build without them takes the Stream object.
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+_raw_device = getattr(torch._C, "_cuda_getDevice", None)
+
+
 def _stream(stream):
     if stream is None:
-        if torch.cuda.is_initialized():
-            return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+        if _raw_stream is not None and _raw_device is not None and torch.cuda.is_initialized():
+            return _raw_stream(_raw_device())
         stream = torch.cuda.current_stream()
     return stream.cuda_stream
 
