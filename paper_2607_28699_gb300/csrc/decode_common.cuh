@@ -165,7 +165,7 @@ __device__ __forceinline__ void prefetch_map(const CUtensorMap* map) {
 // 43.9), 38 of 51 and 53 pages 20.0 (22.1 with shares from 0).
 // ph keeps the streams' round robin running across the cuts, so
 // every stream gets ceil or floor of the share's pages / n.
-constexpr uint32_t kCutPages = 12;  
+constexpr uint32_t kCutPages = 12;
 
 struct WsSeg {
     int b, h, a, e, ph, ctx, np;
@@ -274,10 +274,9 @@ __device__ __forceinline__ bool flat_first_segment(const DecodeParams& p, WsSeg&
 }
 
 // Next segment of the flattened plan (the next sequence with pages); false
-// at the end of the CTA's share, and always in the split plan.
-template <int kStreams, bool kFlat>
+// at the end of the CTA's share.
+template <int kStreams>
 __device__ __forceinline__ bool ws_next_segment(const DecodeParams& p, WsSeg& sg) {
-    if constexpr (!kFlat) return false;
     const int done = sg.ph + (sg.e - sg.a);
     do {   // sequences without pages hold no part of the share
         sg.vb += flat_span(sg.np);
@@ -337,18 +336,15 @@ __device__ __forceinline__ void warm_queries(const DecodeParams& p, int b, int h
 
 // Flattened plan: each warp's walker lives in a shared slot, so that only the
 // current segment's indices take registers in the page loop; lane 0 advances it.
-template <int kStreams, bool kFlat>
+template <int kStreams>
 __device__ __forceinline__ bool ws_step(const DecodeParams& p, WsSeg* slot, int lane) {
-    if constexpr (!kFlat) {
-        return false;
-    } else {
-        __syncwarp();
-        int more = 0;
-        if (lane == 0) more = ws_next_segment<kStreams, true>(p, *slot);
-        __syncwarp();
-        return __shfl_sync(0xffffffffu, more, 0) != 0;
-    }
+    __syncwarp();
+    int more = 0;
+    if (lane == 0) more = ws_next_segment<kStreams>(p, *slot);
+    __syncwarp();
+    return __shfl_sync(0xffffffffu, more, 0) != 0;
 }
+
 template <int kStreams>
 __device__ __forceinline__ int ws_seg_pages(const WsSeg& sg, int w, int& first) {
     first = sg.a + (int)((unsigned)(w - sg.ph + kStreams) % kStreams);

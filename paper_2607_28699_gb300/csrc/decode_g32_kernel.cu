@@ -201,7 +201,7 @@ __global__ void __launch_bounds__(kGwThreads, 1) decode_g32_ws_kernel(const __gr
             }
         };
         if constexpr (kFlat) {
-            for (bool more = have; more && !stop; more = ws_step<kGwPairs, true>(p, my_seg, lane)) produce(*my_seg);
+            for (bool more = have; more && !stop; more = ws_step<kGwPairs>(p, my_seg, lane)) produce(*my_seg);
         } else {
             produce(sg);
         }
@@ -663,7 +663,7 @@ __global__ void __launch_bounds__(kGwThreads, 1) decode_g32_ws_kernel(const __gr
         }
     };
     if constexpr (kFlat) {
-        for (bool more = have; more; more = ws_step<kGwPairs, true>(p, my_seg, lane)) consume(*my_seg);
+        for (bool more = have; more; more = ws_step<kGwPairs>(p, my_seg, lane)) consume(*my_seg);
     } else {
         if (have) consume(sg);
     }

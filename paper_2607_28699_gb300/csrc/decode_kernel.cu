@@ -32,9 +32,7 @@
 #include <cuda.h>
 #include <cudaTypedefs.h>
 
-#include <algorithm>
 #include <climits>
-#include <mutex>
 
 #include "decode_common.cuh"
 #include "write_row.cuh"
@@ -991,7 +989,7 @@ __global__ void __launch_bounds__(kWsThreads, 1) decode_ws_kernel(const __grid_c
             }
         };
         if constexpr (kFlat) {
-            for (bool more = have; more && !stop; more = ws_step<kWsPairs, true>(p, my_seg, lane)) produce(*my_seg);
+            for (bool more = have; more && !stop; more = ws_step<kWsPairs>(p, my_seg, lane)) produce(*my_seg);
         } else {
             produce(sg);
         }
@@ -1441,7 +1439,7 @@ __global__ void __launch_bounds__(kWsThreads, 1) decode_ws_kernel(const __grid_c
         }
     };
     if constexpr (kFlat) {
-        for (bool more = have; more; more = ws_step<kWsPairs, true>(p, my_seg, lane)) consume(*my_seg);
+        for (bool more = have; more; more = ws_step<kWsPairs>(p, my_seg, lane)) consume(*my_seg);
     } else {
         if (have) consume(sg);
     }

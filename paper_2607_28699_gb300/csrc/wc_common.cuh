@@ -52,28 +52,6 @@ __device__ __forceinline__ uint4 philox(uint32_t c0, uint32_t c1, uint32_t c2, u
     return make_uint4(c0, c1, c2, c3);
 }
 
-// N independent Philox4x32-10 calls advanced round by round: counters in
-// (x0, x1, x2, x3)[j], results in place.  The calls' multiplies issue back to
-// back, so their latencies overlap (one call's rounds are a dependent chain).
-template <int N>
-__device__ __forceinline__ void philox_n(uint32_t (&x0)[N], uint32_t (&x1)[N], uint32_t (&x2)[N], uint32_t (&x3)[N],
-                                         const PhiloxKeys& key) {
-#pragma unroll
-    for (int r = 0; r < kPhiloxRounds; ++r) {
-#pragma unroll
-        for (int j = 0; j < N; ++j) {
-            const uint64_t p0 = (uint64_t)kPhiloxM0 * x0[j];
-            const uint64_t p1 = (uint64_t)kPhiloxM1 * x2[j];
-            const uint32_t n0 = (uint32_t)(p1 >> 32) ^ x1[j] ^ key.k0[r];
-            const uint32_t n2 = (uint32_t)(p0 >> 32) ^ x3[j] ^ key.k1[r];
-            x1[j] = (uint32_t)p1;
-            x3[j] = (uint32_t)p0;
-            x0[j] = n0;
-            x2[j] = n2;
-        }
-    }
-}
-
 // Philox4x32-10 at (c0, c1, c2, 0) and (c0, c1, c2, 1) (a K row and the V row of the same
 // token), round by round: 36 wide multiplies instead of 40.
 __device__ __forceinline__ void philox_rows(uint32_t c0, uint32_t c1, uint32_t c2, const PhiloxKeys& key, uint4& w0,
@@ -119,7 +97,7 @@ __device__ __forceinline__ PhiloxGroup philox_group(uint32_t g, uint32_t c1, con
 // Philox4x32-10 at (slot, c1, g, tag) for four groups g and tags 0 (w[0]: a K row),
 // 1 (w[1]: the V row of the same token).  The eight calls advance round by round,
 // so their multiplies overlap, and a product that two calls share is taken once:
-// 127 wide multiplies instead of 160 (134 with the group constants redrawn).
+// 127 wide multiplies instead of 160 (135 with the group constants redrawn).
 __device__ __forceinline__ void philox_kv(uint32_t slot, const PhiloxGroup (&gr)[4], const PhiloxKeys& key,
                                           uint32_t (&w)[2][4][4]) {
     const uint64_t ps = (uint64_t)kPhiloxM0 * slot;
