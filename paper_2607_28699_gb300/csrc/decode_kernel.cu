@@ -55,8 +55,14 @@ constexpr int kOffVw = 320;              // value witness [16][2] fp16 (value si
 constexpr int kSmallStride = 384;
 constexpr int kOffQ = 2 * kTileRegion + kWarps * kStages * kSmallStride + kWarps * kStages * 8;   // query fragment (kQShared)
 constexpr int kQBytes = 16 * 32 * 4;
-constexpr int kSmemBytes = kOffQ + kQBytes + 1024;
-static_assert(kOffQ % 16 == 0 && 2 * (kSmemBytes + 1024) <= 228 * 1024, "two CTAs per SM");
+// Only the variants that use the query fragment's 2 KiB have them (fp8, value side, 300 pages
+// x 4 heads: 7.60 us a decode without them, 7.95 with them).
+template <bool kInt8, int kX>
+struct TwoPerSm {
+    static constexpr bool kQShared = kInt8 && (kX & (kXTierB | kXValue)) != 0;
+    static constexpr int kSmemBytes = kOffQ + (kQShared ? kQBytes : 0) + 1024;
+    static_assert(kOffQ % 16 == 0 && 2 * (kSmemBytes + 1024) <= 228 * 1024, "two CTAs per SM");
+};
 
 // decode_kernel's parameters: the code tiles' tensor maps and the call.
 struct DkParams {
@@ -146,7 +152,7 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) decode_kernel(const __gr
     // Tier B and the value side of the dithered cache read the query fragment (the same in every
     // warp) from shared memory page by page: with its 16 registers held through the PV products
     // they spill (3% of a call; the plain and the repair variant do not gain).
-    constexpr bool kQShared = kInt8 && (kTierB || kValue);
+    constexpr bool kQShared = TwoPerSm<kInt8, kX>::kQShared;
     uint4* q_s = reinterpret_cast<uint4*>(smem + kOffQ) + lane;
     if constexpr (kQShared) {
         if (warp == 0) {
@@ -808,7 +814,7 @@ __global__ void __launch_bounds__(kWsThreads, 1) decode_ws_kernel(const __grid_c
     uint8_t* stages = smem + pw * kWsStages * St::kBytes;
     uint64_t* full = reinterpret_cast<uint64_t*>(smem + Sm::kStages) + pw * 2 * kWsStages;
     uint64_t* empty = full + kWsStages;
-    if (kBits == 10 && threadIdx.x == 32 * kWsPairs) {   // 10-bit: 1.6% off a step and no spills; 8-bit: nothing
+    if (kBits == 10 && threadIdx.x == 32 * kWsPairs) {   // 10-bit: 1.6% off a step; 8-bit: nothing
         prefetch_map(&wp.k_map);
         prefetch_map(&wp.v_map);
     }
@@ -1841,14 +1847,15 @@ cudaError_t launch_merge_x(const DecodeParams& p, int x, cudaStream_t stream) {
 template <bool kInt8, int kX>
 static cudaError_t launch_two_per_sm(const DecodeParams& p, cudaStream_t stream) {
     static PerDevice<Configured, cudaError_t> configured;
-    if (cudaError_t e = configure(configured, decode_kernel<kInt8, kX>, kSmemBytes)) return e;
+    constexpr int kSmem = TwoPerSm<kInt8, kX>::kSmemBytes;
+    if (cudaError_t e = configure(configured, decode_kernel<kInt8, kX>, kSmem)) return e;
     DkParams dp;
     dp.p = p;
     if (!encode_page_map(&dp.k_map, p.k_codes, p.num_pages, p.num_kv_heads) ||
         !encode_page_map(&dp.v_map, p.v_codes, p.num_pages, p.num_kv_heads))
         return cudaErrorInvalidValue;
     const dim3 grid(p.splits, p.num_kv_heads, p.batch);
-    cudaError_t e = launch_pdl(decode_kernel<kInt8, kX>, grid, dim3(kThreads), kSmemBytes, stream, dp);
+    cudaError_t e = launch_pdl(decode_kernel<kInt8, kX>, grid, dim3(kThreads), kSmem, stream, dp);
     if (e != cudaSuccess) return e;
     // the merge is a programmatic dependent too: its CTAs are scheduled while
     // the decode grid drains and wait (griddepcontrol.wait) for all of it
