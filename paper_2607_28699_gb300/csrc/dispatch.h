@@ -33,7 +33,7 @@ constexpr bool write_two_tasks(int scheme, int bits, int64_t n_tok, int64_t num_
 // The wide cluster's copies are 16 bytes; it is launched while every head's cluster is resident
 // at once (resident: the device's answer for that launch, 14 on GB300; 0 where 16 CTAs cannot be
 // placed).  Heads, us narrow / wide: 4 heads, 1024 rows 3.8 / 4.6, 2048 4.5 / 4.6, 4096 4.8 / 4.4,
-// 8192 6.3 / 5.3, 32768 15.2 / 9.3; 4096 rows, 8 heads 5.5 / 5.3, 16 6.6 / 8.6, 32 6.9 / 12.7;
+// 8192 6.3 / 5.3, 32768 14.9 / 8.7; 4096 rows, 8 heads 5.5 / 5.3, 16 6.6 / 8.6, 32 6.9 / 12.7;
 // 65536 rows, 8 heads 46.0 / 26.6, 16 55.3 / 52.3, 32 79.9 / 93.5.
 constexpr int kWidePairRows = 4096;
 constexpr bool pairs_wide(int n_tok, bool aligned16, int num_kv_heads, int resident) {

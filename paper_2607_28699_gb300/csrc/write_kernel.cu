@@ -34,8 +34,8 @@ namespace {
 // then specialised for each, and their Philox calls share the products that do not see
 // the tag.  A write of a few tokens takes one task per warp (K rows in warps 0 and 2, V
 // rows in 1 and 3): there one row's latency is what counts.  Measured at 32768 x 4 tokens
-// and heads against K and V rows in separate warps (us): 8-bit dither 31.1 -> 26.4, 10-bit
-// 39.7 -> 36.3, fp8 18.1 -> 15.7, grouped 50.1 -> 44.9 (55.4 before its packed pass).
+// and heads against K and V rows in separate warps (us): 8-bit dither 30.4 -> 26.5, 10-bit
+// 39.7 -> 35.6, fp8 17.6 -> 15.1, grouped with its packed pass 53.4 -> 44.3.
 constexpr int write_units_per_cta(int tasks) { return 2 * 4 * tasks; }
 
 // Two ways of cutting the units (token, KV head) into 4-unit tasks:
@@ -46,9 +46,9 @@ constexpr int write_units_per_cta(int tasks) { return 2 * 4 * tasks; }
 //            units, K or V, so a one-token write of up to 8 KV heads is a single CTA
 //            (decode steps, where every SM the next decode needs counts).
 // Resident CTAs per SM the register budget is sized for, the best of 5 .. 9 in each case
-// (us at 32768 x 4): 8-bit dither seven at 72 registers 26.9 (six 28.5, eight 28.2, with
-// 36 bytes of spill), 10-bit six 35.7 (seven 36.5), grouped six 44.3 with 56 bytes of spill
-// (seven 44.1 with 84, which costs the 2047 x 8 write 10%), fp8 eight 15.3 (ten 15.7).  One
+// (at 32768 x 4): 8-bit dither seven at 72 registers (six 6% slower, eight, with 36 bytes of
+// spill, 5%), 10-bit six (seven 2% slower), grouped six with 56 bytes of spill (seven, with 84,
+// 0.5% faster, but the 2047 x 8 write 10% slower), fp8 eight (ten 3% slower).  One
 // task per warp: seven, so that the small writes that take it are one wave (1000 x 8: grouped
 // 5.6, six 6.3).
 __host__ __device__ constexpr int write_min_blocks(int scheme, int bits, int tasks) {
@@ -167,7 +167,7 @@ __global__ void __launch_bounds__(128, write_min_blocks(kScheme, kBits, kTasks))
 // Both clusters add the same numbers in the same order.  Bytes in flight bound the narrow
 // one (4 loads a warp: 32 KB an SM, 1.8 TB/s over 32 SMs); the wide one keeps 64 KB an SM in
 // a ring of asynchronous copies on twice the SMs, as deeper batches of loads into registers
-// were split up again by the compiler (8.7).  16384 rows x 4 heads: 9.6 -> 6.7 us.
+// were split up again by the compiler (8.7).  16384 rows x 4 heads: 9.3 -> 6.0 us.
 constexpr int kSelPairRing = 16;   // wide: copies in flight per lane
 
 __device__ __forceinline__ void copy16_or_zero(uint4* dst, const __half* src, bool valid) {
