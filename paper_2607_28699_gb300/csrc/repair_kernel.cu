@@ -21,8 +21,8 @@
 // stable passes over 7-bit digits instead.  Both give the same order, so the sums that
 // follow are the same bits.
 // Measured, network of compare-exchanges (the only sort before) -> this: 784 cells of 2048
-// pages 58.6 -> 21.3 us, half of their contributions zero 58.7 -> 17.7, all equal 59.3 -> 19.5;
-// 2800 of 512 43.5 -> 18.5; 8400 of 100 119 -> 13.6; 196 of 8192 99 -> 36.  Twice or four times
+// pages 58.7 -> 21.0 us, half of their contributions zero 58.6 -> 17.5, all equal 59.2 -> 19.4;
+// 2800 of 512 43.6 -> 18.4; 8400 of 100 119 -> 13.1; 196 of 8192 99 -> 31.  Twice or four times
 // the buckets at 784 x 2048: no faster.
 #include <climits>
 
@@ -45,9 +45,9 @@ __device__ __forceinline__ float key_value(unsigned long long key) { return __ui
 
 // A CTA of T threads sorts K keys per thread; KS: positions per thread of the sums.
 // T grows with the table (K = 4 up to 4096 pages), so that a small cell costs few warps
-// and barriers: 2800 cells of 512 pages took 24.8 us with 512 threads, 16.2 with 256.
+// and barriers (repair_wide has both sides).
 // Threads per SM that the register budget leaves room for: all 2048 with one or two keys a
-// thread, 1536 with four (at most 40 registers: 2800 cells of 512 pages 18.5 us, without it 23.9),
+// thread, 1536 with four (at most 40 registers: 2800 cells of 512 pages 18.4 us, without it 23.9),
 // 1024 with more.
 constexpr int min_ctas(int T, int K) {
     const int n = (K <= 2 ? 2048 : K <= 4 ? 1536 : 1024) / T;
